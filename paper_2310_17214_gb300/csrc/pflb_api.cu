@@ -430,13 +430,14 @@ int pflb_create_domain(const pflb_domain_desc* desc, pflb_domain** out) {
     return fail(nullptr, PFLB_ERR_CUDA, "%s", cudaGetErrorString(e));
   }
   const size_t n = (size_t)N;
-  // partial sums: one slot per block of the 1-D init grid or of any tile grid
-  // (the step's 32 x 8 tiles and the batch's tile shapes)
-  long long tiles = 0;
+  // partial sums: one slot per block of the 1-D init grid or of any tile grid:
+  // tiles of 32 x 2 cells and more in 2-D, 32 x 8 columns of at least one plane
+  // in 3-D, the batch's tile shapes
+  long long tiles = (long long)((D.nx + 31) / 32) *
+                    (D.dim == 3 ? (long long)((D.ny + 7) / 8) * D.nz : (D.ny + 1) / 2);
   for (int cfg = 0; cfg < BATCH_SHAPES; ++cfg)
     tiles = std::max<long long>(tiles, (long long)((D.nx + batch_tx(cfg) - 1) / batch_tx(cfg)) *
-                                           ((D.ny + batch_ty(cfg) - 1) / batch_ty(cfg)) *
-                                           (D.dim == 3 ? (D.nz + 15) / 16 : 1));
+                                           ((D.ny + batch_ty(cfg) - 1) / batch_ty(cfg)));
   const long long blocks = std::max<long long>((N + BLOCK - 1) / BLOCK, tiles);
   bool ok = true;
   auto al = [&](void** p, size_t bytes) {

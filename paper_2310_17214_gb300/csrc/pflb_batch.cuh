@@ -15,44 +15,31 @@
 // every domain's P0 is current for the next launch.
 #pragma once
 
+#include "pflb_half.cuh"
 #include "pflb_kernels.cuh"
 
 namespace pflb {
 
-template <int K, class Real, class Store>
-struct BatchDom {
-  Params<Real, K> P;
-  State<Real, Store> S[2];  // S[q]: input state in ping-pong buffer q
-  int p0_closed;
-  int cur0;                 // buffer holding the input at even batch steps
-};
-
-// Tile shapes the batch can run: 32 x 8, 32 x 16 (two rows per thread),
-// 64 x 4.
+// Tile shapes the batch can run.
 constexpr int BATCH_SHAPES = 3;
-template <int CFG> struct BatchShape;
-template <> struct BatchShape<0> { using T = Tile<2, 32, 1>; };
-template <> struct BatchShape<1> { using T = Tile<2, 32, 2>; };
-template <> struct BatchShape<2> { using T = Tile<2, 64, 1>; };
+template <class Real, int CFG> struct BatchShape;
+template <class Real> struct BatchShape<Real, 0> { using T = Tile<typename VecOf<Real>::V, 32, 8>; };
+template <class Real> struct BatchShape<Real, 1> { using T = Tile<typename VecOf<Real>::V, 32, 16>; };
+template <class Real> struct BatchShape<Real, 2> { using T = Tile<typename VecOf<Real>::V, 64, 4>; };
 
 __host__ __device__ constexpr int batch_tx(int cfg) { return cfg == 2 ? 64 : 32; }
 __host__ __device__ constexpr int batch_ty(int cfg) { return cfg == 0 ? 8 : (cfg == 1 ? 16 : 4); }
 
-template <class Real, class Store, class T_> struct BatchMinBlocks {
-  static constexpr int value = sizeof(Real) == 8 ? 2 : (T_::RPT > 1 ? 3 : 4);
-};
-
-template <int K, class Real, class Store, class T_>
-__global__ void __launch_bounds__(BLOCK, (BatchMinBlocks<Real, Store, T_>::value))
-batch_step_kernel(const BatchDom<K, Real, Store>* __restrict__ doms,
+template <int K, class Real, class T_>
+__global__ void __launch_bounds__(T_::NT, (MinBlocks<K, T_>::value))
+batch_step_kernel(const BatchDom<K, Real, Real>* __restrict__ doms,
                   const int* __restrict__ tile_begin, int ndom, int flip,
                   unsigned* __restrict__ tile_ctr) {
-  using PL = Plane<Real, K, T_::HP, n_mom<2, Store>()>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PL* planes = reinterpret_cast<PL*>(smem_raw);
+  Real* pl = reinterpret_cast<Real*>(smem_raw);
   __shared__ double red_sh[96];
   __shared__ Params<Real, K> Psh;
-  __shared__ State<Real, Store> Ssh;
+  __shared__ State<Real, Real> Ssh;
   __shared__ int p0c_sh;
   __shared__ int next_sh[2];
 
@@ -74,7 +61,7 @@ batch_step_kernel(const BatchDom<K, Real, Store>* __restrict__ doms,
     }
     if (lo != cur_dom) {
       __syncthreads();  // the previous tile is done with the shared copies
-      const BatchDom<K, Real, Store>& D = doms[lo];
+      const BatchDom<K, Real, Real>& D = doms[lo];
       constexpr int PW = sizeof(Params<Real, K>) / 4;
       const uint32_t* src = reinterpret_cast<const uint32_t*>(&D.P);
       uint32_t* dst = reinterpret_cast<uint32_t*>(&Psh);
@@ -92,17 +79,11 @@ batch_step_kernel(const BatchDom<K, Real, Store>* __restrict__ doms,
     const int lt = t - tile_begin[lo];
     const int nbx = (Psh.nx + T_::TX - 1) / T_::TX;
     double sI, sIn, sOut;
-    step_tile<2, K, Real, Store, T_>(Psh, Ssh, lt % nbx, lt / nbx, 0, planes, red_sh, sI, sIn,
-                                     sOut);
+    step_tile<K, Real, T_>(Psh, Ssh, lt % nbx, lt / nbx, pl, red_sh, sI, sIn, sOut);
     const unsigned nb = (unsigned)(tile_begin[lo + 1] - tile_begin[lo]);
     publish_partials_at(sI, sIn, sOut, Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0,
                         Psh.eos_c, Psh.inv_rho_ref, (unsigned)lt, nb, true);
   }
-}
-
-template <int K, class Real, class Store, class T_>
-constexpr size_t batch_smem_bytes() {
-  return sizeof(Plane<Real, K, T_::HP, n_mom<2, Store>()>);
 }
 
 }  // namespace pflb

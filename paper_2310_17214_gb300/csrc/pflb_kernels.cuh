@@ -12,18 +12,20 @@
 //   the last block to arrive.
 //
 // Layout: SoA in HBM, g[i*N + cell], Y[k*N + cell]; cell = x + nx*(y + ny*z).
-// A block owns a TX x TY tile of one or more z-planes.  It stages T, Y, phi,
-// Ts of the tile plus a one-cell halo in shared memory and evaluates the
-// per-cell properties (EOS density, viscosity, conductivity, diffusivity
-// factor) once per staged cell; the FD stencils and grad(rho) then read their
-// neighbours from shared memory.  In 3-D the block marches along z with a
-// ring of three staged planes (2.5-D blocking).  The populations are pulled
-// straight from HBM: warps map to 32 consecutive x, so every load is a
-// contiguous or one-element-shifted 128-byte line.
+// A block owns a tile of 32 columns of one or more z-planes (3-D:
+// pflb_step3d.cuh).  It stages T, Y, phi, Ts of the tile plus a one-cell halo
+// in shared memory and evaluates the per-cell properties (EOS density,
+// viscosity, conductivity, diffusivity factor) once per staged cell; the FD
+// stencils and grad(rho) then read their neighbours from shared memory.  The
+// populations are pulled straight from HBM.  In FP32 a thread owns two
+// neighbouring cells and works on them with packed arithmetic (pflb_vec.cuh).
+// FP16-stored populations have their own update (pflb_half.cuh).
 #pragma once
 
 #include <cuda_fp16.h>
 #include <stdint.h>
+
+#include "pflb_vec.cuh"
 
 namespace pflb {
 
@@ -75,22 +77,6 @@ template <> struct Lattice<3> {
   }
 };
 
-// Tile shape: TX x (256 / TX) RPT cells per plane, 256 threads; in 2-D every
-// thread can own RPT rows and issues the population loads of its cells before
-// the staging barrier (PREFETCH), so the two load phases overlap.  Measured
-// on GB300 for the single-domain step: 32 x 8 with one row per thread is
-// fastest (two rows spill at the 64-register cap); the prefetch helps the
-// FP16-stored path.  The batched step lets its autotuner pick among shapes.
-// 3-D blocks march over ZC planes.
-template <int DIM, int TXv = 32, int RPTv = 1> struct Tile {
-  static constexpr int RPT = RPTv;
-  static constexpr bool PREFETCH = DIM == 2;
-  static constexpr int TX = TXv, TY = (256 / TXv) * RPT;
-  static constexpr int ZC = DIM == 3 ? 16 : 1;
-  static constexpr int HX = TX + 2, HY = TY + 2, HP = HX * HY;
-  static constexpr int NPL = DIM == 3 ? 3 : 1;  // staged planes
-};
-
 // ------------------------------------------------------------ parameters
 // FP64 chemistry data of the implicit integrator.
 template <int K>
@@ -139,12 +125,14 @@ struct Params {
   Real u_in, T_in;
   Real Y_in[KK];
   Real M0, cp0;
-  Real invM[KK], cp[KK], hf[KK], Dlat[KK];
+  Real invM[KK], cp[KK], hf[KK];
+  Real Dlat[KK], Dlat_h[KK];  // diffusivity in lattice units, half of it
   Real cpD[KK];            // cp_k Dlat_k (enthalpy-flux cross term)
   int D_Tdep;
   Real inv_DTref, D_exp;
   int Ts_field;
-  Real Ts_uniform, Cs, Lams;  // solid rho cp / rho_ref, lambda_s dt / (rho_ref dx^2)
+  Real Ts_uniform, Cs;     // solid rho cp / rho_ref
+  Real Lams, Lams_h;       // lambda_s dt / (rho_ref dx^2), half of it
   Real phi_min;
   int chem, J;
   Real A_lat[JMAX];        // A dt / rho_ref
@@ -225,8 +213,18 @@ struct State {
   DevScalars* scal;
   double* partials;        // this step's block partials: [blocks][4]
   unsigned* counter;
+  int even;                // pairs of cells are aligned words: nx even, arrays aligned
   Real* ob;                // characteristic outlet: P_h, u_x of columns nx-1 and nx-2 and rho
                            // of column nx-1 of this step, [5][ny nz] (else null)
+};
+
+// A domain of a batch's work list (pflb_batch.cuh).
+template <int K, class Real, class Store>
+struct BatchDom {
+  Params<Real, K> P;
+  State<Real, Store> S[2];  // S[q]: input state in ping-pong buffer q
+  int p0_closed;
+  int cur0;                 // buffer holding the input at even batch steps
 };
 
 // ----------------------------------------------------- storage codecs
@@ -268,51 +266,6 @@ template <> struct Codec<__half, float> {
   }
 };
 
-// ---------------------------------------------------------- arithmetic
-// FP32 uses the fast hardware approximations (a few ulp); FP64 stays IEEE.
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
-
-// Packed FP32 pairs (the f32x2 arithmetic of sm_100 and later: one
-// instruction for two lanes of independent FP32 work).
-__device__ __forceinline__ uint64_t f2_bits(float2 v) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
-  return r;
-}
-__device__ __forceinline__ float2 f2_of(uint64_t r) {
-  float2 v;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
-  return v;
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  uint64_t d;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)),
-      "l"(f2_bits(c)));
-  return f2_of(d);
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-  uint64_t d;
-  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
-  return f2_of(d);
-}
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-  uint64_t d;
-  asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
-  return f2_of(d);
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  uint64_t d;
-  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
-  return f2_of(d);
-}
-__device__ __forceinline__ float2 splat2(float a) { return make_float2(a, a); }
-
-__device__ __forceinline__ float fexp(float x) { return __expf(x); }
-__device__ __forceinline__ double fexp(double x) { return exp(x); }
-__device__ __forceinline__ float fpow(float x, float y) { return __powf(x, y); }
-__device__ __forceinline__ double fpow(double x, double y) { return pow(x, y); }
-
 template <class Real> __device__ __forceinline__ Real scal_P0(const DevScalars* s);
 template <> __device__ __forceinline__ double scal_P0<double>(const DevScalars* s) { return s->P0; }
 template <> __device__ __forceinline__ float scal_P0<float>(const DevScalars* s) { return s->P0_f; }
@@ -330,12 +283,15 @@ template <> __device__ __forceinline__ double scal_dP0r<double>(const DevScalars
 template <> __device__ __forceinline__ float scal_dP0r<float>(const DevScalars* s) { return s->dP0r_f; }
 
 // ------------------------------------------------------------ physics
+// The per-cell functions below are written over V: one cell (Real) or a pair
+// of x-neighbours (float2), see pflb_vec.cuh.
 // Viscosity: Sutherland (Sec. 4, eq. muT) or constant, lattice units.
-template <class Real, int K>
-__device__ __forceinline__ Real viscosity(const Params<Real, K>& P, Real T) {
-  if (!P.sutherland) return P.mu_lat;
-  Real t = T * P.inv_suth_T;
-  return P.mu_lat * t * sqrt(t) * fdiv(P.suth_TS, T + P.suth_S);
+template <class Real, int K, class V>
+__device__ __forceinline__ V viscosity(const Params<Real, K>& P, V T) {
+  if (!P.sutherland) return splat<V>(P.mu_lat);
+  const V t = vmuls<V>(P.inv_suth_T, T);
+  return vmul(vmul(vmuls<V>(P.mu_lat, t), fsqrt(t)),
+              fdiv(splat<V>(P.suth_TS), vadds<V>(P.suth_S, T)));
 }
 
 // Viscosity and conductivity of the gas of composition Y at T (lattice
@@ -346,109 +302,114 @@ __device__ __forceinline__ Real viscosity(const Params<Real, K>& P, Real T) {
 // Phi_kj = (1 + sqrt(mu_k / mu_j) (M_j / M_k)^(1/4))^2 / (sqrt(8) sqrt(1 + M_k / M_j)),
 // lambda = (sum_k X_k lambda_k + 1 / sum_k X_k / lambda_k) / 2 with
 // lambda_k = mu_k (1.32 cv_k + 1.77 R / M_k).
-template <class Real, int K>
-__device__ __forceinline__ void transport(const Params<Real, K>& P, Real T, const Real* Y,
-                                          Real invMw, Real cp, Real& mu, Real& lam) {
+template <class Real, int K, class V>
+__device__ __forceinline__ void transport(const Params<Real, K>& P, V T, const V* Y, V invMw, V cp,
+                                          V& mu, V& lam) {
+  const V one = splat<V>(Real(1));
   if constexpr (K > 0) {
     if (P.mix) {
-      Real X[K], m[K], sm[K], ism[K];
-      const Real Mw = fdiv(Real(1), invMw);
+      V X[K], m[K], sm[K], ism[K];
+      const V Mw = vrcp(invMw);
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        X[k] = Y[k] * P.invM[k] * Mw;
-        const Real t = T * P.inv_suth_Tk[k];
-        m[k] = P.mu_lat_k[k] * t * sqrt(t) * fdiv(P.suth_TSk[k], T + P.suth_Sk[k]);
-        sm[k] = sqrt(m[k]);
-        ism[k] = fdiv(Real(1), sm[k]);
+        X[k] = vmul(vmuls<V>(P.invM[k], Y[k]), Mw);
+        const V t = vmuls<V>(P.inv_suth_Tk[k], T);
+        m[k] = vmul(vmul(vmuls<V>(P.mu_lat_k[k], t), fsqrt(t)),
+                    fdiv(splat<V>(P.suth_TSk[k]), vadds<V>(P.suth_Sk[k], T)));
+        sm[k] = fsqrt(m[k]);
+        ism[k] = vrcp(sm[k]);
       }
-      Real mm = 0, l1 = 0, l2 = 0;
+      V mm = splat<V>(Real(0)), l1 = mm, l2 = mm;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        Real den = 0;
+        V den = splat<V>(Real(0));
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-          const Real a = Real(1) + sm[k] * ism[j] * P.wA[k][j];
-          den += a * a * P.wB[k][j] * X[j];
+          const V a = vfma(vmuls<V>(P.wA[k][j], sm[k]), ism[j], one);
+          den = vfma(vmul(a, a), vmuls<V>(P.wB[k][j], X[j]), den);
         }
-        mm += m[k] * X[k] * fdiv(Real(1), den);
-        const Real lk = m[k] * P.eucken_k[k];
-        l1 += X[k] * lk;
-        l2 += X[k] * fdiv(Real(1), lk);
+        mm = vfma(vmul(m[k], X[k]), vrcp(den), mm);
+        const V lk = vmuls<V>(P.eucken_k[k], m[k]);
+        l1 = vfma(X[k], lk, l1);
+        l2 = vfma(X[k], vrcp(lk), l2);
       }
       mu = mm;
-      lam = Real(0.5) * (l1 + fdiv(Real(1), l2));
+      lam = vmuls<V>(Real(0.5), vadd(l1, vrcp(l2)));
       return;
     }
   }
-  mu = viscosity(P, T);
-  lam = mu * cp * P.inv_Pr;
+  mu = viscosity<Real, K, V>(P, T);
+  lam = vmuls<V>(P.inv_Pr, vmul(mu, cp));
 }
 
-template <class Real, int K>
-__device__ __forceinline__ Real mixture_invMw(const Params<Real, K>& P, const Real* Y) {
+template <class Real, int K, class V>
+__device__ __forceinline__ V mixture_invMw(const Params<Real, K>& P, const V* Y) {
   if constexpr (K == 0) {
-    return Real(1) / P.M0;
+    return splat<V>(fdiv(Real(1), P.M0));
   } else {
-    Real s = 0;
+    V s = vmuls<V>(P.invM[0], Y[0]);
 #pragma unroll
-    for (int k = 0; k < K; ++k) s += Y[k] * P.invM[k];
+    for (int k = 1; k < K; ++k) s = vfmas<V>(P.invM[k], Y[k], s);
     return s;
   }
 }
 
-template <class Real, int K>
-__device__ __forceinline__ Real mixture_cp(const Params<Real, K>& P, const Real* Y) {
+template <class Real, int K, class V>
+__device__ __forceinline__ V mixture_cp(const Params<Real, K>& P, const V* Y) {
   if constexpr (K == 0) {
-    return P.cp0;
+    return splat<V>(P.cp0);
   } else {
-    Real s = 0;
+    V s = vmuls<V>(P.cp[0], Y[0]);
 #pragma unroll
-    for (int k = 0; k < K; ++k) s += Y[k] * P.cp[k];
+    for (int k = 1; k < K; ++k) s = vfmas<V>(P.cp[k], Y[k], s);
     return s;
   }
 }
 
 // Explicit Arrhenius rates (Sec. 3.2.2 eq. 8, Sec. 3.3 eq. 9), per lattice
 // step per rho_ref: om[k] = omega_k dt / rho_ref, omT likewise (J/kg).
-template <class Real, int K>
-__device__ __forceinline__ void rates(const Params<Real, K>& P, Real T, const Real* Y, Real rho,
-                                      Real invT, Real* om, Real& omT) {
+template <class Real, int K, class V>
+__device__ __forceinline__ void rates(const Params<Real, K>& P, V T, const V* Y, V rho, V invT,
+                                      V* om, V& omT) {
+  const V zero = splat<V>(Real(0));
 #pragma unroll
-  for (int k = 0; k < K; ++k) om[k] = 0;
-  Real C[Params<Real, K>::KK];
+  for (int k = 0; k < K; ++k) om[k] = zero;
+  V C[Params<Real, K>::KK];
 #pragma unroll
-  for (int k = 0; k < K; ++k) C[k] = rho * P.rho_ref_M[k] * (Y[k] > Real(0) ? Y[k] : Real(0));
+  for (int k = 0; k < K; ++k)
+    C[k] = vmul(vmuls<V>(P.rho_ref_M[k], rho), vsel(vgt(Y[k], zero), Y[k], zero));
 #pragma unroll 1
   for (int j = 0; j < P.J; ++j) {
-    Real kf = P.A_lat[j] * fexp(-P.EaR[j] * invT);
-    if (P.b[j] != Real(0)) kf *= fpow(T, P.b[j]);
-    Real q = kf;
+    V kf = vmuls<V>(P.A_lat[j], fexp(vmuls<V>(-P.EaR[j], invT)));
+    if (P.b[j] != Real(0)) kf = vmul(kf, fpow(T, P.b[j]));
+    V q = kf;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const Real o = P.order[j][k];
-      if (o == Real(1)) q *= C[k];
-      else if (o == Real(2)) q *= C[k] * C[k];
-      else if (o != Real(0)) q *= fpow(C[k], o);
+      if (o == Real(1)) q = vmul(q, C[k]);
+      else if (o == Real(2)) q = vmul(q, vmul(C[k], C[k]));
+      else if (o != Real(0)) q = vmul(q, fpow(C[k], o));
     }
     if (P.rev[j]) {
       // k_r = k_f / K_c, K_c = exp(dS/R - dH/(R T)) (p_ref/(R T))^(sum s)
-      const Real Kc = fexp(P.dS_R[j] - P.dH_R[j] * invT) * fpow(P.p_ref_R * invT, P.dn[j]);
-      Real qr = fdiv(kf, Kc);
+      const V Kc = vmul(fexp(vfmas<V>(-P.dH_R[j], invT, splat<V>(P.dS_R[j]))),
+                        fpow(vmuls<V>(P.p_ref_R, invT), P.dn[j]));
+      V qr = fdiv(kf, Kc);
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const Real o = P.rorder[j][k];
-        if (o == Real(1)) qr *= C[k];
-        else if (o == Real(2)) qr *= C[k] * C[k];
-        else if (o != Real(0)) qr *= fpow(C[k], o);
+        if (o == Real(1)) qr = vmul(qr, C[k]);
+        else if (o == Real(2)) qr = vmul(qr, vmul(C[k], C[k]));
+        else if (o != Real(0)) qr = vmul(qr, fpow(C[k], o));
       }
-      q -= qr;
+      q = vsub(q, qr);
     }
 #pragma unroll
-    for (int k = 0; k < K; ++k) om[k] += P.stoichM[j][k] * q;
+    for (int k = 0; k < K; ++k) om[k] = vfmas<V>(P.stoichM[j][k], q, om[k]);
   }
-  Real wt = 0;
+  V wt = zero;
 #pragma unroll
-  for (int k = 0; k < K; ++k) wt -= P.hf[k] * om[k];
+  for (int k = 0; k < K; ++k) wt = vfmas<V>(-P.hf[k], om[k], wt);
   omT = wt;
 }
 
@@ -874,10 +835,10 @@ __device__ __forceinline__ Real first_order(const MA& A, int i, int src, int dx,
   Real cj = 0;
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {
-    if (L::c(i, a) > 0) cj += A.mom(1 + a, src, dx, dy, dz);
-    if (L::c(i, a) < 0) cj -= A.mom(1 + a, src, dx, dy, dz);
+    if (L::c(i, a) > 0) cj = vadd(cj, A.mom(1 + a, src, dx, dy, dz));
+    if (L::c(i, a) < 0) cj = vsub(cj, A.mom(1 + a, src, dx, dy, dz));
   }
-  return Real(L::w(i)) * (A.mom(0, src, dx, dy, dz) + Real(3) * cj);
+  return vmul(Real(L::w(i)), vfma(Real(3), cj, A.mom(0, src, dx, dy, dz)));
 }
 
 template <class Real, int K>
@@ -888,7 +849,7 @@ __device__ __forceinline__ Real inlet_u(const Params<Real, K>& P, Real u, const 
     if (P.bc[2 * a] != BC_WALL) continue;
     Real n = Real(a == 1 ? P.ny : P.nz);
     Real s = Real(xyz[a]) + Real(0.5);
-    u *= Real(4) * s * (n - s) / (n * n);
+    u = vmul(u, fdiv(vmul(vmul(Real(4), s), vsub(n, s)), vmul(n, n)));
   }
   return u;
 }
@@ -917,22 +878,80 @@ __device__ __forceinline__ void wall_pops(const Params<Real, K>& P, const State<
     if (L::c(i, a) != s) continue;
     Real cu = 0;
 #pragma unroll
-    for (int b = 0; b < DIM; ++b) cu += Real(L::c(i, b)) * P.wall_u[F][b];
-    gin[i] = own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom) +
-             Real(2) * Real(L::w(i)) * rho_c * cu;
+    for (int b = 0; b < DIM; ++b) {
+      if (L::c(i, b) > 0) cu = vadd(cu, P.wall_u[F][b]);
+      if (L::c(i, b) < 0) cu = vsub(cu, P.wall_u[F][b]);
+    }
+    gin[i] = vfma(vmul(Real(2 * L::w(i)), rho_c), cu,
+                  own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom));
   }
+}
+
+// The boundary rules of a cell on non-periodic faces: directions that cross a
+// non-periodic face are replaced, in the order outlet, inlet, walls (the wall
+// of the lowest axis last, so it wins on edges and corners): half-way
+// bounce-back on walls (moving walls add 2 w rho c.u_w), the inlet as a moving
+// wall with the inlet velocity and inlet density, the outlet as
+// anti-bounce-back at P_h = 0 with wall velocity uw.
+template <int DIM, class Real, class Store, int K, class MA>
+__device__ __forceinline__ void edge_rules(const Params<Real, K>& P, const State<Real, Store>& S,
+                                           int c, const int xyz[3], Real rho_c, Real rho_in,
+                                           const Real* uw, Real* gin, const MA& mom) {
+  using L = Lattice<DIM>;
+  const int x = xyz[0], y = xyz[1], z = DIM == 3 ? xyz[2] : 0;
+  const bool per0 = P.bc[0] == BC_PERIODIC, per1 = P.bc[1] == BC_PERIODIC;
+  const bool per2 = P.bc[2] == BC_PERIODIC, per3 = P.bc[3] == BC_PERIODIC;
+  const bool per4 = P.bc[4] == BC_PERIODIC, per5 = P.bc[5] == BC_PERIODIC;
+  // non-periodic faces the cell lies on
+  const bool f0 = x == 0 && !per0, f1 = x == P.nx - 1 && !per1;
+  const bool f2 = y == 0 && !per2, f3 = y == P.ny - 1 && !per3;
+  const bool f4 = DIM == 3 && z == 0 && !per4, f5 = DIM == 3 && z == P.nz - 1 && !per5;
+  if (!(f0 || f1 || f2 || f3 || f4 || f5)) return;
+  if (f1 && P.bc[1] == BC_OUTLET) {
+    Real uu = 0;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) uu = vfma(uw[a], uw[a], uu);
+    const Real pb2 = P.nscbc ? Real(2) * scal_pb<Real>(S.scal) : Real(0);
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+      if (L::c(i, 0) != -1) continue;
+      Real cu = 0;
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) {
+        if (L::c(i, a) > 0) cu = vadd(cu, uw[a]);
+        if (L::c(i, a) < 0) cu = vsub(cu, uw[a]);
+      }
+      gin[i] = vfma(Real(L::w(i)), vfma(rho_c, vfma(vmul(Real(3), cu), cu, -uu), pb2),
+                    -own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom));
+    }
+  }
+  if (f0 && P.bc[0] == BC_INLET) {
+    Real ui = inlet_u(P, P.feed ? scal_u_in<Real>(S.scal) : P.u_in, xyz, DIM);
+    if (P.inlet_parabolic == 2) ui = vmul(ui, vsub(Real(1), S.phi[c]));
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+      if (L::c(i, 0) != 1) continue;
+      gin[i] = vfma(vmul(Real(2 * L::w(i)), rho_in), ui,
+                    own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom));
+    }
+  }
+  // walls, the highest axis first so that the lowest axis wins on edges
+  if (DIM == 3) {
+    wall_pops<DIM, 5>(P, S, c, f5, rho_c, gin, mom);
+    wall_pops<DIM, 4>(P, S, c, f4, rho_c, gin, mom);
+  }
+  wall_pops<DIM, 3>(P, S, c, f3, rho_c, gin, mom);
+  wall_pops<DIM, 2>(P, S, c, f2, rho_c, gin, mom);
+  wall_pops<DIM, 1>(P, S, c, f1, rho_c, gin, mom);
+  wall_pops<DIM, 0>(P, S, c, f0, rho_c, gin, mom);
 }
 
 // Pull streaming of every population into the cell.  A cell off every face
 // reads its upstream neighbours at fixed offsets.  On a face, along each axis
 // the upstream neighbour coordinate wraps across a periodic face and is
 // clamped to the cell itself across any other face; every direction is read
-// from there.  Directions that cross a non-periodic face are then replaced by the
-// boundary rules, in the order outlet, inlet, walls (the wall of the lowest
-// axis last, so it wins on edges and corners): half-way bounce-back on walls
-// (moving walls add 2 w rho c.u_w), the inlet as a moving wall with the inlet
-// velocity and inlet density, the outlet as anti-bounce-back at P_h = 0 with
-// wall velocity uw.
+// from there.  Directions that cross a non-periodic face are then replaced by
+// the boundary rules.
 template <int DIM, class Real, class Store, int K, class MA>
 __device__ __forceinline__ void pull(const Params<Real, K>& P, const State<Real, Store>& S, int c,
                                      const int xyz[3], Real rho_c, Real rho_in, const Real* uw,
@@ -982,45 +1001,7 @@ __device__ __forceinline__ void pull(const Params<Real, K>& P, const State<Real,
                                        first_order<DIM, Real>(mom, i, src, -cx, -cy, -cz));
     else gin[i] = r;
   }
-  // non-periodic faces the cell lies on
-  const bool f0 = x == 0 && !per0, f1 = x == P.nx - 1 && !per1;
-  const bool f2 = y == 0 && !per2, f3 = y == P.ny - 1 && !per3;
-  const bool f4 = DIM == 3 && z == 0 && !per4, f5 = DIM == 3 && z == P.nz - 1 && !per5;
-  if (!(f0 || f1 || f2 || f3 || f4 || f5)) return;
-  if (f1 && P.bc[1] == BC_OUTLET) {
-    Real uu = 0;
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) uu += uw[a] * uw[a];
-    const Real pb2 = P.nscbc ? Real(2) * scal_pb<Real>(S.scal) : Real(0);
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-      if (L::c(i, 0) != -1) continue;
-      Real cu = 0;
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) cu += Real(L::c(i, a)) * uw[a];
-      gin[i] = -own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom) +
-               Real(L::w(i)) * (pb2 + rho_c * (Real(3) * cu * cu - uu));
-    }
-  }
-  if (f0 && P.bc[0] == BC_INLET) {
-    Real ui = inlet_u(P, P.feed ? scal_u_in<Real>(S.scal) : P.u_in, xyz, DIM);
-    if (P.inlet_parabolic == 2) ui *= Real(1) - S.phi[c];
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-      if (L::c(i, 0) != 1) continue;
-      gin[i] = own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom) +
-               Real(2) * Real(L::w(i)) * rho_in * ui;
-    }
-  }
-  // walls, the highest axis first so that the lowest axis wins on edges
-  if (DIM == 3) {
-    wall_pops<DIM, 5>(P, S, c, f5, rho_c, gin, mom);
-    wall_pops<DIM, 4>(P, S, c, f4, rho_c, gin, mom);
-  }
-  wall_pops<DIM, 3>(P, S, c, f3, rho_c, gin, mom);
-  wall_pops<DIM, 2>(P, S, c, f2, rho_c, gin, mom);
-  wall_pops<DIM, 1>(P, S, c, f1, rho_c, gin, mom);
-  wall_pops<DIM, 0>(P, S, c, f0, rho_c, gin, mom);
+  edge_rules<DIM>(P, S, c, xyz, rho_c, rho_in, uw, gin, mom);
 }
 
 // ----------------------------------------------------------- reductions
@@ -1035,10 +1016,12 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // values are summed within the warp with compensation (the pair s + e is
 // exact up to the final rounding), warps are combined in FP64.
 // Warp part of the sums below (result in lane 0).
-template <class Real>
-__device__ __forceinline__ double warp_sum(Real v) {
-  if constexpr (sizeof(Real) == 4) {
-    float s = v, e = 0.f;
+template <class V>
+__device__ __forceinline__ double warp_sum(V v) {
+  if constexpr (sizeof(typename Lanes<V>::S) == 4) {
+    float s, e = 0.f;
+    if constexpr (Lanes<V>::n == 2) two_sum(v.x, v.y, s, e);
+    else s = v;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const float so = __shfl_down_sync(0xffffffffu, s, o);
@@ -1060,8 +1043,8 @@ __device__ __forceinline__ double warp_sum(Real v) {
 // The three sums of a tile (I, and the two fluxes when `bc` holds) with one
 // barrier, grouped exactly as block_sum; results valid in thread 0.  `sh`
 // holds 96 doubles and is free again after the block's next barrier.
-template <class Real>
-__device__ __forceinline__ void block_sum3(Real a, Real b, Real c, bool bc, double* sh,
+template <class V, class Real>
+__device__ __forceinline__ void block_sum3(V a, Real b, Real c, bool bc, double* sh,
                                            double& ra, double& rb, double& rc) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const double wa = warp_sum(a);
@@ -1238,349 +1221,508 @@ static __global__ void finalize_kernel(const double* partials, unsigned nb, DevS
   combine_partials(partials, nb, scal, 0, false, 0.0, eos_c, inv_rho_ref);
 }
 
+// ------------------------------------------------------------ tiles
+// A block owns TX x TY cells of a plane; a thread owns LN neighbouring cells
+// in x (two in FP32 compute, one in FP64) in each of RPT rows.
+//
+// Two cells per thread in FP32: one cell per thread was bound by instruction
+// issue, and a pair halves it -- packed f32x2 arithmetic, 64-bit shared-memory
+// and global accesses, one set of addresses and parameter reads for two cells:
+// 1,742 -> 847 warp instructions x 32 per cell of the 3-D bed.  Now bound by
+// latency (10 to 16 warps per SM, a third of the issue slots used): 256 x 128 x
+// 128 bed 394 -> 249 us a step, 1024 x 256 bed 17.5 -> 15.5, 48 channel beds 365
+// -> 288.  FP64 is bound by the FP64 pipe; sharing te / to between opposite
+// directions, the face sums and the reciprocals below took the 1001 x 251 bed
+// from 410 to 320 us.
+template <class Real> struct VecOf { using V = Real; };
+template <> struct VecOf<float> { using V = float2; };
+
+template <class V_, int TXv, int TYv, int RPTv = 1> struct Tile {
+  using V = V_;
+  static constexpr int LN = Lanes<V>::n;
+  static constexpr int TX = TXv, TY = TYv;
+  static constexpr int RPT = TX * TY / LN / RPTv > 256 ? TX * TY / LN / 256 : RPTv;
+  static constexpr int NT = TX * TY / LN / RPT;  // threads
+  static constexpr int TXT = TX / LN;            // threads per row
+  // staged rows start LN cells left of the tile, so that a pair of cells is
+  // an aligned 64-bit word of its row
+  static constexpr int XO = LN;
+  static constexpr int HX = TX + 2 * XO, HY = TY + 2, HP = HX * HY;
+};
+
 // ------------------------------------------------ staged tile (smem)
 // Fields per staged cell: T, phi_s, rho, kappa_T = phi_f lambda, mu, f_D
 // (diffusivity factor), Ts, phi_f rho f_D, then Y_k.
 enum { F_T = 0, F_PHI, F_RHO, F_KT, F_MU, F_FD, F_TS, F_RF, F_Y0 };
 
-template <class Real, int K, int HP, int NM = 0>
-struct Plane {
-  Real f[F_Y0 + K + NM][HP];  // NM moment fields (P, j) after the species
-};
+// A pair / a cell of an array: `even` says that a pair is one aligned word
+// (State::even), `two` that the second cell of the pair exists.
+template <class V, class T>
+__device__ __forceinline__ V load_cells(const T* __restrict__ p, bool even, bool two);
+template <> __device__ __forceinline__ double load_cells<double, double>(const double* __restrict__ p, bool, bool) {
+  return __ldg(p);
+}
+template <> __device__ __forceinline__ float load_cells<float, float>(const float* __restrict__ p, bool, bool) {
+  return __ldg(p);
+}
+template <> __device__ __forceinline__ float2 load_cells<float2, float>(const float* __restrict__ p, bool even,
+                                                                        bool two) {
+  if (even) return __ldg(reinterpret_cast<const float2*>(p));
+  return make_float2(__ldg(p), two ? __ldg(p + 1) : 0.f);
+}
+__device__ __forceinline__ void store_cells(double* p, double v, bool, bool) { *p = v; }
+__device__ __forceinline__ void store_cells(float* p, float v, bool, bool) { *p = v; }
+__device__ __forceinline__ void store_cells(float* p, float2 v, bool even, bool two) {
+  if (even) {
+    *reinterpret_cast<float2*>(p) = v;
+  } else {
+    p[0] = v.x;
+    if (two) p[1] = v.y;
+  }
+}
+// Values of the staged fields of one position (cell or pair) into the plane.
+template <int K, class Real, class V, int HP>
+__device__ __forceinline__ void stage_fields(const Params<Real, K>& P, Real* __restrict__ pl, int h,
+                                             V T, V phis, V Ts, const V* Y, Real P0) {
+  const V one = splat<V>(Real(1));
+  const V phif = vsub(one, phis);
+  const V invMw = mixture_invMw<Real, K, V>(P, Y);
+  const V rho = fdiv(splat<V>(P0 * P.eos_cr), vmul(T, invMw));
+  const V cp = mixture_cp<Real, K, V>(P, Y);
+  V mu, lam;
+  transport<Real, K, V>(P, T, Y, invMw, cp, mu, lam);
+  V fD = one;
+  if constexpr (K > 0) {
+    if (P.D_Tdep) fD = fpow(vmuls<V>(P.inv_DTref, T), P.D_exp);
+  }
+  auto put = [&](int f, V v) { *reinterpret_cast<V*>(pl + f * HP + h) = v; };
+  put(F_T, T);
+  put(F_PHI, phis);
+  put(F_RHO, rho);
+  put(F_KT, vmul(phif, lam));
+  put(F_MU, mu);
+  put(F_FD, fD);
+  put(F_TS, Ts);
+  put(F_RF, vmul(vmul(phif, rho), fD));
+#pragma unroll
+  for (int k = 0; k < K; ++k) put(F_Y0 + k, Y[k]);
+}
+
+// Coordinate v of an axis of n cells: wrapped on periodic faces, else clamped.
+__device__ __forceinline__ int wrap_or_clamp(int v, int n, bool per) {
+  if (v < 0) v = per ? v + n : 0;
+  if (v >= n) v = per ? v - n : n - 1;
+  return v < 0 ? 0 : (v >= n ? n - 1 : v);  // tiles wider than n
+}
 
 // Stage plane z (may be -1 or nz: ghost plane) of the block's tile with its
-// xy halo.  Out-of-domain halo cells follow the ghost rules: periodic faces
-// wrap; otherwise the adjacent cell's values, with the inlet state (T_in,
-// Y_in) on the inlet face and the wall temperature on a wall that has one.
-template <int DIM, class Real, class Store, int K, int HP, class T_ = Tile<DIM>,
-          int NM = n_mom<DIM, Store>()>
-__device__ __forceinline__ void stage_plane(const Params<Real, K>& P, const State<Real, Store>& S,
-                                            Plane<Real, K, HP, NM>& pl, int x0, int y0, int z,
-                                            Real P0) {
-  static_assert(T_::HP == HP, "plane and tile shape disagree");
+// xy halo into `pl` ([fields][HP]).  Out-of-domain halo cells follow the ghost
+// rules: periodic faces wrap; otherwise the adjacent cell's values, with the
+// inlet state (T_in, Y_in) on the inlet face and the wall temperature on a
+// wall that has one.
+template <int DIM, int K, class Real, class T_>
+__device__ __forceinline__ void stage_plane(const Params<Real, K>& P, const State<Real, Real>& S,
+                                            Real* __restrict__ pl, int x0, int y0, int z, Real P0) {
+  using V = typename T_::V;
+  constexpr int LN = T_::LN, HP = T_::HP, PW = T_::HX / LN;
+  constexpr int KK = Params<Real, K>::KK;
   // tiles whose halo lies inside the lattice need no ghost rules
-  const bool inner = x0 >= 1 && y0 >= 1 && x0 + T_::TX < P.nx && y0 + T_::TY < P.ny &&
+  const bool inner = x0 >= LN && y0 >= 1 && x0 + T_::TX + LN <= P.nx && y0 + T_::TY < P.ny &&
                      (DIM == 2 || (z >= 0 && z < P.nz));
-  for (int h = threadIdx.x; h < HP; h += blockDim.x) {
-    const int hx = h % T_::HX, hy = h / T_::HX;
-    int q[3] = {x0 - 1 + hx, y0 - 1 + hy, z};
-    int ghost_face = -1;
-    int nout = 0;
+  const bool even = LN == 1 || S.even;
+  struct Raw { V T, phis, Ts, Y[KK]; };
+  auto load = [&](int p, Raw& R) {
+    V &T = R.T, &phis = R.phis, &Ts = R.Ts, *Y = R.Y;
+    const int hy = p / PW, hx = (p - hy * PW) * LN;
+    const int x = x0 - LN + hx, y = y0 - 1 + hy;
+    // source columns of the position's cells, start of the source row
+    int xa = x, xb = x + 1, row = P.nx * (y + P.ny * z);
+    if (!inner) {
+      const bool per0 = P.bc[0] == BC_PERIODIC;
+      xa = wrap_or_clamp(x, P.nx, per0);
+      xb = wrap_or_clamp(x + 1, P.nx, per0);
+      const int yc = wrap_or_clamp(y, P.ny, P.bc[2] == BC_PERIODIC);
+      const int zc = DIM == 3 ? wrap_or_clamp(z, P.nz, P.bc[4] == BC_PERIODIC) : 0;
+      row = P.nx * (yc + P.ny * zc);
+    }
+    if (LN == 1 || (even && xb == xa + 1 && (xa & 1) == 0)) {
+      const int c = row + xa;
+      T = load_cells<V>(S.T_in + c, true, true);
+      phis = load_cells<V>(S.phi + c, true, true);
+      Ts = P.Ts_field ? load_cells<V>(S.Ts_in + c, true, true) : splat<V>(P.Ts_uniform);
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      if (inner) break;
-      const int n = a == 0 ? P.nx : (a == 1 ? P.ny : P.nz);
-      if (q[a] < 0 || q[a] >= n) {
-        const int face = 2 * a + (q[a] >= n ? 1 : 0);
-        if (P.bc[face] == BC_PERIODIC) {
-          q[a] = q[a] < 0 ? q[a] + n : q[a] - n;
-          if (q[a] < 0 || q[a] >= n) q[a] = q[a] < 0 ? 0 : n - 1;  // tiles wider than n
-        } else {
-          q[a] = q[a] < 0 ? 0 : n - 1;
-          ghost_face = face;
-          ++nout;
+      for (int k = 0; k < K; ++k) Y[k] = load_cells<V>(S.Y_in + (size_t)k * P.N + c, true, true);
+    } else {
+      const int ca = row + xa, cb = row + xb;
+      auto two = [&](const Real* b) {
+        V v;
+        set_lane(v, 0, __ldg(b + ca));
+        set_lane(v, LN - 1, __ldg(b + cb));
+        return v;
+      };
+      T = two(S.T_in);
+      phis = two(S.phi);
+      Ts = P.Ts_field ? two(S.Ts_in) : splat<V>(P.Ts_uniform);
+#pragma unroll
+      for (int k = 0; k < K; ++k) Y[k] = two(S.Y_in + (size_t)k * P.N);
+    }
+    if (!inner) {
+      // one step outside exactly one non-periodic face: the face's ghost state
+      const int fy = y < 0 ? 2 : (y >= P.ny ? 3 : -1);
+      const int fz = DIM == 3 ? (z < 0 ? 4 : (z >= P.nz ? 5 : -1)) : -1;
+      const bool gy = fy >= 0 && P.bc[fy] != BC_PERIODIC, gz = fz >= 0 && P.bc[fz] != BC_PERIODIC;
+#pragma unroll
+      for (int l = 0; l < LN; ++l) {
+        const int fx = x + l < 0 ? 0 : (x + l >= P.nx ? 1 : -1);
+        const bool gx = fx >= 0 && P.bc[fx] != BC_PERIODIC;
+        if ((gx ? 1 : 0) + (gy ? 1 : 0) + (gz ? 1 : 0) != 1) continue;
+        const int face = gx ? fx : (gy ? fy : fz);
+        const int bc = P.bc[face];
+        if (bc == BC_INLET) {
+          set_lane(T, l, P.T_in);
+#pragma unroll
+          for (int k = 0; k < K; ++k) set_lane(Y[k], l, P.Y_in[k]);
+        } else if (bc == BC_WALL && P.wall_T[face] > Real(0)) {
+          set_lane(T, l, P.wall_T[face]);
         }
       }
     }
-    const int c = q[0] + P.nx * (q[1] + P.ny * q[2]);
-    Real T = __ldg(S.T_in + c);
-    const Real phis = __ldg(S.phi + c);
-    const Real Ts = P.Ts_field ? __ldg(S.Ts_in + c) : P.Ts_uniform;
-    Real Y[Params<Real, K>::KK];
-#pragma unroll
-    for (int k = 0; k < K; ++k) Y[k] = __ldg(S.Y_in + (size_t)k * P.N + c);
-    if (nout == 1) {
-      const int bc = P.bc[ghost_face];
-      if (bc == BC_INLET) {
-        T = P.T_in;
-#pragma unroll
-        for (int k = 0; k < K; ++k) Y[k] = P.Y_in[k];
-      } else if (bc == BC_WALL && P.wall_T[ghost_face] > Real(0)) {
-        T = P.wall_T[ghost_face];
-      }
+  };
+  auto finish = [&](int p, const Raw& R) {
+    const int hy = p / PW, hx = (p - hy * PW) * LN;
+    stage_fields<K, Real, V, HP>(P, pl, hy * T_::HX + hx, R.T, R.phis, R.Ts, R.Y, P0);
+  };
+  if constexpr (DIM == 2 && K == 0) {
+    // two positions' loads in flight (with species their registers spill)
+    for (int p = threadIdx.x; p < PW * T_::HY; p += 2 * T_::NT) {
+      Raw a, b;
+      const bool second = p + T_::NT < PW * T_::HY;
+      load(p, a);
+      if (second) load(p + T_::NT, b);
+      finish(p, a);
+      if (second) finish(p + T_::NT, b);
     }
-    const Real phif = Real(1) - phis;
-    const Real invMw = mixture_invMw(P, Y);
-    const Real rho = fdiv(P0 * P.eos_cr, T * invMw);
-    const Real cp = mixture_cp(P, Y);
-    Real mu, lam;
-    transport(P, T, Y, invMw, cp, mu, lam);
-    Real fD = Real(1);
-    if constexpr (K > 0) {
-      if (P.D_Tdep) fD = fpow(T * P.inv_DTref, P.D_exp);
-    }
-    pl.f[F_T][h] = T;
-    pl.f[F_PHI][h] = phis;
-    pl.f[F_RHO][h] = rho;
-    pl.f[F_KT][h] = phif * lam;
-    pl.f[F_MU][h] = mu;
-    pl.f[F_FD][h] = fD;
-    pl.f[F_TS][h] = Ts;
-    pl.f[F_RF][h] = phif * rho * fD;
-#pragma unroll
-    for (int k = 0; k < K; ++k) pl.f[F_Y0 + k][h] = Y[k];
-    if constexpr (NM > 0) {
-#pragma unroll
-      for (int a = 0; a < NM; ++a) pl.f[F_Y0 + K + a][h] = __ldg(S.M_in + (size_t)a * P.N + c);
+  } else {
+    for (int p = threadIdx.x; p < PW * T_::HY; p += T_::NT) {
+      Raw a;
+      load(p, a);
+      finish(p, a);
     }
   }
 }
 
-// Staged-plane accessor: own and neighbour values of the staged fields and
-// properties (the populations come from global memory).
-template <int DIM, class Real, bool PRE = false, class TL = Tile<DIM>, int MF = 0,
-          bool STASH = false>
+// Accessor of the update over the staged planes: own and neighbour values (a
+// neighbour of a pair in x is half of the pair itself and one more cell).
+template <class Real, class T_>
 struct PlaneAcc {
-  static constexpr int HP = TL::HP;
-  static constexpr bool has_pops = PRE;  // populations prefetched into registers
-  static constexpr bool kStash = STASH;  // pulled populations wait in shared memory
+  using V = typename T_::V;
+  static constexpr int HP = T_::HP;
   const Real* __restrict__ cen;
   const Real* __restrict__ zm;
   const Real* __restrict__ zp;
   int h;
-  const Real* pre;
-  bool pv;  // pre holds this cell's populations
-  Real* st; // stash, [Q][BLOCK] (STASH)
-  __device__ __forceinline__ Real c(int f) const { return cen[f * HP + h]; }
-  __device__ __forceinline__ Real n(int f, int a, int s) const {
-    if (a == 0) return cen[f * HP + h + s];
-    if (a == 1) return cen[f * HP + h + s * TL::HX];
-    return (s < 0 ? zm : zp)[f * HP + h];
+  __device__ __forceinline__ V c(int f) const {
+    return *reinterpret_cast<const V*>(cen + f * HP + h);
   }
-  template <class Store>
-  __device__ __forceinline__ Real pop(int i, Real) const { return PRE ? pre[i] : Real(0); }
-  // moment a of the staged cell at offset (dx, dy, dz) (FP16 storage; MF is
-  // the first moment field, src the cell's global index, unused here)
-  __device__ __forceinline__ Real mom(int a, int, int dx, int dy, int dz) const {
-    const Real* p = dz < 0 ? zm : (dz > 0 ? zp : cen);
-    return p[(MF + a) * HP + h + dx + dy * TL::HX];
+  __device__ __forceinline__ V n(int f, int a, int s, V own) const {
+    if (a == 0) {
+      const Real v = cen[f * HP + h + (s < 0 ? -1 : T_::LN)];
+      if constexpr (T_::LN == 1) return v;
+      else return s < 0 ? make_float2(v, own.x) : make_float2(own.y, v);
+    }
+    if (a == 1) return *reinterpret_cast<const V*>(cen + f * HP + h + s * T_::HX);
+    return *reinterpret_cast<const V*>((s < 0 ? zm : zp) + f * HP + h);
   }
 };
 
+// ------------------------------------------------------------ streaming
+// Faces that a cell lies on and that are not periodic.
+struct Faces {
+  bool f[6];
+  __device__ __forceinline__ bool any() const {
+    return f[0] || f[1] || f[2] || f[3] || f[4] || f[5];
+  }
+};
+template <int DIM, class Real, int K>
+__device__ __forceinline__ Faces faces_of(const Params<Real, K>& P, int x, int y, int z) {
+  Faces e;
+  e.f[0] = x == 0 && P.bc[0] != BC_PERIODIC;
+  e.f[1] = x == P.nx - 1 && P.bc[1] != BC_PERIODIC;
+  e.f[2] = y == 0 && P.bc[2] != BC_PERIODIC;
+  e.f[3] = y == P.ny - 1 && P.bc[3] != BC_PERIODIC;
+  e.f[4] = DIM == 3 && z == 0 && P.bc[4] != BC_PERIODIC;
+  e.f[5] = DIM == 3 && z == P.nz - 1 && P.bc[5] != BC_PERIODIC;
+  return e;
+}
+// Populations that stream into the cell(s) starting at x: the upstream
+// neighbour coordinate wraps across a periodic face and is clamped to the
+// cell across any other face (the boundary rules then replace those values).
+// Along x a pair reads columns x-1, x (directions to +x), x, x+1 (an aligned
+// pair when rows are even) and x+1, x+2 (directions to -x).
+template <int DIM, int K, class Real, class V>
+__device__ __forceinline__ void load_pops(const Params<Real, K>& P, const State<Real, Real>& S,
+                                          int x, int y, int z, V* __restrict__ out) {
+  using L = Lattice<DIM>;
+  constexpr int LN = Lanes<V>::n;
+  const bool per0 = P.bc[0] == BC_PERIODIC, per2 = P.bc[2] == BC_PERIODIC,
+             per4 = P.bc[4] == BC_PERIODIC;
+  const int xm = x > 0 ? x - 1 : (per0 ? P.nx - 1 : x);
+  const int x1 = x + 1 < P.nx ? x + 1 : (per0 ? 0 : x);
+  const int x2 = x + 2 < P.nx ? x + 2 : (per0 ? x + 2 - P.nx : x1);
+  const int ym = y > 0 ? y - 1 : (per2 ? P.ny - 1 : y);
+  const int yp = y < P.ny - 1 ? y + 1 : (per2 ? 0 : y);
+  int zz[3] = {0, 0, 0};
+  if (DIM == 3) {
+    zz[0] = z > 0 ? z - 1 : (per4 ? P.nz - 1 : z);
+    zz[1] = z;
+    zz[2] = z < P.nz - 1 ? z + 1 : (per4 ? 0 : z);
+  }
+  int row[3][3];  // [1 + dz][1 + dy]: start of the row
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    if (DIM == 2 && b != 1) continue;
+    row[b][0] = P.nx * (ym + P.ny * zz[b]);
+    row[b][1] = P.nx * (y + P.ny * zz[b]);
+    row[b][2] = P.nx * (yp + P.ny * zz[b]);
+  }
+  const bool even = S.even;
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const int cx = L::c(i, 0), r = row[DIM == 3 ? 1 - L::c(i, 2) : 1][1 - L::c(i, 1)];
+    const Real* g = S.g_in + (size_t)i * P.N;
+    if constexpr (LN == 1) {
+      out[i] = __ldg(g + (r + (cx > 0 ? xm : (cx < 0 ? x1 : x))));
+    } else if (cx == 0 && even) {
+      out[i] = __ldg(reinterpret_cast<const float2*>(g + (r + x)));
+    } else {
+      out[i].x = __ldg(g + (r + (cx > 0 ? xm : (cx < 0 ? x1 : x))));
+      out[i].y = __ldg(g + (r + (cx > 0 ? x : (cx < 0 ? x2 : x1))));
+    }
+  }
+}
 
 // ------------------------------------------------------ the fused step
+// Where a thread's cell or pair lies: lattice index of the first cell, the
+// coordinates, whether pairs are aligned words, whether a second cell exists.
+struct CellPos {
+  int c, x, y, z;
+  bool even, two;
+};
+
 // Per cell: (a1) pull + moments + implicit drag, (c) reaction source,
 // (b) FD transport of Y_k, T, Ts, low-Mach divergence, (a) source + BGK
-// collision + store, (d) contribution to the FP64 reduction.
-template <int DIM, int K, class Real, class Store, class Acc>
-__device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const State<Real, Store>& S,
-                                            const Acc& A, int c, const int xyz[3], Real P0,
-                                            Real dlnP0, Real dP0r, Real& fin, Real& fout) {
+// collision + store, (d) contribution to the FP64 reduction (returned per
+// cell; fluxes through the inlet / outlet face in fin, fout).  `gin` holds the
+// streamed populations (load_pops) and is overwritten.
+template <int DIM, int K, class Real, class V, class Acc>
+__device__ __forceinline__ V cell_update(const Params<Real, K>& P, const State<Real, Real>& S,
+                                         const Acc& A, V* __restrict__ gin, const CellPos q,
+                                         Real P0, Real dlnP0, Real dP0r, Real& fin, Real& fout) {
   using L = Lattice<DIM>;
   constexpr int Q = L::Q;
   constexpr int KK = Params<Real, K>::KK;
+  constexpr int LN = Lanes<V>::n;
   constexpr Real CS2 = Real(1) / Real(3);
-  auto at = [&](int f, int a, int s) -> Real { return A.n(f, a, s); };
+  using Mask = typename Lanes<V>::M;
+  const V zero = splat<V>(Real(0)), one = splat<V>(Real(1));
 
-  const Real T0 = A.c(F_T);
-  const Real phis = A.c(F_PHI);
-  const Real phif = Real(1) - phis;
-  const Real rho = A.c(F_RHO);
-  const Real mu = A.c(F_MU);
-  const Real fD = A.c(F_FD);
-  const Real Ts0 = A.c(F_TS);
-  Real Y0[KK];
-#pragma unroll
-  for (int k = 0; k < K; ++k) Y0[k] = A.c(F_Y0 + k);
-  const Real invMw = mixture_invMw(P, Y0);
-  const Real cp = mixture_cp(P, Y0);
-  const Real lam = mu * cp * P.inv_Pr;
-  const Real Kd = P.Au_eta2 * mu * phif * phis * phis;
-  const Real invT = fdiv(Real(1), T0);
+  const V T0 = A.c(F_T), phis = A.c(F_PHI), rho = A.c(F_RHO), mu = A.c(F_MU);
+  const V phif = vsub(one, phis);
+  const V Kd = vmul(vmul(vmuls<V>(P.Au_eta2, mu), phif), vmul(phis, phis));
 
-  // cells on a non-periodic face (their pull takes the boundary rules)
-  bool edge = (xyz[0] == 0 && P.bc[0] != BC_PERIODIC) || (xyz[0] == P.nx - 1 && P.bc[1] != BC_PERIODIC) ||
-              (xyz[1] == 0 && P.bc[2] != BC_PERIODIC) || (xyz[1] == P.ny - 1 && P.bc[3] != BC_PERIODIC);
-  if (DIM == 3)
-    edge = edge || (xyz[2] == 0 && P.bc[4] != BC_PERIODIC) ||
-           (xyz[2] == P.nz - 1 && P.bc[5] != BC_PERIODIC);
-
-  // (a1) pull streaming, moments, implicit drag
-  Real rho_in = 0;
-  if (edge && P.bc[0] == BC_INLET) {
-    Real Yin[KK];
+  // (a1) boundary rules of the streamed populations
+  const V inv_rk = vrcp(vfmas<V>(Real(0.5), Kd, rho));
+  const int xl = q.x + (LN == 2 && q.two ? 1 : 0);  // last cell
+  const Faces e0 = faces_of<DIM>(P, q.x, q.y, q.z);
+  const Faces e1 = faces_of<DIM>(P, xl, q.y, q.z);
+  if (e0.any() || e1.any()) {
+    Real rho_in = 0;
+    if (P.bc[0] == BC_INLET) {
+      Real Yin[KK];
 #pragma unroll
-    for (int k = 0; k < K; ++k) Yin[k] = P.Y_in[k];
-    rho_in = fdiv(P0 * P.eos_cr, P.T_in * mixture_invMw(P, Yin));
-  }
-  constexpr bool FO = IsHalf<Store>::value;  // FP16 residual storage
-  Real gin[Q];
-  Real u[3] = {0, 0, 0}, uw[3] = {0, 0, 0}, mraw[3] = {0, 0, 0};
-  const bool outlet_cell = P.bc[1] == BC_OUTLET && xyz[0] == P.nx - 1;
-  const Real inv_rk = fdiv(Real(1), rho + Real(0.5) * Kd);
-  for (int pass = 0; pass < (outlet_cell ? 2 : 1); ++pass) {
-    if (Acc::has_pops && A.pv) {  // populations prefetched for this cell
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        // prefetched values are raw stored numbers (scaled residuals with FP16)
-        gin[i] = A.template pop<Store>(i, Real(L::w(i)) * P.g_inv_scale);
-        if constexpr (FO)
-          gin[i] = Codec<Store, Real>::dec(gin[i], Real(L::w(i)) * P.g_inv_scale,
-                                           first_order<DIM, Real>(A, i, 0, -L::c(i, 0), -L::c(i, 1),
-                                                                  DIM == 3 ? -L::c(i, 2) : 0));
-      }
-    } else {
-      pull<DIM>(P, S, c, xyz, rho, rho_in, uw, gin, A);
+      for (int k = 0; k < K; ++k) Yin[k] = P.Y_in[k];
+      rho_in = fdiv(P0 * P.eos_cr, vmul(P.T_in, mixture_invMw<Real, K, Real>(P, Yin)));
     }
+#pragma unroll
+    for (int l = 0; l < LN; ++l) {
+      if (l == 1 && !q.two) break;
+      const int xyz[3] = {q.x + l, q.y, q.z};
+      const Faces& e = l == 0 ? e0 : e1;
+      if (!e.any()) continue;
+      Real gl[Q], uw[3] = {0, 0, 0};
+#pragma unroll
+      for (int i = 0; i < Q; ++i) gl[i] = get_lane(gin[i], l);
+      const GlobalMom<Real> gm{S.M_in, P.N};
+      edge_rules<DIM>(P, S, q.c + l, xyz, get_lane(rho, l), rho_in, uw, gl, gm);
+      if (e.f[1] && P.bc[1] == BC_OUTLET) {
+        // the outlet rule again with the cell's own first-pass velocity
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+          Real m = 0;
+#pragma unroll
+          for (int i = 0; i < Q; ++i) {
+            if (L::c(i, a) > 0) m = vadd(m, gl[i]);
+            if (L::c(i, a) < 0) m = vsub(m, gl[i]);
+          }
+          const Real d = vfma(get_lane(Kd, l), P.u_s[a], P.Fb[a]);
+          uw[a] = vmul(vfma(Real(3), m, vmul(Real(0.5), d)), get_lane(inv_rk, l));
+        }
+        edge_rules<DIM>(P, S, q.c + l, xyz, get_lane(rho, l), rho_in, uw, gl, gm);
+      }
+#pragma unroll
+      for (int i = 0; i < Q; ++i) set_lane(gin[i], l, gl[i]);
+    }
+  }
+  // moments from the sums and differences of opposite populations
+  V sg = gin[0], mraw[3] = {zero, zero, zero}, u[3] = {zero, zero, zero};
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const int j = L::opp(i);
+    if (j < i) continue;
+    const V d = vsub(gin[i], gin[j]);
+    sg = vadd(sg, vadd(gin[i], gin[j]));
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-      Real m = 0;
-#pragma unroll
-      for (int i = 0; i < Q; ++i)
-        if (L::c(i, a) != 0) m += Real(L::c(i, a)) * gin[i];
-      mraw[a] = m;
-      u[a] = (m * Real(3) + Real(0.5) * (P.Fb[a] + Kd * P.u_s[a])) * inv_rk;
-      uw[a] = u[a];
+      if (L::c(i, a) > 0) mraw[a] = i == 1 + (DIM == 2 ? a : 2 * a) ? d : vadd(mraw[a], d);
+      if (L::c(i, a) < 0) mraw[a] = vsub(mraw[a], d);
     }
   }
-  Real sg = 0;
 #pragma unroll
-  for (int i = 0; i < Q; ++i) sg += gin[i];
-
-  // the pulled populations are needed again only by the collision: with a
-  // stash they wait in shared memory instead of 9 / 19 registers
-  if constexpr (Acc::kStash) {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) A.st[i * BLOCK + threadIdx.x] = gin[i];
+  for (int a = 0; a < DIM; ++a) {
+    const V d = vfmas<V>(P.u_s[a], Kd, splat<V>(P.Fb[a]));
+    u[a] = vmul(vfmas<V>(Real(3), mraw[a], vmuls<V>(Real(0.5), d)), inv_rk);
   }
 
-  const bool fluid_on = phif >= P.phi_min;
-  const bool solid_on = P.Ts_field ? (phis >= P.phi_min) : true;
-  Real SI = 0;
-  if (fluid_on && solid_on)
-    SI = P.mix ? P.AT_eta2 * A.c(F_KT) * phis * phis * (Ts0 - T0)  // staged phi_f lambda
-               : P.AT_eta2 * lam * phif * phis * phis * (Ts0 - T0);
+  const V Ts0 = A.c(F_TS), kc = A.c(F_KT), rf0 = A.c(F_RF);
+  V Y0[KK];
+#pragma unroll
+  for (int k = 0; k < K; ++k) Y0[k] = A.c(F_Y0 + k);
+  const V invMw = mixture_invMw<Real, K, V>(P, Y0);
+  const V cp = mixture_cp<Real, K, V>(P, Y0);
+  const V invT = vrcp(T0);
+  const Mask fluid = vge(phif, splat<V>(P.phi_min));
+  const Mask solid = vge(phis, splat<V>(P.phi_min));
+  // exchange with the solid; kappa_T = phi_f lambda
+  V SI = vmul(vmul(vmuls<V>(P.AT_eta2, kc), vmul(phis, phis)), vsub(Ts0, T0));
+  SI = vsel(fluid, SI, zero);
+  if (P.Ts_field) SI = vsel(solid, SI, zero);
 
   // (c) reaction source
-  Real om[KK], omT = 0;
+  V om[KK], omT = zero;
 #pragma unroll
-  for (int k = 0; k < KK; ++k) om[k] = 0;
+  for (int k = 0; k < KK; ++k) om[k] = zero;
   if constexpr (K > 0) {
-    if (P.chem == 1) rates(P, T0, Y0, rho, invT, om, omT);
+    if (P.chem == 1) rates<Real, K, V>(P, T0, Y0, rho, invT, om, omT);
     if (P.chem >= 2) {
       // increments of the chemistry pre-pass (implicit integrator or surrogate)
 #pragma unroll
-      for (int k = 0; k < K; ++k) om[k] = __ldg(S.src + (size_t)k * P.N + c);
-      omT = __ldg(S.src + (size_t)K * P.N + c);
+      for (int k = 0; k < K; ++k) om[k] = load_cells<V>(S.src + (size_t)k * P.N + q.c, q.even, q.two);
+      omT = load_cells<V>(S.src + (size_t)K * P.N + q.c, q.even, q.two);
     }
   }
 
-  const Real iphr = fluid_on ? fdiv(Real(1), phif * rho) : Real(0);
-  const Real rf0 = A.c(F_RF);
+  // 1 / (phi_f rho) and 1 / (phi_f rho cp), zero in frozen cells; the negated
+  // velocity of the convection terms is zero there too, so that frozen cells
+  // change nothing
+  const V irc = vsel(fluid, vrcp(vmul(vmul(phif, rho), cp)), zero);
+  const V iphr = vmul(irc, cp);
+  V un[DIM];
+  Mask up[DIM];
+#pragma unroll
+  for (int a = 0; a < DIM; ++a) {
+    un[a] = vsel(fluid, vneg(u[a]), zero);
+    up[a] = vgt(u[a], zero);
+  }
 
-  // (b) species; the face factors (phi_f rho f_D averaged over the face) are
-  // shared by every species, and the central differences of Y_k feed the
-  // enthalpy-flux cross term of the temperature equation
-  Real Yn[KK];
-  Real sYm = 0;  // sum_k (1/M_k) DY_k/Dt dt for the divergence
-  Real sx[3] = {0, 0, 0};  // sum_k cp_k D_k (Y_k(+) - Y_k(-)) per axis
-  {
-    Real fm[DIM], fp[DIM];
+  // (b) species; the face factors (phi_f rho f_D summed over the face; their
+  // 1/2 sits in D_k) are shared by every species, and the central differences
+  // of Y_k feed the enthalpy-flux cross term of the temperature equation and,
+  // weighted with 1/M_k, the divergence
+  V Yn[KK];
+  V sYm = zero;     // sum_k (1/M_k) (dY_k + u.grad Y_k)
+  V sx[DIM];        // sum_k cp_k D_k (Y_k(+) - Y_k(-)) per axis
+#pragma unroll
+  for (int a = 0; a < DIM; ++a) sx[a] = zero;
+  if constexpr (K > 0) {
+    V fm[DIM], fp[DIM], sI[DIM];
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-      fm[a] = Real(0.5) * (rf0 + at(F_RF, a, -1));
-      fp[a] = Real(0.5) * (rf0 + at(F_RF, a, +1));
-    }
-    // FP32: species in pairs with packed f32x2 arithmetic; the last one of an
-    // odd count (and every species in FP64) one at a time
-    constexpr int KP = sizeof(Real) == 4 ? (K / 2) * 2 : 0;
-    if constexpr (KP > 0) {
-      float2 sx2[3] = {splat2(0.f), splat2(0.f), splat2(0.f)}, sYm2 = splat2(0.f);
-      const float2 prf = splat2(-phif * rho), pf = splat2(phif), ip = splat2(iphr);
-#pragma unroll
-      for (int k = 0; k < KP; k += 2) {
-        const float2 y0 = make_float2(Y0[k], Y0[k + 1]);
-        float2 adv = splat2(0.f), dif = splat2(0.f), cen = splat2(0.f);
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-          const float2 dm = sub2(y0, make_float2(at(F_Y0 + k, a, -1), at(F_Y0 + k + 1, a, -1)));
-          const float2 dp = sub2(make_float2(at(F_Y0 + k, a, +1), at(F_Y0 + k + 1, a, +1)), y0);
-          adv = fma2(splat2(u[a]), u[a] > 0.f ? dm : dp, adv);
-          dif = fma2(splat2(fp[a]), dp, dif);
-          dif = fma2(splat2(-fm[a]), dm, dif);
-          const float2 sd = add2(dp, dm);
-          cen = fma2(splat2(u[a]), sd, cen);
-          sx2[a] = fma2(make_float2(P.cpD[k], P.cpD[k + 1]), sd, sx2[a]);
-        }
-        float2 dY = fma2(prf, adv, fma2(make_float2(P.Dlat[k], P.Dlat[k + 1]), dif,
-                                        mul2(pf, make_float2(om[k], om[k + 1]))));
-        dY = fluid_on ? mul2(dY, ip) : splat2(0.f);
-        const float2 yn = add2(y0, dY);
-        Yn[k] = yn.x;
-        Yn[k + 1] = yn.y;
-        // material increment: the step's increment plus u.grad Y_k (central)
-        const float2 dm2 = fluid_on ? fma2(splat2(0.5f), cen, dY) : splat2(0.f);
-        sYm2 = fma2(make_float2(P.invM[k], P.invM[k + 1]), dm2, sYm2);
-      }
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) sx[a] += sx2[a].x + sx2[a].y;
-      sYm += sYm2.x + sYm2.y;
+      fm[a] = vneg(vadd(rf0, A.n(F_RF, a, -1, rf0)));
+      fp[a] = vadd(rf0, A.n(F_RF, a, +1, rf0));
+      sI[a] = zero;
     }
 #pragma unroll
-    for (int k = KP; k < K; ++k) {
-      Real adv = 0, dif = 0, cen = 0;
+    for (int k = 0; k < K; ++k) {
+      V adv = zero, dif = zero;
 #pragma unroll
       for (int a = 0; a < DIM; ++a) {
-        const Real dm = Y0[k] - at(F_Y0 + k, a, -1), dp = at(F_Y0 + k, a, +1) - Y0[k];
-        adv += u[a] * (u[a] > Real(0) ? dm : dp);
-        dif += fp[a] * dp - fm[a] * dm;
-        cen += u[a] * (dp + dm);
-        sx[a] += P.cpD[k] * (dp + dm);
+        const V dm = vsub(Y0[k], A.n(F_Y0 + k, a, -1, Y0[k]));
+        const V dp = vsub(A.n(F_Y0 + k, a, +1, Y0[k]), Y0[k]);
+        const V sd = vadd(dp, dm);
+        adv = vfma(un[a], vsel(up[a], dm, dp), adv);
+        dif = vfma(fp[a], dp, dif);
+        dif = vfma(fm[a], dm, dif);
+        sI[a] = vfmas<V>(P.invM[k], sd, sI[a]);
+        sx[a] = vfmas<V>(P.cpD[k], sd, sx[a]);
       }
-      const Real dY = fluid_on ? (-phif * rho * adv + P.Dlat[k] * dif + phif * om[k]) * iphr
-                               : Real(0);
-      Yn[k] = Y0[k] + dY;
-      // material increment: the step's increment plus u.grad Y_k (central)
-      sYm += (fluid_on ? dY + Real(0.5) * cen : Real(0)) * P.invM[k];
+      const V dY = vfma(iphr, vfmas<V>(P.Dlat_h[k], dif, vmul(phif, om[k])), adv);
+      Yn[k] = vadd(Y0[k], dY);
+      sYm = vfmas<V>(P.invM[k], dY, sYm);
     }
+    V cen = zero;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) cen = vfma(un[a], sI[a], cen);
+    sYm = vfmas<V>(Real(-0.5), cen, sYm);
   }
 
   // (b) temperature
-  Real Tn = Ts0, dTm = Ts0 - T0;  // frozen cells take the solid temperature
-  if (fluid_on) {
-    Real adv = 0, dif = 0, cross = 0, cen = 0;
-    const Real kc = A.c(F_KT);
+  V Tn, dTm;
+  {
+    const V fD = A.c(F_FD);
+    V adv = zero, dif = zero, cross = zero, cen = zero;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-      const Real tm = at(F_T, a, -1), tp = at(F_T, a, +1);
-      adv += u[a] > Real(0) ? u[a] * (T0 - tm) : u[a] * (tp - T0);
-      cen += u[a] * (tp - tm);
-      const Real km = Real(0.5) * (kc + at(F_KT, a, -1));
-      const Real kp = Real(0.5) * (kc + at(F_KT, a, +1));
-      dif += kp * (tp - T0) - km * (T0 - tm);
-      if constexpr (K > 0) cross += Real(0.25) * fD * sx[a] * (tp - tm);
+      const V dm = vsub(T0, A.n(F_T, a, -1, T0)), dp = vsub(A.n(F_T, a, +1, T0), T0);
+      const V sd = vadd(dp, dm);
+      adv = vfma(un[a], vsel(up[a], dm, dp), adv);
+      cen = vfma(un[a], sd, cen);
+      dif = vfma(vadd(kc, A.n(F_KT, a, +1, kc)), dp, dif);
+      dif = vfma(vneg(vadd(kc, A.n(F_KT, a, -1, kc))), dm, dif);
+      if constexpr (K > 0) cross = vfma(sx[a], sd, cross);
     }
-    const Real rhs = -phif * rho * cp * adv + dif + phif * (rho * cross + dP0r + omT + SI);
-    const Real dTn = rhs * iphr * fdiv(Real(1), cp);
-    Tn = T0 + dTn;
-    dTm = dTn + Real(0.5) * cen;  // plus u.grad T (central)
+    V src = vadd(vadds<V>(dP0r, omT), SI);
+    if constexpr (K > 0) src = vfma(vmul(rho, fD), vmuls<V>(Real(0.25), cross), src);
+    const V dTn = vfma(irc, vfmas<V>(Real(0.5), dif, vmul(phif, src)), adv);
+    // frozen cells take the solid temperature
+    Tn = vsel(fluid, vadd(T0, dTn), Ts0);
+    dTm = vsel(fluid, vfmas<V>(Real(-0.5), cen, dTn), vsub(Ts0, T0));  // plus u.grad T (central)
   }
 
   // solid temperature
   if (P.Ts_field) {
-    Real Tsn = Ts0;
-    if (phis >= P.phi_min) {
-      Real dif = 0;
+    V Tsn = Ts0;
+    if (vany(solid)) {
+      V dif = zero;
 #pragma unroll
       for (int a = 0; a < DIM; ++a) {
-        const Real km = Real(0.5) * (phis + at(F_PHI, a, -1)) * P.Lams;
-        const Real kp = Real(0.5) * (phis + at(F_PHI, a, +1)) * P.Lams;
-        dif += kp * (at(F_TS, a, +1) - Ts0) - km * (Ts0 - at(F_TS, a, -1));
+        const V sm = vsub(Ts0, A.n(F_TS, a, -1, Ts0)), sp = vsub(A.n(F_TS, a, +1, Ts0), Ts0);
+        dif = vfma(vadd(phis, A.n(F_PHI, a, +1, phis)), sp, dif);
+        dif = vfma(vneg(vadd(phis, A.n(F_PHI, a, -1, phis))), sm, dif);
       }
-      Tsn = Ts0 + fdiv(dif - phif * SI, phis * P.Cs);
+      const V num = vfma(vneg(phif), SI, vmuls<V>(P.Lams_h, dif));
+      V dTs = fdiv(num, vmuls<V>(P.Cs, phis));
       if (P.moving) {
         // a moving solid carries its temperature with u_s (upwind)
-        Real advs = 0;
 #pragma unroll
         for (int a = 0; a < DIM; ++a) {
           const Real us = P.u_s[a];
-          if (us > Real(0)) advs += us * (Ts0 - at(F_TS, a, -1));
-          else if (us < Real(0)) advs += us * (at(F_TS, a, +1) - Ts0);
+          if (us > Real(0)) dTs = vfmas<V>(-us, vsub(Ts0, A.n(F_TS, a, -1, Ts0)), dTs);
+          else if (us < Real(0)) dTs = vfmas<V>(-us, vsub(A.n(F_TS, a, +1, Ts0), Ts0), dTs);
         }
-        Tsn -= advs;
       }
+      Tsn = vsel(solid, vadd(Ts0, dTs), Ts0);
     }
-    S.Ts_out[c] = Tsn;
+    store_cells(S.Ts_out + q.c, Tsn, q.even, q.two);
   }
 
   // low-Mach divergence: continuity with the EOS at uniform P0,
@@ -1588,251 +1730,195 @@ __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const Stat
   // increments taken as the step's increments plus u.grad with central
   // differences, the gradient the source takes of rho (with the upwind
   // gradient the discrete continuity would keep a first-order mass defect)
-  Real D = dTm * invT;
-  if constexpr (K > 0) D += fdiv(sYm, invMw);
-  D -= dlnP0;
+  V D = vfma(dTm, invT, splat<V>(-dlnP0));
+  if constexpr (K > 0) D = vadd(D, fdiv(sYm, invMw));
 
   // (a) source and BGK collision: omega = 1/tau = 2 rho / (rho + 6 mu)
-  Real G[3] = {0, 0, 0}, F[3] = {0, 0, 0};
+  V G[DIM], F[DIM];
+  V uG = zero;
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {
-    G[a] = CS2 * Real(0.5) * (at(F_RHO, a, +1) - at(F_RHO, a, -1));
-    F[a] = P.Fb[a] - Kd * (u[a] - P.u_s[a]);
+    G[a] = vmuls<V>(CS2 * Real(0.5), vsub(A.n(F_RHO, a, +1, rho), A.n(F_RHO, a, -1, rho)));
+    F[a] = vfma(vneg(Kd), vadds<V>(-P.u_s[a], u[a]), splat<V>(P.Fb[a]));
+    uG = vfma(u[a], G[a], uG);
   }
   // P_h: the pulled zeroth moment plus half the zeroth moment of the source,
   // sum_i Xi_i = u.G + rho cs^2 D, so that a step adds the whole source
-  Real uG = 0;
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) uG += u[a] * G[a];
-  const Real Ph = sg + Real(0.5) * (rho * CS2 * D + uG);
-  if (P.nscbc && xyz[0] >= P.nx - 2) {
+  const V rho3 = vmuls<V>(CS2, rho);
+  const V Ph = vfmas<V>(Real(0.5), vfma(rho3, D, uG), sg);
+  if (P.nscbc && xl >= P.nx - 2) {
     // the two outlet columns of this step for the characteristic outlet
-    const int NF = P.ny * P.nz, f = xyz[1] + P.ny * xyz[2];
-    const int col = xyz[0] == P.nx - 1 ? 0 : 1;
-    S.ob[(size_t)(2 * col) * NF + f] = Ph;
-    S.ob[(size_t)(2 * col + 1) * NF + f] = u[0];
-    if (col == 0) S.ob[(size_t)4 * NF + f] = rho;
+    const int NF = P.ny * P.nz, f = q.y + P.ny * q.z;
+#pragma unroll
+    for (int l = 0; l < LN; ++l) {
+      if (l == 1 && !q.two) break;
+      if (q.x + l < P.nx - 2) continue;
+      const int col = q.x + l == P.nx - 1 ? 0 : 1;
+      S.ob[(size_t)(2 * col) * NF + f] = get_lane(Ph, l);
+      S.ob[(size_t)(2 * col + 1) * NF + f] = get_lane(u[0], l);
+      if (col == 0) S.ob[(size_t)4 * NF + f] = get_lane(rho, l);
+    }
   }
-  const Real omega = fdiv(Real(2) * rho, rho + Real(6) * mu);
-  const Real src_w = Real(1) - Real(0.5) * omega;
+  const V omega = fdiv(vmuls<V>(Real(2), rho), vfmas<V>(Real(6), mu, rho));
+  const V src_w = vfmas<V>(Real(-0.5), omega, one);
+  const V keep = vsub(one, omega);
   // f_eq / rho - w = w e with e = 3 cu + 9/2 cu^2 - 3/2 uu;
   // g_eq = cs2 f_eq + w (P_h - rho cs2) = w (P_h + rho e / 3);
   // Xi = w [(c - u).(G e + F (1 + e)) + rho cs2 D] = w [(c.H - u.H) e + c.F - u.F + rho cs2 D]
-  // with H = G + F.  Collected per cell: g* = (1 - omega) g + w [A0 + B e + src_w x],
-  // A0 = omega P_h + src_w rho cs2 D, B = omega rho cs2, x = (c.H - u.H) e + c.F - u.F.
-  Real H[3] = {0, 0, 0};
-  Real uu = 0, uH = 0, uF = 0;
+  // with H = G + F.  Split into the parts even and odd in c, e = E + O:
+  //   g* = keep g + w (te + to),  O = 3 cu,  E = O^2 / 2 - 3/2 uu,
+  //   te = A0 + B E + c.Hs O,  to = B O + c.Hs E + c.Fs,
+  // with s = 1 - omega / 2, Hs = s H, Fs = s F, B = omega rho cs2 - s u.H and
+  // A0 = omega P_h + s (rho cs2 D - u.F); a direction and its opposite share
+  // te and to.
+  V u3[DIM], Hs[DIM], Fs[DIM];
+  V uu = zero, uHs = zero, uFs = zero;
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {
-    H[a] = G[a] + F[a];
-    uu += u[a] * u[a];
-    uH += u[a] * H[a];
-    uF += u[a] * F[a];
+    Fs[a] = vmul(src_w, F[a]);
+    Hs[a] = vfma(src_w, G[a], Fs[a]);
+    u3[a] = vmuls<V>(Real(3), u[a]);
+    uu = vfma(u[a], u[a], uu);
+    uHs = vfma(u[a], Hs[a], uHs);
+    uFs = vfma(u[a], Fs[a], uFs);
   }
-  const Real rho3 = rho * CS2;
-  const Real A0 = omega * Ph + src_w * (rho3 * D);
-  const Real B = omega * rho3;
-  const Real uu15 = Real(1.5) * uu;
-  const Real keep = Real(1) - omega;
-  // FP16 storage: the post-collision moments of this cell in closed form
-  // (sum_i w_i e_i = 0, sum_i w_i x_i = u.G, sum_i w_i c_i e_i = u,
-  // sum_i w_i c_i x_i = F / 3 on the isotropic lattice); any values would do,
-  // since readers add back exactly what is subtracted here, but these leave
-  // a residual of second order in u
-  Real Pst = 0, jst[3] = {0, 0, 0};
-  if constexpr (FO) {
-    Pst = keep * sg + A0 + src_w * (uH - uF);
+  const V uu15 = vmuls<V>(Real(-1.5), uu);
+  const V or3 = vmul(omega, rho3);
+  const V B = vsub(or3, uHs);
+  V A0 = vfma(omega, Ph, vmul(src_w, vmul(rho3, D)));
+  A0 = vsub(A0, uFs);
+  gin[0] = vfma(keep, gin[0], vmuls<V>(Real(L::w(0)), vfma(uu15, B, A0)));
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) jst[a] = keep * mraw[a] + B * u[a] + src_w * CS2 * F[a];
-  }
-  // FP32 updates a direction and its opposite together with packed f32x2
-  // arithmetic (c.u, c.H, c.F of the opposite are the negated ones); the rest
-  // direction, and every direction in FP64, one at a time
-  constexpr bool PAIRS = sizeof(Real) == 4;
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    if constexpr (PAIRS) {
-      if (L::opp(i) < i) continue;  // done with its opposite
-    }
-    Real cu = 0, cH = 0, cF = 0, cj = 0;
+  for (int i = 1; i < Q; ++i) {
+    const int j = L::opp(i);
+    if (j < i) continue;  // done with its opposite
+    V O = zero, cH = zero, cF = zero;
+    bool first = true;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-      if (L::c(i, a) > 0) { cu += u[a]; cH += H[a]; cF += F[a]; cj += jst[a]; }
-      if (L::c(i, a) < 0) { cu -= u[a]; cH -= H[a]; cF -= F[a]; cj -= jst[a]; }
-    }
-    Real gi = gin[i];
-    if constexpr (Acc::kStash) gi = A.st[i * BLOCK + threadIdx.x];
-    if constexpr (PAIRS) {
-      if (i > 0) {
-        const int j = L::opp(i);
-        Real gj = gin[j];
-        if constexpr (Acc::kStash) gj = A.st[j * BLOCK + threadIdx.x];
-        const float2 cu2 = make_float2(cu, -cu);
-        const float2 e = fma2(cu2, fma2(cu2, splat2(4.5f), splat2(3.f)), splat2(-uu15));
-        const float2 x = fma2(sub2(make_float2(cH, -cH), splat2(uH)), e,
-                              sub2(make_float2(cF, -cF), splat2(uF)));
-        float2 t = fma2(splat2(B), e, splat2(A0));
-        t = fma2(splat2(src_w), x, t);
-        const float w = float(L::w(i));
-        float2 g = fma2(splat2(keep), make_float2(gi, gj), mul2(splat2(w), t));
-        if constexpr (FO)
-          g = sub2(g, mul2(splat2(w), fma2(splat2(3.f), make_float2(cj, -cj), splat2(Pst))));
-        Codec<Store, Real>::store(S.g_out + (size_t)i * P.N + c, g.x,
-                                  P.g_scale * Real(1.0 / L::w(i)));
-        Codec<Store, Real>::store(S.g_out + (size_t)j * P.N + c, g.y,
-                                  P.g_scale * Real(1.0 / L::w(j)));
-        continue;
+      if (L::c(i, a) == 0) continue;
+      if (first) {  // the first direction of a pair starts with +1
+        O = u3[a];
+        cH = Hs[a];
+        cF = Fs[a];
+        if (L::c(i, a) < 0) { O = vneg(O); cH = vneg(cH); cF = vneg(cF); }
+        first = false;
+      } else if (L::c(i, a) > 0) {
+        O = vadd(O, u3[a]);
+        cH = vadd(cH, Hs[a]);
+        cF = vadd(cF, Fs[a]);
+      } else {
+        O = vsub(O, u3[a]);
+        cH = vsub(cH, Hs[a]);
+        cF = vsub(cF, Fs[a]);
       }
     }
-    const Real w = Real(L::w(i));
-    const Real e = cu * (Real(3) + Real(4.5) * cu) - uu15;
-    const Real x = (cH - uH) * e + (cF - uF);
-    Real g = keep * gi + w * (A0 + B * e + src_w * x);
-    if constexpr (FO) g -= w * (Pst + Real(3) * cj);
-    Codec<Store, Real>::store(S.g_out + (size_t)i * P.N + c, g, P.g_scale * Real(1.0 / L::w(i)));
+    const V E = vfma(vmuls<V>(Real(0.5), O), O, uu15);
+    const V te = vfma(E, B, vfma(cH, O, A0));
+    const V to = vfma(O, B, vfma(cH, E, cF));
+    const V p = vmuls<V>(Real(L::w(i)), te);
+    const V gi = vfma(keep, gin[i], vfmas<V>(Real(L::w(i)), to, p));
+    const V gj = vfma(keep, gin[j], vfmas<V>(Real(-L::w(i)), to, p));
+    gin[i] = gi;
+    gin[j] = gj;
   }
-  if constexpr (FO) {
-    S.M_out[c] = Pst;
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) S.M_out[(size_t)(1 + a) * P.N + c] = jst[a];
-  }
-
-  S.T_out[c] = Tn;
+  for (int i = 0; i < Q; ++i)
+    store_cells(S.g_out + (size_t)i * P.N + q.c, gin[i], q.even, q.two);
+  store_cells(S.T_out + q.c, Tn, q.even, q.two);
 #pragma unroll
-  for (int k = 0; k < K; ++k) S.Y_out[(size_t)k * P.N + c] = Yn[k];
+  for (int k = 0; k < K; ++k) store_cells(S.Y_out + (size_t)k * P.N + q.c, Yn[k], q.even, q.two);
 
   // (d) contributions to the reduction
-  const Real fx = phif * rho * u[0];
-  fin = (xyz[0] == 0 && P.bc[0] == BC_INLET) ? fx : Real(0);
-  fout = outlet_cell ? fx : Real(0);
+  fin = fout = Real(0);
+  if (q.x == 0 && P.bc[0] == BC_INLET)
+    fin = get_lane(phif, 0) * get_lane(rho, 0) * get_lane(u[0], 0);
+  if (xl == P.nx - 1 && P.bc[1] == BC_OUTLET) {
+    const int l = LN == 2 && q.two ? 1 : 0;
+    fout = get_lane(phif, l) * get_lane(rho, l) * get_lane(u[0], l);
+  }
   // 0 * P_h is NaN when any pulled population is: a NaN confined to the
   // populations reaches the FP64 reduction (and the status word) this step
-  return phif * fdiv(Real(1), Tn * mixture_invMw(P, Yn)) + Real(0) * Ph;
+  V r = vfma(zero, Ph, vmul(phif, vrcp(vmul(Tn, mixture_invMw<Real, K, V>(P, Yn)))));
+  if (LN == 2 && !q.two) set_lane(r, 1, Real(0));
+  return r;
 }
 
-// Resident blocks per SM requested from the register allocator: 2-D FP32 /
-// FP16 storage at <= 64 registers (4 blocks), 3-D FP32 at <= 80 (3 blocks),
-// 3-D FP16 storage, whose decode holds the source cells' moments, at <= 128
-// (2 blocks); FP64 is bound by the FP64 pipe and keeps the registers it needs.
-template <int DIM, class Real, class Store> struct MinBlocks {
-  static constexpr int value =
-      sizeof(Real) == 8 ? (DIM == 3 ? 1 : 2) : (DIM == 2 ? 4 : (IsHalf<Store>::value ? 2 : 3));
+// Resident threads per SM asked of the register allocator in 2-D.  FP32 pairs
+// wait on latency, so more resident blocks pay until they spill: without
+// species 64 registers (1024 threads; 48 beds: 359 us a step at 512 threads,
+// 288 at 1024), with species 128 (512 threads; the 1024 x 256 bed: 15.5 us, 16.6
+// at 640, 17.6 at 768).  FP64 is bound by the FP64 pipe: 128 registers.
+template <int K, class T_> struct MinBlocks {
+  static constexpr int value = (T_::LN == 2 && K == 0 ? 1024 : 512) / T_::NT;
 };
 
-// One tile of the fused step (tile (bx, by) of the xy grid, z-chunk bz in
-// 3-D): stages the tile's planes in `planes` (shared memory), updates its
-// cells and returns the block sums of the reduction in thread 0 (I, inlet
-// flux, outlet flux).  Every thread of the block calls it.
-template <int DIM, int K, class Real, class Store, class T_ = Tile<DIM>>
-__device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<Real, Store>& S,
-                                          int bx, int by, int bz,
-                                          Plane<Real, K, T_::HP, n_mom<DIM, Store>()>* planes,
-                                          double* red_sh,
-                                          double& sI, double& sIn, double& sOut) {
+// One 2-D tile of the fused step (tile (bx, by)): stages the tile in `pl`
+// (shared memory), updates its cells and returns the block sums of the
+// reduction in thread 0 (I, inlet flux, outlet flux).  Every thread of the
+// block calls it.  The population loads of the thread's cells are issued
+// before the staging, so the two load phases overlap.
+template <int K, class Real, class T_>
+__device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<Real, Real>& S,
+                                          int bx, int by, Real* pl, double* red_sh, double& sI,
+                                          double& sIn, double& sOut) {
+  using V = typename T_::V;
+  constexpr int Q = Lattice<2>::Q, LN = T_::LN, RPT = T_::RPT, RS = T_::TY / RPT;
   const Real P0 = scal_P0<Real>(S.scal);
   const Real dlnP0 = scal_dlnP0<Real>(S.scal);
   const Real dP0r = scal_dP0r<Real>(S.scal);
-
-  const int tx = threadIdx.x % T_::TX, ty = threadIdx.x / T_::TX;
+  const int tx = (threadIdx.x % T_::TXT) * LN, ty = threadIdx.x / T_::TXT;
   const int x0 = bx * T_::TX, y0 = by * T_::TY;
-  const int x = x0 + tx, y = y0 + ty;
-  const int h = (ty + 1) * T_::HX + (tx + 1);
-  const bool in_xy = x < P.nx && y < P.ny;
-  const int z_begin = bz * T_::ZC;
-  const int z_end = DIM == 3 ? min(z_begin + T_::ZC, P.nz) : 1;
+  const int x = x0 + tx;
   const bool flux_block = (x0 == 0 && P.bc[0] == BC_INLET) ||
                           (x0 + T_::TX >= P.nx && P.bc[1] == BC_OUTLET);
-
-  Real accI = 0, accIn = 0, accOut = 0;
-  if constexpr (DIM == 2) {
-    using L = Lattice<2>;
-    constexpr int RPT = T_::RPT;
-    constexpr int RS = T_::TY / RPT;  // row stride between a thread's cells
-    // population loads of the thread's interior cells, issued before staging
-    Real pre[RPT][L::Q];
-    bool pv[RPT];
+  const bool even = LN == 1 || S.even;
+  V accI = splat<V>(Real(0));
+  Real accIn = 0, accOut = 0;
+  V g[RPT][Q];
 #pragma unroll
-    for (int r = 0; r < RPT; ++r) pv[r] = false;
-    if constexpr (T_::PREFETCH) {
+  for (int r = 0; r < RPT; ++r)
+    if (x < P.nx && y0 + ty + r * RS < P.ny)
+      load_pops<2, K, Real, V>(P, S, x, y0 + ty + r * RS, 0, g[r]);
+  stage_plane<2, K, Real, T_>(P, S, pl, x0, y0, 0, P0);
+  __syncthreads();
 #pragma unroll
-      for (int r = 0; r < RPT; ++r) {
-        const int yr = y0 + ty + r * RS;
-        const bool inner = x > 0 && x < P.nx - 1 && yr > 0 && yr < P.ny - 1;
-        pv[r] = inner;
-        if (inner) {
-          const int c = x + P.nx * yr;
-#pragma unroll
-          for (int i = 0; i < L::Q; ++i)
-            pre[r][i] = Codec<Store, Real>::raw(
-                S.g_in + (size_t)i * P.N + c - L::c(i, 0) - L::c(i, 1) * P.nx);
-        }
-      }
-    }
-    stage_plane<DIM, Real, Store, K, T_::HP, T_>(P, S, planes[0], x0, y0, 0, P0);
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < RPT; ++r) {
-      const int yr = y0 + ty + r * RS;
-      if (x < P.nx && yr < P.ny) {
-        const int c = x + P.nx * yr;
-        const int xyz[3] = {x, yr, 0};
-        const int hr = (ty + r * RS + 1) * T_::HX + (tx + 1);
-        Real fi, fo;
-        const PlaneAcc<DIM, Real, T_::PREFETCH, T_, F_Y0 + K> A{&planes[0].f[0][0], nullptr,
-                                                                nullptr, hr, pre[r], pv[r],
-                                                                nullptr};
-        accI += cell_update<DIM, K, Real, Store>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
-        accIn += fi;
-        accOut += fo;
-      }
-    }
-  } else {
-    // ring of three staged planes: slot (z mod 3)
-    stage_plane<DIM, Real, Store, K, T_::HP, T_>(P, S, planes[(z_begin + 2) % 3], x0, y0,
-                                                 z_begin - 1, P0);
-    stage_plane<DIM, Real, Store, K, T_::HP, T_>(P, S, planes[z_begin % 3], x0, y0, z_begin, P0);
-    for (int z = z_begin; z < z_end; ++z) {
-      stage_plane<DIM, Real, Store, K, T_::HP, T_>(P, S, planes[(z + 1) % 3], x0, y0, z + 1, P0);
-      __syncthreads();
-      if (in_xy) {
-        const int c = x + P.nx * (y + P.ny * z);
-        const int xyz[3] = {x, y, z};
-        Real fi, fo;
-        const PlaneAcc<DIM, Real, false, T_, F_Y0 + K, true> A{
-            &planes[z % 3].f[0][0], &planes[(z + 2) % 3].f[0][0],
-            &planes[(z + 1) % 3].f[0][0], h, nullptr, false,
-            reinterpret_cast<Real*>(planes + T_::NPL)};
-        accI += cell_update<DIM, K, Real, Store>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
-        accIn += fi;
-        accOut += fo;
-      }
-      __syncthreads();
+  for (int r = 0; r < RPT; ++r) {
+    const int yr = y0 + ty + r * RS;
+    if (x < P.nx && yr < P.ny) {
+      const CellPos q{x + P.nx * yr, x, yr, 0, even, x + 1 < P.nx};
+      const PlaneAcc<Real, T_> A{pl, nullptr, nullptr,
+                                 (ty + r * RS + 1) * T_::HX + tx + T_::XO};
+      Real fi, fo;
+      accI = vadd(accI, cell_update<2, K, Real, V>(P, S, A, g[r], q, P0, dlnP0, dP0r, fi, fo));
+      accIn += fi;
+      accOut += fo;
     }
   }
-
   // (d) block partials in FP64 (one barrier)
-  block_sum3<Real>(accI, accIn, accOut, flux_block, red_sh, sI, sIn, sOut);
+  block_sum3(accI, accIn, accOut, flux_block, red_sh, sI, sIn, sOut);
 }
 
-template <int DIM, int K, class Real, class Store>
-__global__ void __launch_bounds__(BLOCK, MinBlocks<DIM, Real, Store>::value)
-step_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
+template <int DIM, int K, class Real, class T_>
+constexpr size_t step_smem_bytes() {
+  return sizeof(Real) * (F_Y0 + K) * T_::HP * (DIM == 3 ? 3 : 1);
+}
+
+template <int K, class Real, class T_>
+__global__ void __launch_bounds__(T_::NT, (MinBlocks<K, T_>::value))
+step_kernel(const __grid_constant__ Params<Real, K> P, const State<Real, Real> S, int p0_closed,
             const double* __restrict__ prev_partials, unsigned prev_nb) {
-  using T_ = Tile<DIM>;
-  using PL = Plane<Real, K, T_::HP, n_mom<DIM, Store>()>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PL* planes = reinterpret_cast<PL*>(smem_raw);
+  Real* pl = reinterpret_cast<Real*>(smem_raw);
   __shared__ double red_sh[96];
 
   // deferred combine of the previous step's partials (fixed P0 only): block
   // 0's first warp does it while the other blocks start on their cells
-  if (prev_partials && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 &&
-      threadIdx.x < 32)
+  if (prev_partials && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32)
     combine_partials(prev_partials, prev_nb, S.scal, 0, false, 0.0, P.eos_c, P.inv_rho_ref);
 
   double sI, sIn, sOut;
-  step_tile<DIM, K, Real, Store, T_>(P, S, blockIdx.x, blockIdx.y, blockIdx.z, planes, red_sh,
-                                     sI, sIn, sOut);
+  step_tile<K, Real, T_>(P, S, blockIdx.x, blockIdx.y, pl, red_sh, sI, sIn, sOut);
   // deterministic finish by the last block (closed P0) or deferred
   publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
                    P.inv_rho_ref);
@@ -1843,15 +1929,13 @@ step_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
 // clears the other one for the next step), so no block waits for a second
 // wave and cheap tiles do not leave SMs idle.  Reduction slots are the tile
 // indices, as in step_kernel.
-template <int DIM, int K, class Real, class Store, class T_>
-__global__ void __launch_bounds__(BLOCK, (sizeof(Real) == 8 ? 2 : (T_::RPT > 1 ? 3 : 4)))
-step_persistent_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
-                       const double* __restrict__ prev_partials, unsigned prev_nb,
+template <int K, class Real, class T_>
+__global__ void __launch_bounds__(T_::NT, (MinBlocks<K, T_>::value))
+step_persistent_kernel(const __grid_constant__ Params<Real, K> P, const State<Real, Real> S,
+                       int p0_closed, const double* __restrict__ prev_partials, unsigned prev_nb,
                        unsigned* __restrict__ tile_ctr, int parity) {
-  static_assert(DIM == 2, "the persistent step walks 2-D tiles");
-  using PL = Plane<Real, K, T_::HP, n_mom<DIM, Store>()>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PL* planes = reinterpret_cast<PL*>(smem_raw);
+  Real* pl = reinterpret_cast<Real*>(smem_raw);
   __shared__ double red_sh[96];
   __shared__ int next_sh[2];
 
@@ -1872,18 +1956,10 @@ step_persistent_kernel(const Params<Real, K> P, const State<Real, Store> S, int 
     par ^= 1;
     if (threadIdx.x == 0) next_sh[par] = (int)atomicAdd(ctr, 1u);
     double sI, sIn, sOut;
-    step_tile<DIM, K, Real, Store, T_>(P, S, t % nbx, t / nbx, 0, planes, red_sh, sI, sIn,
-                                       sOut);
+    step_tile<K, Real, T_>(P, S, t % nbx, t / nbx, pl, red_sh, sI, sIn, sOut);
     publish_partials_at(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0,
                         P.eos_c, P.inv_rho_ref, (unsigned)t, (unsigned)total, p0_closed != 0);
   }
-}
-
-// staged planes, and in 3-D the stash of the pulled populations
-template <int DIM, int K, class Real, class Store, class T_ = Tile<DIM>>
-constexpr size_t step_smem_bytes() {
-  return sizeof(Plane<Real, K, T_::HP, n_mom<DIM, Store>()>) * T_::NPL +
-         (DIM == 3 ? sizeof(Real) * Lattice<DIM>::Q * BLOCK : 0);
 }
 
 // ------------------------------------------- chemistry pre-pass (implicit)

@@ -14,6 +14,7 @@
 #include "../../include/pflb.h"
 #include "pflb_batch.cuh"
 #include "pflb_chem.cuh"
+#include "pflb_half.cuh"
 #include "pflb_step3d.cuh"
 #include "pflb_kernels.cuh"
 #include "pflb_surrogate.cuh"
@@ -100,7 +101,7 @@ struct Launcher {
   // FP32 compute with 16-byte rows), 2 / 3 = persistent staged tiles 32 x 8 /
   // 32 x 16 (2-D); returns false if not available here
   virtual bool select_kernel(int k, const Buffers& B, int cur) = 0;
-  virtual int kernel() const = 0;
+  virtual int kernel() = 0;
   // learned chemistry (six-species mechanism only)
   virtual bool set_surrogate(const SurrArgs& a) = 0;
   // chemistry pre-pass of the current state into B.src; increments (dY, dT)
@@ -170,6 +171,7 @@ Params<Real, K> make_params(const pflb_domain_desc& d, const pflb_mechanism& m, 
     P.cp[k] = Real(m.cp[k]);
     P.hf[k] = Real(m.hf[k]);
     P.Dlat[k] = Real(m.Dref[k] * h2);
+    P.Dlat_h[k] = Real(0.5) * P.Dlat[k];
     P.cpD[k] = Real(m.cp[k] * m.Dref[k] * h2);
     P.rho_ref_M[k] = Real(d.rho_ref / m.M[k]);
   }
@@ -180,6 +182,7 @@ Params<Real, K> make_params(const pflb_domain_desc& d, const pflb_mechanism& m, 
   P.Ts_uniform = Real(d.Ts_uniform);
   P.Cs = Real(d.rhocp_s / d.rho_ref);
   P.Lams = Real(d.lambda_s * h2 / d.rho_ref);
+  P.Lams_h = Real(0.5) * P.Lams;
   P.phi_min = Real(d.phi_min);
   P.chem = K > 0 ? m.chem_mode : 0;
   P.J = K > 0 ? m.J : 0;
@@ -342,16 +345,61 @@ struct LauncherImpl final : Launcher {
     S.partials = B.partials + (size_t)4 * B.slots * cur;
     S.counter = B.counter;
     S.ob = static_cast<Real*>(B.ob);
+    // a pair of x-neighbours is one aligned word of every array the step
+    // touches (a caller's own arrays may start anywhere)
+    const uintptr_t bits =
+        reinterpret_cast<uintptr_t>(S.g_in) | reinterpret_cast<uintptr_t>(S.g_out) |
+        reinterpret_cast<uintptr_t>(S.T_in) | reinterpret_cast<uintptr_t>(S.T_out) |
+        reinterpret_cast<uintptr_t>(S.Y_in) | reinterpret_cast<uintptr_t>(S.Y_out) |
+        reinterpret_cast<uintptr_t>(S.Ts_in) | reinterpret_cast<uintptr_t>(S.Ts_out) |
+        reinterpret_cast<uintptr_t>(S.phi) | reinterpret_cast<uintptr_t>(S.src);
+    S.even = (P.nx % 2 == 0 && bits % (2 * sizeof(Real)) == 0) ? 1 : 0;
     return S;
   }
   int blocks() const { return (P.N + BLOCK - 1) / BLOCK; }
-  // tile grid of the fused step (32 x 8 tiles; 3-D blocks march 16 planes)
-  dim3 step_grid() const {
-    using T_ = Tile<DIM>;
-    return dim3((P.nx + T_::TX - 1) / T_::TX, (P.ny + T_::TY - 1) / T_::TY,
-                DIM == 3 ? (P.nz + T_::ZC - 1) / T_::ZC : 1);
+  // tiles of the staged step: 32 x step_ty() cells; in 3-D a block takes a run of
+  // at most kChunk planes
+  using V = typename VecOf<Real>::V;
+  static constexpr bool kHalf = MODE == MODE_FP16;
+  static constexpr int kChunk = kHalf ? 16 : 32;
+  using HalfTile = half_store::Tile<DIM>;
+  dim3 step_grid() {
+    const unsigned gx = (P.nx + 31) / 32, gy = (P.ny + step_ty() - 1) / step_ty();
+    if (DIM == 3 && kHalf) return dim3(gx, gy, (P.nz + kChunk - 1) / kChunk);
+    return DIM == 3 ? dim3(gx * gy * chunks_per_tile(P.nz, kChunk)) : dim3(gx, gy);
   }
-  long long step_blocks() const {
+  int sm_count() {
+    if (sms == 0) {
+      int dev = 0;
+      if (cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 1;
+    }
+    return sms;
+  }
+  int sms = 0;
+  // Rows of the staged 2-D tile.  FP64 is bound by the FP64 pipe of the busiest
+  // SM: the height whose tiles spread best, counting an SM's tiles times the
+  // pipe work of one (a staged cell costs about a quarter of an update).  A
+  // 128 x 64 channel has 32 tiles of 8 rows, on as many SMs, or 128 of 2 rows.
+  int ty_cached = 0;
+  int step_ty() {
+    if (DIM == 3 || sizeof(Real) == 4) return 8;
+    if (ty_cached == 0) {
+      double best = 0;
+      for (int ty = 8; ty >= 2; ty /= 2) {
+        const long long tiles = (long long)((P.nx + 31) / 32) * ((P.ny + ty - 1) / ty);
+        const double cost =
+            double((tiles + sm_count() - 1) / sm_count()) * (32 * ty + 0.25 * 34 * (ty + 2));
+        if (ty_cached == 0 || cost < best) {
+          best = cost;
+          ty_cached = ty;
+        }
+      }
+    }
+    return ty_cached;
+  }
+  long long step_blocks() {
     dim3 g = step_grid();
     return (long long)g.x * g.y * g.z;
   }
@@ -404,9 +452,16 @@ struct LauncherImpl final : Launcher {
   const void* map_key[2][5] = {};
   int tma_state = 0;  // 0 unknown, 1 usable, -1 not usable
   int tma_grid = 0;
-  // default step kernel: the z-march for 3-D FP32 storage (fastest measured on
-  // the 3-D bed), the staged-tile kernel otherwise
-  int kernel_sel = (DIM == 3 && MODE == MODE_FP32) ? 4 : 0;
+  // step kernel; -1: the default, the staged tiles, but equal runs of the z-march
+  // for 3-D domains of less than 16 planes a resident block, where the shrinking
+  // runs of the tiled schedule cannot even out (64^3 FP64: 508 us against 1100)
+  int kernel_sel = -1;
+  int resolved() {
+    if (kernel_sel >= 0) return kernel_sel;
+    if (DIM == 2 || kHalf) return 0;
+    const long long planes = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8) * P.nz;
+    return planes < 16LL * sm_count() * (sizeof(Real) == 8 ? 1 : 3) ? 4 : 0;
+  }
   long long wait_limit = kDefaultWaitCycles;
   void set_wait_limit(long long cycles) override { wait_limit = cycles; }
   SurrArgs surr;
@@ -449,64 +504,120 @@ struct LauncherImpl final : Launcher {
     return false;
   }
 
-  // persistent z-march (3-D): grid = resident blocks per SM x SMs
+  // the grid of resident blocks of a kernel (cached in `grid`, at most `most`)
+  template <class Kern>
+  static cudaError_t resident_grid(Kern kern, int threads, size_t smem, int& grid,
+                                   long long most = 1LL << 30) {
+    if (grid != 0) return cudaSuccess;
+    int dev = 0, sms = 0, occ = 0;
+    cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
+    if (e == cudaSuccess) grid = (int)std::min<long long>((long long)std::max(1, occ) * sms, most);
+    return e;
+  }
+
+  // 3-D step: the persistent z-march (grid = resident blocks per SM x SMs) or,
+  // with chunked = true, one block per tile and kChunk planes
   int mgrid[2] = {0, 0};
   template <bool PRE>
-  cudaError_t step_march(Buffers& B, int cur, cudaStream_t st, const double* prev) {
+  cudaError_t step_march(Buffers& B, int cur, cudaStream_t st, const double* prev, bool chunked) {
     if constexpr (DIM == 3) {
-      constexpr size_t smem = march_smem_bytes<K, Real, Store>();
-      auto kern = step3d_march_kernel<K, Real, Store, PRE>;
       int& grid = mgrid[PRE ? 1 : 0];
-      if (grid == 0) {
-        int dev = 0, sms = 0, occ = 0;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e == cudaSuccess) e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-          e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, BLOCK, smem);
+      if constexpr (kHalf) {
+        constexpr size_t smem = half_store::march_smem_bytes<K, Real, Store>();
+        auto kern = half_store::step3d_march_kernel<K, Real, Store, PRE>;
+        const cudaError_t e = resident_grid(kern, BLOCK, smem, grid, B.slots);
         if (e != cudaSuccess) return e;
-        grid = std::max(1, occ) * sms;
-        if (grid > B.slots) grid = (int)B.slots;
+        kern<<<grid, BLOCK, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb);
+        B.last_nb = grid;
+      } else {
+        using T_ = typename MarchTile<Real>::T;
+        constexpr size_t smem = step_smem_bytes<3, K, Real, T_>();
+        auto kern = step3d_march_kernel<K, Real, PRE>;
+        const cudaError_t e = resident_grid(kern, T_::NT, smem, grid, B.slots);
+        if (e != cudaSuccess) return e;
+        const int nb = chunked ? (int)step_blocks() : grid;
+        if (nb > B.slots) return cudaErrorInvalidValue;
+        kern<<<nb, T_::NT, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb,
+                                       chunked ? kChunk : 0);
+        B.last_nb = nb;
       }
-      kern<<<grid, BLOCK, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb);
-      B.last_nb = grid;
       return cudaGetLastError();
     } else {
       return cudaErrorNotSupported;
     }
   }
 
-  // persistent 2-D step with tile shape T_ (kernels 2: 32 x 8, 3: 32 x 16)
-  int pgrid[2] = {0, 0};
-  template <class T_>
-  cudaError_t step_persistent(Buffers& B, int cur, cudaStream_t st, const double* prev,
-                              int& grid_cache) {
-    if constexpr (DIM == 2) {
-      constexpr size_t smem = step_smem_bytes<DIM, K, Real, Store, T_>();
-      auto kern = step_persistent_kernel<DIM, K, Real, Store, T_>;
-      if (grid_cache == 0) {
-        int dev = 0, sms = 0, occ = 0;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e == cudaSuccess) e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-          e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, BLOCK, smem);
+  // staged tiles, one block each (in 3-D, FP16 storage: kChunk planes of one)
+  cudaError_t step_tiled(Buffers& B, int cur, cudaStream_t st, const double* prev) {
+    if constexpr (DIM == 3 && !kHalf) {
+      return step_march<false>(B, cur, st, prev, true);
+    } else {
+      const dim3 grid = step_grid();
+      if (step_blocks() > B.slots) return cudaErrorInvalidValue;
+      auto launch = [&](auto kern, int threads, size_t smem) -> cudaError_t {
+        const cudaError_t e =
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        grid_cache = std::max(1, occ) * sms;
+        kern<<<grid, threads, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb);
+        return cudaGetLastError();
+      };
+      cudaError_t e;
+      if constexpr (kHalf) {
+        e = launch(half_store::step_kernel<DIM, K, Real, Store>, BLOCK,
+                   half_store::step_smem_bytes<DIM, K, Real, Store>());
+      } else if constexpr (sizeof(Real) == 4) {
+        using T_ = Tile<V, 32, 8>;
+        e = launch(step_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>());
+      } else {
+        using T8 = Tile<V, 32, 8>;
+        using T4 = Tile<V, 32, 4>;
+        using T2 = Tile<V, 32, 2>;
+        const int ty = step_ty();
+        e = ty == 8 ? launch(step_kernel<K, Real, T8>, T8::NT, step_smem_bytes<2, K, Real, T8>())
+            : ty == 4 ? launch(step_kernel<K, Real, T4>, T4::NT, step_smem_bytes<2, K, Real, T4>())
+                      : launch(step_kernel<K, Real, T2>, T2::NT, step_smem_bytes<2, K, Real, T2>());
       }
-      const int tiles = ((P.nx + T_::TX - 1) / T_::TX) * ((P.ny + T_::TY - 1) / T_::TY);
+      if (e == cudaSuccess) B.last_nb = step_blocks();
+      return e;
+    }
+  }
+
+  // persistent 2-D step with 32 x 8 (kernel 2) or 32 x 16 (kernel 3) tiles
+  int pgrid[2] = {0, 0};
+  template <int TY>
+  cudaError_t step_persistent(Buffers& B, int cur, cudaStream_t st, const double* prev) {
+    if constexpr (DIM == 2) {
+      int& cached = pgrid[TY == 8 ? 0 : 1];
+      const int tiles = ((P.nx + 31) / 32) * ((P.ny + TY - 1) / TY);
       if (tiles > B.slots) return cudaErrorInvalidValue;
-      kern<<<std::min(grid_cache, tiles), BLOCK, smem, st>>>(
-          P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb, B.tile_ctr, cur);
-      B.last_nb = tiles;
-      return cudaGetLastError();
+      auto launch = [&](auto kern, int threads, size_t smem) -> cudaError_t {
+        const cudaError_t e = resident_grid(kern, threads, smem, cached);
+        if (e != cudaSuccess) return e;
+        kern<<<std::min(cached, tiles), threads, smem, st>>>(
+            P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb, B.tile_ctr, cur);
+        return cudaGetLastError();
+      };
+      cudaError_t e;
+      if constexpr (kHalf) {
+        using T_ = half_store::Tile<2, 32, TY / 8>;
+        e = launch(half_store::step_persistent_kernel<2, K, Real, Store, T_>, BLOCK,
+                   half_store::step_smem_bytes<2, K, Real, Store, T_>());
+      } else {
+        using T_ = Tile<V, 32, TY>;
+        e = launch(step_persistent_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>());
+      }
+      if (e == cudaSuccess) B.last_nb = tiles;
+      return e;
     } else {
       return cudaErrorNotSupported;
     }
   }
-  int kernel() const override { return kernel_sel; }
+  int kernel() override { return resolved(); }
 
   static constexpr bool kBatchable = DIM == 2 && K == 0;
   size_t batch_entry_bytes() const override {
@@ -524,18 +635,28 @@ struct LauncherImpl final : Launcher {
       std::memcpy(dst, &e, sizeof(e));
     }
   }
+  // the batch kernel of a tile shape, its threads and shared memory
+  template <int CFG, class F>
+  static auto with_batch_kernel(F f) {
+    if constexpr (kHalf) {
+      using T_ = typename half_store::BatchShape<CFG>::T;
+      return f(half_store::batch_step_kernel<K, Real, Store, T_>, BLOCK,
+               half_store::step_smem_bytes<2, K, Real, Store, T_>());
+    } else {
+      using T_ = typename BatchShape<Real, CFG>::T;
+      return f(batch_step_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>());
+    }
+  }
   template <int CFG>
   static int batch_occ_of() {
-    using T_ = typename BatchShape<CFG>::T;
-    int nb = 0;
-    auto kern = batch_step_kernel<K, Real, Store, T_>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)batch_smem_bytes<K, Real, Store, T_>()) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, BLOCK,
-                                                      batch_smem_bytes<K, Real, Store, T_>()) !=
-            cudaSuccess)
-      return 0;
-    return nb;
+    return with_batch_kernel<CFG>([](auto kern, int threads, size_t smem) {
+      int nb = 0;
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+              cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem) != cudaSuccess)
+        return 0;
+      return nb;
+    });
   }
   int batch_occupancy(int cfg) const override {
     if constexpr (kBatchable) {
@@ -548,10 +669,11 @@ struct LauncherImpl final : Launcher {
   template <int CFG>
   static cudaError_t batch_launch_cfg(const void* entries, const int* tile_begin, int ndom,
                                       int grid, int flip, unsigned* ctr, cudaStream_t st) {
-    using T_ = typename BatchShape<CFG>::T;
-    batch_step_kernel<K, Real, Store, T_><<<grid, BLOCK, batch_smem_bytes<K, Real, Store, T_>(), st>>>(
-        static_cast<const BatchDom<K, Real, Store>*>(entries), tile_begin, ndom, flip, ctr);
-    return cudaGetLastError();
+    return with_batch_kernel<CFG>([&](auto kern, int threads, size_t smem) {
+      kern<<<grid, threads, smem, st>>>(static_cast<const BatchDom<K, Real, Store>*>(entries),
+                                        tile_begin, ndom, flip, ctr);
+      return cudaGetLastError();
+    });
   }
   cudaError_t batch_launch(const void* entries, const int* tile_begin, int ndom, int cfg, int grid,
                            int flip, unsigned* ctr, cudaStream_t st) const override {
@@ -589,7 +711,7 @@ struct LauncherImpl final : Launcher {
         int dev = 0, sms = 0, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, BLOCK, LY::smem_bytes);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, LY::NT, LY::smem_bytes);
         const long long tiles = (long long)((P.nx + LY::TX - 1) / LY::TX) *
                                 ((P.ny + LY::TY - 1) / LY::TY);
         if (per < 1 || sms < 1) {
@@ -637,7 +759,7 @@ struct LauncherImpl final : Launcher {
       const int tiles_x = (P.nx + LY::TX - 1) / LY::TX;
       const int n_tiles = tiles_x * ((P.ny + LY::TY - 1) / LY::TY);
       const TmaMaps& m = maps[cur];
-      step_tma_kernel<K, Store><<<tma_grid, BLOCK, LY::smem_bytes, st>>>(
+      step_tma_kernel<K, Store><<<tma_grid, LY::NT, LY::smem_bytes, st>>>(
           P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb, m.T, m.phi, m.Ts, m.Y, m.g,
           tiles_x, n_tiles, wait_limit);
       B.last_nb = tma_grid;
@@ -648,7 +770,7 @@ struct LauncherImpl final : Launcher {
   }
 
   // One step's launches on stream st, with its host bookkeeping.
-  cudaError_t one_step(Buffers& B, int& cur, cudaStream_t st, dim3 grid, size_t smem) {
+  cudaError_t one_step(Buffers& B, int& cur, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     if constexpr (K > 0) {
       if (P.chem >= 2) {
@@ -658,22 +780,17 @@ struct LauncherImpl final : Launcher {
     }
     const double* prev = (!p0_closed && B.pending)
                              ? B.partials + (size_t)4 * B.slots * B.last_parity : nullptr;
-    if (kernel_sel == 1 && tma_usable(B, cur)) {
+    const int sel = resolved();
+    if (sel == 1 && tma_usable(B, cur)) {
       e = step_tma(B, cur, st, prev);
       if (e != cudaSuccess) return e;
-    } else if (kernel_sel == 2) {
-      e = step_persistent<Tile<DIM, 32, 1>>(B, cur, st, prev, pgrid[0]);
-      if (e != cudaSuccess) return e;
-    } else if (kernel_sel == 3) {
-      e = step_persistent<Tile<DIM, 32, 2>>(B, cur, st, prev, pgrid[1]);
-      if (e != cudaSuccess) return e;
-    } else if (kernel_sel == 4 || kernel_sel == 5) {
-      e = kernel_sel == 5 ? step_march<true>(B, cur, st, prev) : step_march<false>(B, cur, st, prev);
-      if (e != cudaSuccess) return e;
     } else {
-      step_kernel<DIM, K, Real, Store><<<grid, BLOCK, smem, st>>>(P, state(B, cur), p0_closed,
-                                                                   prev, (unsigned)B.last_nb);
-      B.last_nb = step_blocks();
+      e = sel == 2   ? step_persistent<8>(B, cur, st, prev)
+          : sel == 3 ? step_persistent<16>(B, cur, st, prev)
+          : sel == 4 ? step_march<false>(B, cur, st, prev, false)
+          : sel == 5 ? step_march<true>(B, cur, st, prev, false)
+                            : step_tiled(B, cur, st, prev);
+      if (e != cudaSuccess) return e;
     }
     if (P.feed) {
       e = feed(B, cur, st);
@@ -706,12 +823,8 @@ struct LauncherImpl final : Launcher {
   }
 
   cudaError_t step(Buffers& B, int& cur, int nsteps, cudaStream_t st) override {
-    constexpr size_t smem = step_smem_bytes<DIM, K, Real, Store>();
-    cudaError_t e = cudaFuncSetAttribute(step_kernel<DIM, K, Real, Store>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const dim3 grid = step_grid();
-    if (kernel_sel >= 2 && nsteps > 0) {
+    cudaError_t e = cudaSuccess;
+    if ((resolved() == 2 || resolved() == 3) && nsteps > 0) {
       // both counters start at zero; consecutive steps then clear each other's
       e = cudaMemsetAsync(B.tile_ctr, 0, 2 * sizeof(unsigned), st);
       if (e != cudaSuccess) return e;
@@ -719,7 +832,7 @@ struct LauncherImpl final : Launcher {
     int n = 0;
     if (nsteps >= kGraphMinSteps && !P.moving) {
       for (; n < 2; ++n) {
-        e = one_step(B, cur, st, grid, smem);
+        e = one_step(B, cur, st);
         if (e != cudaSuccess) return e;
       }
       if (!cap_st) {
@@ -734,8 +847,8 @@ struct LauncherImpl final : Launcher {
       cudaGraphExec_t x = nullptr;
       e = cudaStreamBeginCapture(cap_st, cudaStreamCaptureModeRelaxed);
       if (e == cudaSuccess) {
-        cudaError_t e1 = one_step(B, cur, cap_st, grid, smem);
-        if (e1 == cudaSuccess) e1 = one_step(B, cur, cap_st, grid, smem);
+        cudaError_t e1 = one_step(B, cur, cap_st);
+        if (e1 == cudaSuccess) e1 = one_step(B, cur, cap_st);
         e = cudaStreamEndCapture(cap_st, &g);
         if (e == cudaSuccess) e = e1;
       }
@@ -763,7 +876,7 @@ struct LauncherImpl final : Launcher {
       if (e != cudaSuccess) return e;
     }
     for (; n < nsteps; ++n) {
-      e = one_step(B, cur, st, grid, smem);
+      e = one_step(B, cur, st);
       if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();

@@ -119,7 +119,10 @@ struct TmaLayout {
   static constexpr int FBP = (FBOX * 4 + 127) / 128 * 32;  // 128-byte aligned box slot
   static constexpr int OFF_T = 0, OFF_PHI = FBP, OFF_TS = 2 * FBP, OFF_Y = 3 * FBP;
   static constexpr int PBOX = PW * PH;                // Stores per population box
-  static constexpr int HX = TX + 2, HP = HX * (TY + 2);
+  // derived plane: rows start two cells left of the tile, so that a thread's
+  // pair of cells is an aligned word of its row
+  static constexpr int HX = TX + 4, HP = HX * (TY + 2);
+  static constexpr int NT = TX * TY / 2;              // threads, two cells each
   static constexpr int NDER = 5;                      // rho, kT, mu, fD, RF
   static constexpr size_t raw_bytes = ((size_t)(3 * FBP + K * FBOX) * 4 + 127) / 128 * 128;
   static constexpr size_t pop_bytes = (size_t)Q * PBOX * sizeof(Store);
@@ -129,49 +132,45 @@ struct TmaLayout {
   // +128 so the base can be rounded up to a 128-byte boundary in the kernel
   static constexpr size_t bar_off = 2 * stage_bytes + der_bytes;
   static constexpr size_t red_off = bar_off + 64;
-  static constexpr size_t flag_off = red_off + 32 * sizeof(double);
+  static constexpr size_t flag_off = red_off + 96 * sizeof(double);
   static constexpr size_t smem_bytes = flag_off + 16 + 128;
 };
 
-// Accessor over a TMA stage (raw fields, populations) plus the derived plane.
+// Accessor over a TMA stage (raw fields, populations) plus the derived plane,
+// for the pair of cells (lx, lx + 1) of row ly.
 template <int K, class Store>
 struct TmaAcc {
   using LY = TmaLayout<K, Store>;
-  static constexpr bool has_pops = true;
-  static constexpr bool kStash = false;
   const float* __restrict__ raw;
   const Store* __restrict__ pops;
   const float* __restrict__ der;
   int lx, ly;
-  bool pv;  // the stage's population windows are valid for this cell (off every face)
-  __device__ __forceinline__ int ridx(int dx, int dy) const {
-    return (ly + 1 + dy) * LY::FW + lx + LY::XL + dx;
-  }
-  __device__ __forceinline__ int didx(int dx, int dy) const {
-    return (ly + 1 + dy) * LY::HX + lx + 1 + dx;
-  }
-  __device__ __forceinline__ float get(int f, int dx, int dy) const {
+  __device__ __forceinline__ const float* at(int f, int dx, int dy) const {
+    const int r = (ly + 1 + dy) * LY::FW + lx + LY::XL + dx;
+    const int d = (ly + 1 + dy) * LY::HX + lx + 2 + dx;
     switch (f) {
-      case F_T: return raw[LY::OFF_T + ridx(dx, dy)];
-      case F_PHI: return raw[LY::OFF_PHI + ridx(dx, dy)];
-      case F_TS: return raw[LY::OFF_TS + ridx(dx, dy)];
-      case F_RHO: return der[0 * LY::HP + didx(dx, dy)];
-      case F_KT: return der[1 * LY::HP + didx(dx, dy)];
-      case F_MU: return der[2 * LY::HP + didx(dx, dy)];
-      case F_FD: return der[3 * LY::HP + didx(dx, dy)];
-      case F_RF: return der[4 * LY::HP + didx(dx, dy)];
-      default: return raw[LY::OFF_Y + (f - F_Y0) * LY::FBOX + ridx(dx, dy)];
+      case F_T: return raw + LY::OFF_T + r;
+      case F_PHI: return raw + LY::OFF_PHI + r;
+      case F_TS: return raw + LY::OFF_TS + r;
+      case F_RHO: return der + 0 * LY::HP + d;
+      case F_KT: return der + 1 * LY::HP + d;
+      case F_MU: return der + 2 * LY::HP + d;
+      case F_FD: return der + 3 * LY::HP + d;
+      case F_RF: return der + 4 * LY::HP + d;
+      default: return raw + LY::OFF_Y + (f - F_Y0) * LY::FBOX + r;
     }
   }
-  __device__ __forceinline__ float c(int f) const { return get(f, 0, 0); }
-  __device__ __forceinline__ float n(int f, int a, int s) const {
-    return a == 0 ? get(f, s, 0) : get(f, 0, s);
+  __device__ __forceinline__ float2 c(int f) const {
+    return *reinterpret_cast<const float2*>(at(f, 0, 0));
   }
-  template <class S>
-  __device__ __forceinline__ float pop(int i, float w_over_scale) const {
-    const int cx = Lattice<2>::c(i, 0);
-    return Codec<Store, float>::get(pops + i * LY::PBOX + ly * LY::PW + lx - cx + LY::XLP,
-                                    w_over_scale);
+  __device__ __forceinline__ float2 n(int f, int a, int s, float2 own) const {
+    if (a == 1) return *reinterpret_cast<const float2*>(at(f, 0, s));
+    const float v = *at(f, s < 0 ? -1 : 2, 0);
+    return s < 0 ? make_float2(v, own.x) : make_float2(own.y, v);
+  }
+  __device__ __forceinline__ float2 pop(int i) const {
+    const Store* p = pops + i * LY::PBOX + ly * LY::PW + lx - Lattice<2>::c(i, 0) + LY::XLP;
+    return make_float2(p[0], p[1]);
   }
 };
 
@@ -182,8 +181,9 @@ __device__ __forceinline__ void fix_halo(const Params<float, K>& P,
                                          const State<float, Store>& S, float* raw, int x0,
                                          int y0) {
   using LY = TmaLayout<K, Store>;
-  for (int h = threadIdx.x; h < LY::HP; h += blockDim.x) {
-    const int hx = h % LY::HX, hy = h / LY::HX;
+  constexpr int BX = LY::TX + 2;
+  for (int h = threadIdx.x; h < BX * LY::FH; h += LY::NT) {
+    const int hx = h % BX, hy = h / BX;
     int q[2] = {x0 - 1 + hx, y0 - 1 + hy};
     if ((q[0] >= 0 && q[0] < P.nx) && (q[1] >= 0 && q[1] < P.ny)) continue;
     int ghost_face = -1, nout = 0;
@@ -228,36 +228,40 @@ __device__ __forceinline__ void fix_halo(const Params<float, K>& P,
   }
 }
 
-// Properties of every staged cell (tile + halo) from the staged raw fields.
+// Properties of every staged pair of cells (tile + halo) from the staged raw
+// fields.  (The outer cell of the first and last pair of a row is staged but
+// never read.)
 template <int K, class Store>
 __device__ __forceinline__ void derive_plane(const Params<float, K>& P, float* raw,
                                              float* der, float P0) {
   using LY = TmaLayout<K, Store>;
-  for (int h = threadIdx.x; h < LY::HP; h += blockDim.x) {
-    const int hx = h % LY::HX, hy = h / LY::HX;
-    if ((hx == 0 || hx == LY::HX - 1) && (hy == 0 || hy == LY::TY + 1)) continue;  // corners
-    const int r = hy * LY::FW + hx - 1 + LY::XL;
-    const float T = raw[LY::OFF_T + r];
-    const float phis = raw[LY::OFF_PHI + r];
-    if (!P.Ts_field) raw[LY::OFF_TS + r] = P.Ts_uniform;
-    float Y[Params<float, K>::KK];
+  constexpr int PW = LY::HX / 2;
+  for (int h = threadIdx.x; h < PW * LY::FH; h += LY::NT) {
+    const int hy = h / PW, hx = (h - hy * PW) * 2;
+    const int r = hy * LY::FW + hx - 2 + LY::XL, d = hy * LY::HX + hx;
+    auto get = [&](int off) { return *reinterpret_cast<const float2*>(raw + off + r); };
+    auto put = [&](int f, float2 v) { *reinterpret_cast<float2*>(der + f * LY::HP + d) = v; };
+    const float2 T = get(LY::OFF_T), phis = get(LY::OFF_PHI);
+    if (!P.Ts_field) *reinterpret_cast<float2*>(raw + LY::OFF_TS + r) = splat<float2>(P.Ts_uniform);
+    float2 Y[Params<float, K>::KK];
 #pragma unroll
-    for (int k = 0; k < K; ++k) Y[k] = raw[LY::OFF_Y + k * LY::FBOX + r];
-    const float phif = 1.f - phis;
-    const float invMw = mixture_invMw(P, Y);
-    const float rho = fdiv(P0 * P.eos_cr, T * invMw);
-    const float cp = mixture_cp(P, Y);
-    float mu, lam;
-    transport(P, T, Y, invMw, cp, mu, lam);
-    float fD = 1.f;
+    for (int k = 0; k < K; ++k) Y[k] = get(LY::OFF_Y + k * LY::FBOX);
+    const float2 one = splat<float2>(1.f);
+    const float2 phif = vsub(one, phis);
+    const float2 invMw = mixture_invMw<float, K, float2>(P, Y);
+    const float2 rho = fdiv(splat<float2>(P0 * P.eos_cr), vmul(T, invMw));
+    const float2 cp = mixture_cp<float, K, float2>(P, Y);
+    float2 mu, lam;
+    transport<float, K, float2>(P, T, Y, invMw, cp, mu, lam);
+    float2 fD = one;
     if constexpr (K > 0) {
-      if (P.D_Tdep) fD = fpow(T * P.inv_DTref, P.D_exp);
+      if (P.D_Tdep) fD = fpow(vmuls<float2>(P.inv_DTref, T), P.D_exp);
     }
-    der[0 * LY::HP + h] = rho;
-    der[1 * LY::HP + h] = phif * lam;
-    der[2 * LY::HP + h] = mu;
-    der[3 * LY::HP + h] = fD;
-    der[4 * LY::HP + h] = phif * rho * fD;
+    put(0, rho);
+    put(1, vmul(phif, lam));
+    put(2, mu);
+    put(3, fD);
+    put(4, vmul(vmul(phif, rho), fD));
   }
 }
 
@@ -281,7 +285,7 @@ __device__ __forceinline__ void issue_tile(const TmaMapRefs& M, const Params<flo
 }
 
 template <int K, class Store>
-__global__ void __launch_bounds__(BLOCK, 2)
+__global__ void __launch_bounds__((TmaLayout<K, Store>::NT), 2)
 step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_closed,
                 const double* __restrict__ prev_partials, unsigned prev_nb,
                 const __grid_constant__ CUtensorMap mT, const __grid_constant__ CUtensorMap mPhi,
@@ -326,8 +330,9 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
   }
   __syncthreads();
 
-  const int lx = threadIdx.x % LY::TX, ly = threadIdx.x / LY::TX;
-  float accI = 0.f, accIn = 0.f, accOut = 0.f;
+  const int lx = (threadIdx.x % (LY::TX / 2)) * 2, ly = threadIdx.x / (LY::TX / 2);
+  float2 accI = splat<float2>(0.f);
+  float accIn = 0.f, accOut = 0.f;
   bool any_flux = false;
   int first = blockIdx.x;
   if (threadIdx.x == 0 && first < n_tiles)
@@ -367,11 +372,19 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
     const int x = x0 + lx, y = y0 + ly;
     if (x < P.nx && y < P.ny) {
       const TmaAcc<K, Store> A{raw, reinterpret_cast<const Store*>(stage[s] + LY::raw_bytes), der,
-                               lx, ly, x > 0 && x < P.nx - 1 && y > 0 && y < P.ny - 1};
-      const int c = x + P.nx * y;
-      const int xyz[3] = {x, y, 0};
+                               lx, ly};
+      const CellPos q{x + P.nx * y, x, y, 0, S.even != 0, true};  // nx is even here
+      // the stage's population windows are valid off every face
+      float2 g[LY::Q];
+      if (x > 0 && x + 1 < P.nx - 1 && y > 0 && y < P.ny - 1) {
+#pragma unroll
+        for (int i = 0; i < LY::Q; ++i) g[i] = A.pop(i);
+      } else {
+        load_pops<2, K, float, float2>(P, S, x, y, 0, g);
+      }
       float fi, fo;
-      accI += cell_update<2, K, float, Store>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
+      accI = vadd(accI,
+                  cell_update<2, K, float, float2>(P, S, A, g, q, P0, dlnP0, dP0r, fi, fo));
       accIn += fi;
       accOut += fo;
     }
@@ -380,12 +393,8 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
     __syncthreads();
   }
 
-  const double sI = block_sum<float>(accI, red_sh);
-  double sIn = 0, sOut = 0;
-  if (any_flux) {
-    sIn = block_sum<float>(accIn, red_sh);
-    sOut = block_sum<float>(accOut, red_sh);
-  }
+  double sI, sIn, sOut;
+  block_sum3(accI, accIn, accOut, any_flux, red_sh, sI, sIn, sOut);
   publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
                    P.inv_rho_ref);
 }
