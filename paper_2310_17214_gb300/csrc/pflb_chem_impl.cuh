@@ -3,11 +3,24 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "pflb_chem.cuh"
 #include "pflb_surrogate_tc.cuh"
 
 namespace pflb {
+
+// f(number of reactions as a constant): the integrators are compiled per count
+template <class F>
+void with_reactions(int J, F f) {
+  switch (J) {
+    case 0:
+    case 1: return f(std::integral_constant<int, 1>());
+    case 2: return f(std::integral_constant<int, 2>());
+    case 3: return f(std::integral_constant<int, 3>());
+    default: return f(std::integral_constant<int, 4>());
+  }
+}
 
 template <int K, class Real>
 cudaError_t chem_pass_launch(const Params<Real, K>& P, const State<Real, Real>& S, Real* src,
@@ -15,7 +28,9 @@ cudaError_t chem_pass_launch(const Params<Real, K>& P, const State<Real, Real>& 
                              double* stats, double* out, cudaStream_t st) {
   const int blocks = (P.N + BLOCK - 1) / BLOCK;
   if (P.chem == 2) {
-    chem_implicit_kernel<K, Real, Real><<<blocks, BLOCK, 0, st>>>(P, S, src);
+    with_reactions(P.J, [&](auto J) {
+      chem_implicit_kernel<K, J.value, Real, Real><<<blocks, BLOCK, 0, st>>>(P, S, src);
+    });
   } else if (P.chem == 3) {
     if constexpr (K == 6) {
       if (!surr || !fb_idx) return cudaErrorInvalidValue;
@@ -55,8 +70,10 @@ cudaError_t chem_pass_launch(const Params<Real, K>& P, const State<Real, Real>& 
       }
       const int fb_blocks = (int)std::min<long long>(
           ((long long)P.N + FALLBACK_BLOCK - 1) / FALLBACK_BLOCK, (long long)sms * 16);
-      chem_fallback_kernel<K, Real, Real><<<fb_blocks, FALLBACK_BLOCK, 0, st>>>(P, S, src,
-                                                                                fb_idx, fb_count);
+      with_reactions(P.J, [&](auto J) {
+        chem_fallback_kernel<K, J.value, Real, Real>
+            <<<fb_blocks, FALLBACK_BLOCK, 0, st>>>(P, S, src, fb_idx, fb_count);
+      });
     } else {
       return cudaErrorNotSupported;
     }

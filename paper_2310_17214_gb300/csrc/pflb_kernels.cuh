@@ -89,6 +89,10 @@ struct Chem64 {
   double dS_R[JMAX], dH_R[JMAX];  // dS / R, dH / R
   double M[KK], invM[KK], cp[KK], hf[KK];
   double p_ref, ln_pref_R, rho_ref, dt;  // ln_pref_R = ln(p_ref / R)
+  double H[JMAX], cM[JMAX];  // sum_k hf_k Ms_jk, sum_k cp_k Ms_jk
+  double pref_R;             // p_ref / R
+  int used;                  // bit k: species k enters a rate
+  __device__ __forceinline__ bool active(int j) const { return A[j] != 0.0; }
 };
 
 // FP32 copy of the chemistry for the Newton fallback of the surrogate in FP32
@@ -102,6 +106,8 @@ struct Chem32 {
   float Ms[JMAX][KK];  // M_k s_kj
   float invM[KK], cp[KK], hf[KK];
   float ln_pref_R, dt;
+  float H[JMAX], cM[JMAX];
+  __device__ __forceinline__ bool active(int j) const { return on[j] != 0; }
 };
 
 // Everything in lattice units, converted once on the host (pflb_launch.cuh).
@@ -413,101 +419,8 @@ __device__ __forceinline__ void rates(const Params<Real, K>& P, V T, const V* Y,
   omT = wt;
 }
 
-// Power C^o of a concentration for the reaction orders that occur (0, 1, 2,
-// 1/2: multiplications and a square root), pow() otherwise; d = dC^o/dC for
-// C > 0, in the precision LA of the Jacobian.
-template <class LA>
-__device__ __forceinline__ double conc_power(double C, double o, LA& d) {
-  if (o == 1.0) { d = LA(1); return C; }
-  if (o == 0.0) { d = LA(0); return 1.0; }
-  if (o == 2.0) { d = LA(2) * LA(C); return C * C; }
-  if (o == 0.5) {
-    const double s = sqrt(C);
-    d = s > 0.0 ? LA(0.5) / LA(s) : LA(0);
-    return s;
-  }
-  d = C > 0.0 ? LA(o * pow(C, o - 1.0)) : LA(0);
-  return pow(C, o);
-}
-
-// Rates w_k (kg/(m^3 s), FP64) and their Jacobian dw_k/dz_m, z = (Y_1..Y_K,
-// T), in the precision LA: FP64 for FP64 domains; FP32 for FP32 domains,
-// where the Jacobian only steers the Newton iteration and the FP64 residual
-// decides where it converges.
-template <int K, class LA>
-__device__ __forceinline__ void rates_jacobian64(const Chem64<K>& c, const double* z, double rho,
-                                                 double* w, LA (*dw)[K + 1]) {
-  constexpr int KK = K > 0 ? K : 1;
-  constexpr int n = K + 1;
-  const double T = z[K], invT = 1.0 / T;
-  double Cc[KK];
-  LA dC[KK];
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const double d = z[k] > 0 ? rho * c.invM[k] : 0.0;
-    dC[k] = LA(d);
-    Cc[k] = z[k] > 0 ? z[k] * d : 0.0;
-    w[k] = 0;
-#pragma unroll
-    for (int m = 0; m < n; ++m) dw[k][m] = LA(0);
-  }
-  double lnT = 0.0;
-  bool have_lnT = false;
-#pragma unroll
-  for (int j = 0; j < JMAX; ++j) {
-    if (c.A[j] == 0.0) continue;
-    double kf = c.A[j] * exp(-c.EaR[j] * invT);
-    if (c.b[j] != 0.0) kf *= pow(T, c.b[j]);
-    const double dlkf = (c.EaR[j] * invT + c.b[j]) * invT;
-    double kr = 0.0, dlkr = dlkf;
-    if (c.rev[j]) {
-      // K_c = exp(dS/R - dH/(R T)) (p_ref / (R T))^dn
-      double lnKc = c.dS_R[j] - c.dH_R[j] * invT;
-      if (c.dn[j] != 0.0) {
-        if (!have_lnT) { lnT = log(T); have_lnT = true; }
-        lnKc += c.dn[j] * (c.ln_pref_R - lnT);
-      }
-      kr = kf * exp(-lnKc);
-      dlkr = dlkf - (c.dH_R[j] * invT + c.dn[j]) * invT;
-    }
-    LA dq[K + 1];
-#pragma unroll
-    for (int m = 0; m < n; ++m) dq[m] = LA(0);
-#pragma unroll
-    for (int dir = 0; dir < 2; ++dir) {
-      if (dir == 1 && !c.rev[j]) break;
-      const double kk = dir == 0 ? kf : -kr;
-      double Pw[KK], pre[K + 1];
-      LA Dp[KK], suf[K + 1];
-#pragma unroll
-      for (int k = 0; k < K; ++k)
-        Pw[k] = conc_power(Cc[k], dir == 0 ? c.order[j][k] : c.rorder[j][k], Dp[k]);
-      // prefix / suffix products: the product without factor m, no division
-      pre[0] = 1.0;
-      suf[K] = LA(1);
-#pragma unroll
-      for (int k = 0; k < K; ++k) pre[k + 1] = pre[k] * Pw[k];
-#pragma unroll
-      for (int k = K - 1; k >= 0; --k) suf[k] = LA(Pw[k]) * suf[k + 1];
-      const double q = kk * pre[K];
-#pragma unroll
-      for (int k = 0; k < K; ++k) w[k] += c.Ms[j][k] * q;
-      dq[K] += LA(q) * LA(dir == 0 ? dlkf : dlkr);
-#pragma unroll
-      for (int m = 0; m < K; ++m) dq[m] += LA(kk * pre[m]) * suf[m + 1] * Dp[m] * dC[m];
-    }
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-      for (int m = 0; m < n; ++m) dw[k][m] += LA(c.Ms[j][k]) * dq[m];
-  }
-}
-
 // Solve A x = r in place (r <- x) by Gaussian elimination with partial
-// pivoting; false if a pivot is zero.  The compiler keeps a 7 x 7 matrix in
-// local memory here (the row swap after the pivot search defeats its scalar
-// replacement); a fully unrolled form with the matrix in registers was tried
-// and is slower, its register pressure spilling more than the matrix.
+// pivoting; false if a pivot is zero.
 template <int n, class LA>
 __device__ __forceinline__ bool solve_pivoted(LA (*A)[n], LA* r) {
   LA dinv[n];
@@ -529,292 +442,375 @@ __device__ __forceinline__ bool solve_pivoted(LA (*A)[n], LA* r) {
         const LA t = r[col]; r[col] = r[rr]; r[rr] = t;
       }
     }
-    const LA inv = LA(1) / A[col][col];
-    dinv[col] = inv;
+    dinv[col] = LA(1) / A[col][col];
 #pragma unroll
     for (int rr = col + 1; rr < n; ++rr) {
-      const LA f = A[rr][col] * inv;
+      const LA f = vmul(A[rr][col], dinv[col]);
 #pragma unroll
-      for (int k = col + 1; k < n; ++k) A[rr][k] -= f * A[col][k];
-      r[rr] -= f * r[col];
+      for (int k = col + 1; k < n; ++k) A[rr][k] = vfma(-f, A[col][k], A[rr][k]);
+      r[rr] = vfma(-f, r[col], r[rr]);
     }
   }
 #pragma unroll
   for (int rr = n - 1; rr >= 0; --rr) {
     LA s = r[rr];
 #pragma unroll
-    for (int k = rr + 1; k < n; ++k) s -= A[rr][k] * r[k];
-    r[rr] = s * dinv[rr];
+    for (int k = rr + 1; k < n; ++k) s = vfma(-A[rr][k], r[k], s);
+    r[rr] = vmul(s, dinv[rr]);
   }
   return true;
 }
 
-// ----------------------------------------------- implicit chemistry (FP64)
+// ----------------------------------------------------- implicit chemistry
 // One lattice step of the chemistry alone at frozen density (operator
-// splitting), backward Euler: z = (Y_1..Y_K, T), dY/dt = omega/rho,
-// dT/dt = -sum hf omega / (rho cp(Y)).  Newton with the analytic Jacobian and
-// Gaussian elimination with partial pivoting (tolerance 1e-13, <= 30
-// iterations); if it fails the step is split into 2, 4, ..., 64 backward-Euler
-// sub-steps.  Kept out of line so that it does not weigh on the register
-// allocation of the rest of the step.  The arithmetic is laid out for a short
-// dependency chain (FP64 latency sets the time of a warp): reciprocals taken
-// once, square roots for half orders, no dynamic array indices.
-// The state, the rates and the residual are FP64 in every mode; the Jacobian,
-// the Newton matrix and its elimination take the precision LA (FP64 for FP64
-// domains, FP32 for FP32 domains).  A direction from an FP32 elimination is
-// off by about cond(A) x 6e-8 of itself, so the iteration still contracts and
-// stops where the FP64 residual puts the root (the update test is relative
-// to the update, not to the FP32 rounding), and the elimination runs on the
-// FP32 pipe instead of GB300's narrow FP64 one.
-template <int K, class LA>
-__device__ __forceinline__ void chem_be_newton(const Chem64<K>* C0,
-                                            double T0, const double* Y0, double rho,
-                                            double* dY, double* dT) {
-  constexpr int n = K + 1;
-  const auto& c = *C0;
-  const double inv_rho = 1.0 / rho;
-  double zs[K + 1], z[K + 1], y0[K + 1];
-#pragma unroll
-  for (int k = 0; k < K; ++k) y0[k] = Y0[k];
-  y0[K] = T0;
-  int ok = -1;
-  // the sub-step and Newton loops stay rolled: unrolled, they multiply the
-  // fully unrolled Jacobian and elimination by up to 7 x 30 copies
-#pragma unroll 1
-  for (int nsub = 1; nsub <= 64 && ok != 0; nsub *= 2) {
-#pragma unroll
-    for (int m = 0; m < n; ++m) zs[m] = y0[m];
-    ok = 0;
-    const double h = c.dt / nsub, hr = h * inv_rho;
-#pragma unroll 1
-    for (int sub = 0; sub < nsub && ok == 0; ++sub) {
-#pragma unroll
-      for (int m = 0; m < n; ++m) z[m] = zs[m];
-      const double inv_Ts = 1.0 / zs[K];  // temperature scale of the update test
-      ok = -1;
-#pragma unroll 1
-      for (int it = 0; it < 30; ++it) {
-        double w[K + 1];
-        LA A[K + 1][K + 1];  // rows 0..K-1: dw_k/dz_m, then the Newton matrix
-        rates_jacobian64<K, LA>(c, z, rho, w, A);
-        double cp = 0, hw = 0;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          cp += z[k] * c.cp[k];
-          hw += c.hf[k] * w[k];
-        }
-        const double inv_rcp = inv_rho / cp;
-        // Newton system (I - h dF/dz) dz = -(z - zs - h F): residual in FP64,
-        // matrix in LA, built in place (the T row first, from the rates'
-        // Jacobian, then the species rows)
-        const LA hrL = LA(hr), hL = LA(h), inv_rcpL = LA(inv_rcp);
-        const LA hwcL = LA(hw * inv_rcp / cp);
-        LA r[K + 1];
-#pragma unroll
-        for (int m = 0; m < n; ++m) {
-          LA dhw = LA(0);
-#pragma unroll
-          for (int k = 0; k < K; ++k) dhw += LA(c.hf[k]) * A[k][m];
-          LA dFT = -dhw * inv_rcpL;
-          if (m < K) dFT += hwcL * LA(c.cp[m]);
-          A[K][m] = LA(m == K ? 1 : 0) - hL * dFT;
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          r[k] = LA(-(z[k] - zs[k] - hr * w[k]));
-#pragma unroll
-          for (int m = 0; m < n; ++m) A[k][m] = LA(k == m ? 1 : 0) - hrL * A[k][m];
-        }
-        r[K] = LA(-(z[K] - zs[K] + h * hw * inv_rcp));
-        if (!solve_pivoted<K + 1, LA>(A, r)) break;
-        double big = 0;
-        bool bad = false;
-#pragma unroll
-        for (int m = 0; m < n; ++m) {
-          z[m] += double(r[m]);
-          const double e = fabs(double(r[m])) * (m < K ? 1.0 : inv_Ts);
-          if (!(e == e)) bad = true;
-          if (e > big) big = e;
-        }
-        if (bad || !(z[K] > 0)) break;
-        if (big < 1e-13) { ok = 0; break; }
-      }
-#pragma unroll
-      for (int m = 0; m < n; ++m) zs[m] = z[m];
-    }
+// splitting), backward Euler: dY/dt = omega/rho, dT/dt = -sum hf omega / (rho
+// cp(Y)), Newton with the analytic Jacobian (<= 30 iterations); if it fails
+// the step is split into 2, 4, ..., 64 backward-Euler sub-steps.
+//
+// The species only move along the reactions: omega_k = sum_j M_k s_kj q_j, so
+// after its first iteration the Newton iterate of the K + 1 unknowns (Y, T) is
+// Y = Y_s + sum_j Ms_j xi_j, and the T row, with the rows of the reactions
+// inserted, reads dT = R - sum_i a_i dxi_i with
+//   R = -(T - T_s) - sum_j H_j xi_j / cp,  H_j = sum_k hf_k Ms_jk,
+//   a_i = H_i / cp - (h / rho) (sum_j H_j q_j) / cp^2 sum_k cp_k Ms_ik.
+// So the same iteration is carried by the J progress variables xi,
+//   sum_i [delta_ji - hr (Q_ji - q_jT a_i)] dxi_i = hr (q_j + q_jT R) - xi_j,
+//   Q_ji = sum_k dq_j/dY_k Ms_ik,  hr = h / rho,
+// a J x J system (two reactions: 2 x 2) in place of the (K + 1) x (K + 1) one.
+//
+// FP64 domains do everything in FP64.  FP32 domains (LA = float) keep state,
+// rates and right-hand side in FP64 and take the Jacobian, the solve and the
+// update test in FP32: a direction off by about cond(A) x 6e-8 of itself still
+// contracts, and the iteration stops where the FP64 right-hand side puts the
+// root.  The FP64 pipe bounds this pre-pass (one warp instruction every 16
+// cycles per SM, conversions and comparisons included), so the FP32 part takes
+// its own copies of the constants, signs are tested on the bit pattern, and
+// what an iteration needs only if another follows is left to that one (most
+// cells are cold and take one).  2048 x 512 cells of the two-step bed, FP32
+// domain, a step: 1.28 ms with the 7 x 7 system, 1.20 with the 2 x 2 one, 0.74
+// so.
+
+// Power C^o of a concentration for the reaction orders that occur (1, 2, 1/2:
+// multiplications and a square root), pow() otherwise; the second form also
+// gives d = dC^o/dC for C > 0.
+template <class R>
+__device__ __forceinline__ R conc_power(R C, R o) {
+  if (o == R(1)) return C;
+  if (o == R(2)) return C * C;
+  if (o == R(0.5)) return sqrt(C);
+  return pow(C, o);
+}
+template <class R>
+__device__ __forceinline__ R conc_power(R C, R o, R& d) {
+  if (o == R(1)) { d = R(1); return C; }
+  if (o == R(2)) { d = R(2) * C; return C * C; }
+  if (o == R(0.5)) {
+    const R s = sqrt(C);
+    d = s > R(0) ? R(0.5) / s : R(0);
+    return s;
   }
-#pragma unroll
-  for (int k = 0; k < K; ++k) dY[k] = zs[k] - y0[k];
-  *dT = zs[K] - T0;
+  d = C > R(0) ? o * R(pow(C, o - R(1))) : R(0);
+  return pow(C, o);
 }
 
-// ------------------------------------ Newton fallback of FP32 domains (FP32)
-// Rates w_k (kg/(m^3 s)) and their Jacobian dw_k/dz_m in FP32, z = (Y, T);
-// k_f and k_r are taken as exponentials of their logarithms, so that neither
-// over- nor underflows on the way (k_r = exp(ln k_f - ln K_c)).
+// Rate constants of reaction j at T; k_r = 0 for an irreversible reaction.  FP32
+// takes them as exponentials of their logarithms, so that neither over- nor
+// underflows on the way.
 template <int K>
-__device__ __forceinline__ void rates_jacobian32(const Chem32<K>& c, const float* z, float rho,
-                                                 float* w, float (*dw)[K + 1]) {
-  constexpr int KK = K > 0 ? K : 1;
-  constexpr int n = K + 1;
-  const float T = z[K], invT = 1.f / T, lnT = logf(T);
-  float Cc[KK], dC[KK];
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    dC[k] = z[k] > 0.f ? rho * c.invM[k] : 0.f;
-    Cc[k] = z[k] > 0.f ? z[k] * dC[k] : 0.f;
-    w[k] = 0.f;
-#pragma unroll
-    for (int m = 0; m < n; ++m) dw[k][m] = 0.f;
-  }
-#pragma unroll
-  for (int j = 0; j < JMAX; ++j) {
-    if (!c.on[j]) continue;
-    const float lkf = c.lnA[j] + c.b[j] * lnT - c.EaR[j] * invT;
-    const float kf = expf(lkf);
-    const float dlkf = (c.EaR[j] * invT + c.b[j]) * invT;
-    float kr = 0.f, dlkr = dlkf;
-    if (c.rev[j]) {
-      const float lnKc = c.dS_R[j] - c.dH_R[j] * invT + c.dn[j] * (c.ln_pref_R - lnT);
-      kr = expf(lkf - lnKc);
-      dlkr = dlkf - (c.dH_R[j] * invT + c.dn[j]) * invT;
+__device__ __forceinline__ void rate_constants(const Chem64<K>& c, int j, double T, double invT,
+                                               double& kf, double& kr) {
+  kf = c.A[j] * exp(-c.EaR[j] * invT);
+  if (c.b[j] != 0.0) kf *= pow(T, c.b[j]);
+  kr = 0.0;
+  if (c.rev[j]) {
+    // 1 / K_c = exp(dH/(R T) - dS/R) (p_ref / (R T))^(-dn)
+    double lnKi = vfma(c.dH_R[j], invT, -c.dS_R[j]);
+    if (c.dn[j] == -0.5) {
+      kr = kf * exp(lnKi) * sqrt(c.pref_R * invT);
+    } else {
+      if (c.dn[j] != 0.0) lnKi = vfma(-c.dn[j], vsub(c.ln_pref_R, log(T)), lnKi);
+      kr = kf * exp(lnKi);
     }
-    float dq[K + 1];
+  }
+}
+template <int K>
+__device__ __forceinline__ void rate_constants(const Chem32<K>& c, int j, float T, float invT,
+                                               float& kf, float& kr) {
+  const float lnT = logf(T);
+  const float lkf = vfma(-c.EaR[j], invT, vfma(c.b[j], lnT, c.lnA[j]));
+  kf = expf(lkf);
+  kr = 0.f;
+  if (c.rev[j]) {
+    const float lnKc = vfma(c.dn[j], vsub(c.ln_pref_R, lnT), vfma(-c.dH_R[j], invT, c.dS_R[j]));
+    kr = expf(vsub(lkf, lnKc));
+  }
+}
+
+// One Newton iteration's rates: q_j in Real, its derivatives dq_j/dT (qT) and
+// along the reactions (Q[j][i]) in LA.  C_k = rho Y_k / M_k (in Real and in LA)
+// and dC_k = rho / M_k are 0 where Y_k <= 0.  Species of order 0 are skipped
+// (the orders are uniform).
+template <int K, int J, class Real, class LA, class Chem, class ChemL>
+__device__ __forceinline__ void reaction_rates(const Chem& c, const ChemL& cl, const Real* C,
+                                               const LA* CL, const LA* dC, Real T, Real invT,
+                                               Real* q, LA* qT, LA (*Q)[J]) {
+  const LA iT = LA(invT);
 #pragma unroll
-    for (int m = 0; m < n; ++m) dq[m] = 0.f;
+  for (int j = 0; j < J; ++j) {
+    q[j] = Real(0);
+    qT[j] = LA(0);
+#pragma unroll
+    for (int i = 0; i < J; ++i) Q[j][i] = LA(0);
+    if (!c.active(j)) continue;
+    Real kk[2];
+    rate_constants<K>(c, j, T, invT, kk[0], kk[1]);
 #pragma unroll
     for (int dir = 0; dir < 2; ++dir) {
       if (dir == 1 && !c.rev[j]) break;
-      const float kk = dir == 0 ? kf : -kr;
-      float Pw[KK], Dp[KK], pre[K + 1], suf[K + 1];
+      const Real k0 = dir == 0 ? kk[0] : -kk[1];
+      // d ln k / dT of this direction
+      LA dl = vmul(vfma(cl.EaR[j], iT, cl.b[j]), iT);
+      if (dir == 1) dl = vfma(-vfma(cl.dH_R[j], iT, cl.dn[j]), iT, dl);
+      // prefix / suffix products: the product without factor k, no division
+      LA Pw[K], pre[K], Dp[K], prodL = LA(k0), suf = LA(1);
+      Real prod = k0;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        const float o = dir == 0 ? c.order[j][k] : c.rorder[j][k];
-        const float C = Cc[k];
-        if (o == 1.f) { Pw[k] = C; Dp[k] = 1.f; }
-        else if (o == 0.f) { Pw[k] = 1.f; Dp[k] = 0.f; }
-        else if (o == 2.f) { Pw[k] = C * C; Dp[k] = 2.f * C; }
-        else if (o == 0.5f) {
-          const float sq = sqrtf(C);
-          Pw[k] = sq;
-          Dp[k] = sq > 0.f ? 0.5f / sq : 0.f;
-        } else {
-          Pw[k] = powf(C, o);
-          Dp[k] = C > 0.f ? o * powf(C, o - 1.f) : 0.f;
-        }
+        const auto o = dir == 0 ? cl.order[j][k] : cl.rorder[j][k];
+        if (o == LA(0)) continue;
+        pre[k] = prodL;
+        Pw[k] = conc_power(CL[k], o, Dp[k]);
+        prodL = vmul(prodL, Pw[k]);
+        if constexpr (sizeof(Real) != sizeof(LA))
+          prod = vmul(prod, conc_power(C[k], dir == 0 ? c.order[j][k] : c.rorder[j][k]));
       }
-      pre[0] = 1.f;
-      suf[K] = 1.f;
+      if constexpr (sizeof(Real) == sizeof(LA)) prod = prodL;
+      q[j] = vadd(q[j], prod);
+      qT[j] = vfma(prodL, dl, qT[j]);
 #pragma unroll
-      for (int k = 0; k < K; ++k) pre[k + 1] = pre[k] * Pw[k];
+      for (int k = K - 1; k >= 0; --k) {
+        const auto o = dir == 0 ? cl.order[j][k] : cl.rorder[j][k];
+        if (o == LA(0)) continue;
+        const LA d = vmul(vmul(pre[k], suf), vmul(Dp[k], dC[k]));
+        suf = vmul(suf, Pw[k]);
 #pragma unroll
-      for (int k = K - 1; k >= 0; --k) suf[k] = Pw[k] * suf[k + 1];
-      const float q = kk * pre[K];
-#pragma unroll
-      for (int k = 0; k < K; ++k) w[k] += c.Ms[j][k] * q;
-      dq[K] += q * (dir == 0 ? dlkf : dlkr);
-#pragma unroll
-      for (int m = 0; m < K; ++m) dq[m] += kk * (pre[m] * suf[m + 1]) * Dp[m] * dC[m];
+        for (int i = 0; i < J; ++i) Q[j][i] = vfma(d, cl.Ms[i][k], Q[j][i]);
+      }
     }
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-      for (int m = 0; m < n; ++m) dw[k][m] += c.Ms[j][k] * dq[m];
   }
 }
 
-// The backward-Euler step of chem_be_newton in FP32 for the cells that the
-// surrogate rejects in FP32 domains.  FP32 cannot hold the root to the FP64
-// integrator's 1e-13, so the unknown is the sub-step's increment d = z - zs
-// (small numbers keep their relative precision), the residual is
-// d - h F(zs + d), and the iteration stops once every update is below
-// 1e-5 |d_m| + 1e-6 |zs_m| (a few units in the last place of the FP32 field
-// that receives the increment).  On GB300 the FP64 pipe issues one warp
-// instruction every 16 cycles per SM, so the FP64 integrator's chain on a
-// short list of cells takes tens of microseconds; this one runs on the FP32
-// pipe and the special-function unit.
-template <int K>
-__device__ __forceinline__ void chem_be_newton32(const Chem32<K>& c, float T0, const float* Y0,
-                                                 float rho, float* dY, float* dT) {
-  constexpr int n = K + 1;
-  const float inv_rho = 1.f / rho;
-  float y0[K + 1], acc[K + 1];
+// The system of one iteration (see above): matrix A, right-hand side r and the
+// row a of dT.  h0 = h / rho in LA, rhs_j = hr q_j - xi_j, R.
+template <int K, int J, class LA, class ChemL>
+__device__ __forceinline__ void reaction_system(const ChemL& cl, LA hr, LA icp, const LA* q,
+                                                const LA* rhs, const LA* qT, const LA (*Q)[J], LA R,
+                                                LA (*A)[J], LA* r, LA* a) {
+  LA Hq = LA(0);
 #pragma unroll
-  for (int k = 0; k < K; ++k) y0[k] = Y0[k];
-  y0[K] = T0;
+  for (int j = 0; j < J; ++j) Hq = vfma(cl.H[j], q[j], Hq);
+  const LA w = vmul(vmul(hr, Hq), vmul(icp, icp));
 #pragma unroll
-  for (int m = 0; m < n; ++m) acc[m] = 0.f;
+  for (int i = 0; i < J; ++i) a[i] = vfma(-w, cl.cM[i], vmul(cl.H[i], icp));
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    r[j] = vfma(vmul(hr, qT[j]), R, rhs[j]);
+#pragma unroll
+    for (int i = 0; i < J; ++i)
+      A[j][i] = vfma(-hr, vfma(-qT[j], a[i], Q[j][i]), LA(i == j ? 1 : 0));
+  }
+}
+
+// z > 0 by its bits (a comparison would go through the FP64 pipe)
+__device__ __forceinline__ bool positive(double z) { return __double_as_longlong(z) > 0; }
+
+template <int K, int J, class LA, class ChemL>
+__device__ __forceinline__ void chem_be_newton(const Chem64<K>& c, const ChemL& cl, double T0,
+                                               const double* Y0, double rho, double* dY,
+                                               double* dT) {
+  const double inv_rho = 1.0 / rho;
+  double acc[K], accT = 0.0;  // increments of the finished sub-steps
   int ok = -1;
 #pragma unroll 1
   for (int nsub = 1; nsub <= 64 && ok != 0; nsub *= 2) {
-    float zs[K + 1];
 #pragma unroll
-    for (int m = 0; m < n; ++m) {
-      zs[m] = y0[m];
-      acc[m] = 0.f;
-    }
+    for (int k = 0; k < K; ++k) acc[k] = 0.0;
+    accT = 0.0;
     ok = 0;
-    const float h = c.dt / float(nsub), hr = h * inv_rho;
+    const double hr = c.dt / nsub * inv_rho;
+    const LA hrL = LA(hr);
 #pragma unroll 1
     for (int sub = 0; sub < nsub && ok == 0; ++sub) {
-      float d[K + 1];
+      const double Ts = vadd(T0, accT);
+      const LA tolT = LA(1e-13) * LA(Ts);
+      double xi[J], T = Ts, z[K];
 #pragma unroll
-      for (int m = 0; m < n; ++m) d[m] = 0.f;
+      for (int j = 0; j < J; ++j) xi[j] = 0.0;
+#pragma unroll
+      for (int k = 0; k < K; ++k) z[k] = sub == 0 ? Y0[k] : vadd(Y0[k], acc[k]);
       ok = -1;
 #pragma unroll 1
       for (int it = 0; it < 30; ++it) {
-        float z[K + 1], w[K + 1];
-#pragma unroll
-        for (int m = 0; m < n; ++m) z[m] = zs[m] + d[m];
-        if (!(z[K] > 0.f)) break;
-        float A[K + 1][K + 1];
-        rates_jacobian32<K>(c, z, rho, w, A);
-        float cp = 0.f, hw = 0.f;
+        double Cc[K], q[J], R = 0.0;
+        LA CL[K], dC[K], zL[K], cpL = LA(0), qT[J], Q[J][J], A[J][J], r[J], a[J], qL[J], rhs[J];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-          cp += z[k] * c.cp[k];
-          hw += c.hf[k] * w[k];
+          const bool pos = positive(z[k]);
+          zL[k] = LA(z[k]);
+          dC[k] = pos ? LA(rho) * cl.invM[k] : LA(0);
+          CL[k] = vmul(zL[k], dC[k]);
+          if constexpr (sizeof(LA) != 8) {
+            Cc[k] = 0.0;
+            if (c.used & (1 << k)) Cc[k] = pos ? vmul(z[k], vmul(rho, c.invM[k])) : 0.0;
+          }
+          cpL = vfma(zL[k], cl.cp[k], cpL);
         }
-        const float inv_rcp = inv_rho / cp;
-        const float hwc = hw * inv_rcp / cp;
-        float r[K + 1];
+        reaction_rates<K, J, double, LA>(c, cl, Cc, CL, dC, T, 1.0 / T, q, qT, Q);
+        if (it > 0) {  // R = 0 in the first iteration
+          double cp = 0.0, Hxi = 0.0;
 #pragma unroll
-        for (int m = 0; m < n; ++m) {
-          float dhw = 0.f;
+          for (int k = 0; k < K; ++k) cp = vfma(z[k], c.cp[k], cp);
 #pragma unroll
-          for (int k = 0; k < K; ++k) dhw += c.hf[k] * A[k][m];
-          float dFT = -dhw * inv_rcp;
-          if (m < K) dFT += hwc * c.cp[m];
-          A[K][m] = (m == K ? 1.f : 0.f) - h * dFT;
+          for (int j = 0; j < J; ++j) Hxi = vfma(c.H[j], xi[j], Hxi);
+          R = vsub(vsub(Ts, T), Hxi / cp);
         }
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+          qL[j] = LA(q[j]);
+          rhs[j] = LA(vfma(hr, q[j], -xi[j]));
+        }
+        reaction_system<K, J, LA>(cl, hrL, LA(1) / cpL, qL, rhs, qT, Q, LA(R), A, r, a);
+        if (!solve_pivoted<J, LA>(A, r)) break;
+        LA ar = LA(0);
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+          xi[j] = vadd(xi[j], double(r[j]));
+          ar = vfma(a[j], r[j], ar);
+        }
+        const double dTn = vsub(R, double(ar));
+        T = vadd(T, dTn);
+        // update test: species absolute, temperature relative to the start
+        const LA eT = fabs(LA(dTn));
+        bool bad = !(eT == eT), done = eT < tolT;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-          r[k] = -(d[k] - hr * w[k]);
+          LA e = LA(0);
 #pragma unroll
-          for (int m = 0; m < n; ++m) A[k][m] = (k == m ? 1.f : 0.f) - hr * A[k][m];
+          for (int j = 0; j < J; ++j) e = vfma(cl.Ms[j][k], r[j], e);
+          e = fabs(e);
+          if (!(e == e)) bad = true;
+          if (!(e < LA(1e-13))) done = false;
         }
-        r[K] = -(d[K] + h * hw * inv_rcp);
-        if (!solve_pivoted<K + 1, float>(A, r)) break;
-        bool bad = false, done = true;
+        if (bad || !positive(T)) break;
+        if (done) { ok = 0; break; }
 #pragma unroll
-        for (int m = 0; m < n; ++m) {
-          d[m] += r[m];
-          if (!(r[m] == r[m])) bad = true;
-          if (fabsf(r[m]) > 1e-5f * fabsf(d[m]) + 1e-6f * fabsf(zs[m])) done = false;
+        for (int k = 0; k < K; ++k) {
+          double d = 0.0;
+#pragma unroll
+          for (int j = 0; j < J; ++j) d = vfma(c.Ms[j][k], xi[j], d);
+          z[k] = vadd(vadd(Y0[k], acc[k]), d);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        double d = 0.0;
+#pragma unroll
+        for (int j = 0; j < J; ++j) d = vfma(c.Ms[j][k], xi[j], d);
+        acc[k] = vadd(acc[k], d);
+      }
+      accT = vadd(accT, vsub(T, Ts));
+    }
+  }
+  // differences of states, as a full iterate gives them: what the state cannot
+  // resolve is no increment
+#pragma unroll
+  for (int k = 0; k < K; ++k) dY[k] = vsub(vadd(Y0[k], acc[k]), Y0[k]);
+  *dT = accT;
+}
+
+// The same step in FP32 for the cells that the surrogate rejects in FP32
+// domains.  FP32 cannot hold the root to the FP64 integrator's 1e-13: the
+// unknowns are the sub-step's increments (small numbers keep their relative
+// precision), and the iteration stops once every update is below
+// 1e-5 |d_m| + 1e-6 |z_m| (a few units in the last place of the FP32 field
+// that receives the increment).
+template <int K, int J>
+__device__ __forceinline__ void chem_be_newton32(const Chem32<K>& c, float T0, const float* Y0,
+                                                 float rho, float* dY, float* dT) {
+  const float inv_rho = 1.f / rho;
+  float acc[K], accT = 0.f;
+  int ok = -1;
+#pragma unroll 1
+  for (int nsub = 1; nsub <= 64 && ok != 0; nsub *= 2) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[k] = 0.f;
+    accT = 0.f;
+    ok = 0;
+    const float hr = c.dt / float(nsub) * inv_rho;
+#pragma unroll 1
+    for (int sub = 0; sub < nsub && ok == 0; ++sub) {
+      const float Ts = vadd(T0, accT);
+      float xi[J], dTs = 0.f, d[K];
+#pragma unroll
+      for (int j = 0; j < J; ++j) xi[j] = 0.f;
+#pragma unroll
+      for (int k = 0; k < K; ++k) d[k] = 0.f;
+      ok = -1;
+#pragma unroll 1
+      for (int it = 0; it < 30; ++it) {
+        const float T = vadd(Ts, dTs);
+        if (!(T > 0.f)) break;
+        float Cc[K], dC[K], q[J], rhs[J], qT[J], Q[J][J], A[J][J], r[J], a[J], cp = 0.f;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const float z = vadd(vadd(Y0[k], acc[k]), d[k]);
+          dC[k] = z > 0.f ? rho * c.invM[k] : 0.f;
+          Cc[k] = vmul(z, dC[k]);
+          cp = vfma(z, c.cp[k], cp);
+        }
+        reaction_rates<K, J, float, float>(c, c, Cc, Cc, dC, T, 1.f / T, q, qT, Q);
+        const float icp = 1.f / cp;
+        float Hxi = 0.f;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+          Hxi = vfma(c.H[j], xi[j], Hxi);
+          rhs[j] = vfma(hr, q[j], -xi[j]);
+        }
+        const float R = vfma(-Hxi, icp, -dTs);
+        reaction_system<K, J, float>(c, hr, icp, q, rhs, qT, Q, R, A, r, a);
+        if (!solve_pivoted<J, float>(A, r)) break;
+        float dTn = R;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+          xi[j] = vadd(xi[j], r[j]);
+          dTn = vfma(-a[j], r[j], dTn);
+        }
+        dTs = vadd(dTs, dTn);
+        bool bad = !(dTn == dTn);
+        bool done = fabsf(dTn) <= 1e-5f * fabsf(dTs) + 1e-6f * Ts;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          float e = 0.f, s = 0.f;
+#pragma unroll
+          for (int j = 0; j < J; ++j) {
+            e = vfma(c.Ms[j][k], r[j], e);
+            s = vfma(c.Ms[j][k], xi[j], s);
+          }
+          d[k] = s;
+          if (!(e == e)) bad = true;
+          if (fabsf(e) > 1e-5f * fabsf(s) + 1e-6f * fabsf(vadd(Y0[k], acc[k]))) done = false;
         }
         if (bad) break;
         if (done) { ok = 0; break; }
       }
 #pragma unroll
-      for (int m = 0; m < n; ++m) {
-        zs[m] += d[m];
-        acc[m] += d[m];
-      }
+      for (int k = 0; k < K; ++k) acc[k] = vadd(acc[k], d[k]);
+      accT = vadd(accT, dTs);
     }
   }
 #pragma unroll
   for (int k = 0; k < K; ++k) dY[k] = acc[k];
-  *dT = acc[K];
+  *dT = accT;
 }
 
 // Moments read straight from global memory (the moments kernel, no staging).
@@ -1962,10 +1958,17 @@ step_persistent_kernel(const __grid_constant__ Params<Real, K> P, const State<Re
   }
 }
 
+// The chemistry's constants in the precision of the Newton matrix.
+template <class LA, class Real, int K>
+__device__ __forceinline__ const auto& chem_const(const Params<Real, K>& P) {
+  if constexpr (sizeof(LA) == 8) return P.c64;
+  else return P.c32;
+}
+
 // ------------------------------------------- chemistry pre-pass (implicit)
 // Per cell: backward-Euler Newton increments over the step at (T^n, Y^n,
 // rho^n), stored as the FD source terms rho* dY_k and rho* cp dT.
-template <int K, class Real, class Store>
+template <int K, int J, class Real, class Store>
 __global__ void __launch_bounds__(BLOCK)
 chem_implicit_kernel(const __grid_constant__ Params<Real, K> P, const State<Real, Store> S,
                      Real* __restrict__ src) {
@@ -1986,7 +1989,7 @@ chem_implicit_kernel(const __grid_constant__ Params<Real, K> P, const State<Real
     double Yd[KK], dY[KK], dT;
 #pragma unroll
     for (int k = 0; k < K; ++k) Yd[k] = double(Y[k]);
-    chem_be_newton<K, Real>(&P.c64, double(T), Yd, double(rho) * P.c64.rho_ref, dY, &dT);
+    chem_be_newton<K, J, Real>(P.c64, chem_const<Real>(P), double(T), Yd, double(rho) * P.c64.rho_ref, dY, &dT);
 #pragma unroll
     for (int k = 0; k < K; ++k) om[k] = rho * Real(dY[k]);
     omT = rho * mixture_cp(P, Y) * Real(dT);

@@ -229,8 +229,17 @@ Params<Real, K> make_params(const pflb_domain_desc& d, const pflb_mechanism& m, 
     P.c64.cp[k] = m.cp[k];
     P.c64.hf[k] = m.hf[k];
   }
+  for (int j = 0; j < P.J; ++j)
+    for (int k = 0; k < K; ++k) {
+      P.c64.H[j] += m.hf[k] * P.c64.Ms[j][k];
+      P.c64.cM[j] += m.cp[k] * P.c64.Ms[j][k];
+    }
   P.c64.p_ref = m.p_ref > 0 ? m.p_ref : 101325.0;
   P.c64.ln_pref_R = std::log(P.c64.p_ref / R_GAS);
+  P.c64.pref_R = P.c64.p_ref / R_GAS;
+  for (int j = 0; j < P.J; ++j)
+    for (int k = 0; k < K; ++k)
+      if (m.order[j][k] != 0.0 || (m.rev[j] && m.rorder[j][k] != 0.0)) P.c64.used |= 1 << k;
   P.c64.rho_ref = d.rho_ref;
   P.c64.dt = d.dt;
   {
@@ -245,6 +254,8 @@ Params<Real, K> make_params(const pflb_domain_desc& d, const pflb_mechanism& m, 
       f.dS_R[j] = float(c.dS_R[j]);
       f.dH_R[j] = float(c.dH_R[j]);
       f.rev[j] = c.rev[j];
+      f.H[j] = float(c.H[j]);
+      f.cM[j] = float(c.cM[j]);
       for (int k = 0; k < K; ++k) {
         f.order[j][k] = float(c.order[j][k]);
         f.rorder[j][k] = float(c.rorder[j][k]);

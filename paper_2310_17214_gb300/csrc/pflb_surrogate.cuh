@@ -240,7 +240,7 @@ chem_surrogate_kernel(const Params<Real, K> P, const State<Real, Store> S, Real*
   }
 }
 
-template <int K, class Real, class Store>
+template <int K, int J, class Real, class Store>
 __device__ __forceinline__ void fallback_cell(const Params<Real, K>& P, const State<Real, Store>& S,
                                               Real* __restrict__ src, const int c) {
   constexpr int KK = K > 0 ? K : 1;
@@ -253,7 +253,7 @@ __device__ __forceinline__ void fallback_cell(const Params<Real, K>& P, const St
   if constexpr (sizeof(Real) == 4) {
     // FP32 domains: the FP32 integrator (the fields it feeds are FP32)
     float dY[KK], dT;
-    chem_be_newton32<K>(P.c32, T, Y, rho * float(P.c64.rho_ref), dY, &dT);
+    chem_be_newton32<K, J>(P.c32, T, Y, rho * float(P.c64.rho_ref), dY, &dT);
 #pragma unroll
     for (int k = 0; k < K; ++k) src[(size_t)k * P.N + c] = rho * dY[k];
     src[(size_t)K * P.N + c] = rho * mixture_cp(P, Y) * dT;
@@ -261,7 +261,7 @@ __device__ __forceinline__ void fallback_cell(const Params<Real, K>& P, const St
     double Yd[KK], dY[KK], dT;
 #pragma unroll
     for (int k = 0; k < K; ++k) Yd[k] = double(Y[k]);
-    chem_be_newton<K, Real>(&P.c64, double(T), Yd, double(rho) * P.c64.rho_ref, dY, &dT);
+    chem_be_newton<K, J, Real>(P.c64, chem_const<Real>(P), double(T), Yd, double(rho) * P.c64.rho_ref, dY, &dT);
 #pragma unroll
     for (int k = 0; k < K; ++k) src[(size_t)k * P.N + c] = rho * Real(dY[k]);
     src[(size_t)K * P.N + c] = rho * mixture_cp(P, Y) * Real(dT);
@@ -274,14 +274,14 @@ __device__ __forceinline__ void fallback_cell(const Params<Real, K>& P, const St
 // hundred cells spreads over as many SMs as it has warps.
 constexpr int FALLBACK_BLOCK = 32;
 
-template <int K, class Real, class Store>
+template <int K, int J, class Real, class Store>
 __global__ void __launch_bounds__(FALLBACK_BLOCK)
 chem_fallback_kernel(const __grid_constant__ Params<Real, K> P, const State<Real, Store> S,
                      Real* __restrict__ src,
                      const int* __restrict__ fb_idx, const unsigned* __restrict__ fb_count) {
   const unsigned n = *fb_count;
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    fallback_cell<K>(P, S, src, fb_idx[i]);
+    fallback_cell<K, J>(P, S, src, fb_idx[i]);
 }
 
 // src (rho* dY_k, rho* cp dT) -> increments (dY_k, dT) of the current state.
