@@ -66,7 +66,7 @@ __device__ __forceinline__ void mma16816(float c[4], const uint32_t a[4], uint32
 }
 
 // Shared-memory copy of the network for training (weights in both layouts).
-struct SmemNet {
+struct __align__(16) SmemNet {
   __nv_bfloat16 wf[NPAD];
   __nv_bfloat16 wb[NPAD];
   float bias[NPB];
@@ -78,14 +78,6 @@ struct __align__(16) SmemFwd {
 };
 static_assert(NPAD * 2 % 16 == 0 && NPB * 4 % 16 == 0, "16-byte copies of the network");
 
-__device__ __forceinline__ void load_words(uint32_t* dst, const uint32_t* src, int words) {
-  for (int i = threadIdx.x; i < words; i += blockDim.x) dst[i] = src[i];
-}
-__device__ __forceinline__ void load_net(SmemNet& s, const Net& n) {
-  load_words(reinterpret_cast<uint32_t*>(s.wf), reinterpret_cast<const uint32_t*>(n.wf), NPAD / 2);
-  load_words(reinterpret_cast<uint32_t*>(s.wb), reinterpret_cast<const uint32_t*>(n.wb), NPAD / 2);
-  load_words(reinterpret_cast<uint32_t*>(s.bias), reinterpret_cast<const uint32_t*>(n.bias), NPB);
-}
 // 16-byte copy of NV vectors by a block of BT threads, every load issued
 // before the first store (a block loads the network once; a copy that waits
 // on each load in turn costs microseconds per block)
