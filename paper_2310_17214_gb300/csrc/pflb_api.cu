@@ -666,7 +666,9 @@ int pflb_get_fields(pflb_domain* d, unsigned mask, void* dst, size_t bytes, int 
   char* p = out;
   auto put_real = [&](const void* srcp, size_t cnt) -> cudaError_t {
     cudaError_t e;
-    if (d->real_sz == 8) e = esz == 8 ? convert<double, double>(srcp, p, cnt, d->stream)
+    if (d->real_sz == esz)
+      e = cudaMemcpyAsync(p, srcp, cnt * esz, cudaMemcpyDeviceToDevice, d->stream);
+    else if (d->real_sz == 8) e = esz == 8 ? convert<double, double>(srcp, p, cnt, d->stream)
                                       : convert<double, float>(srcp, p, cnt, d->stream);
     else e = esz == 8 ? convert<float, double>(srcp, p, cnt, d->stream)
                       : convert<float, float>(srcp, p, cnt, d->stream);
@@ -678,20 +680,16 @@ int pflb_get_fields(pflb_domain* d, unsigned mask, void* dst, size_t bytes, int 
   if (e == cudaSuccess && (mask & PFLB_FIELD_Y)) e = put_real(d->B.Y[d->cur], n * d->K);
   if (e == cudaSuccess && (mask & PFLB_FIELD_TS)) e = put_real(d->B.Ts[d->cur], n);
   if (e == cudaSuccess && (mask & (PFLB_FIELD_U | PFLB_FIELD_RHO | PFLB_FIELD_PH))) {
-    double* mom = nullptr;
-    e = cudaMallocAsync((void**)&mom, n * (d->dim + 2) * sizeof(double), d->stream);
-    if (e == cudaSuccess) e = d->L->moments(d->B, d->cur, mom, mom + n * d->dim,
-                                            mom + n * (d->dim + 1), d->stream);
-    auto put_d = [&](const double* srcp, size_t cnt) {
-      cudaError_t ee = esz == 8 ? convert<double, double>(srcp, p, cnt, d->stream)
-                                : convert<double, float>(srcp, p, cnt, d->stream);
+    auto take = [&](unsigned field, size_t cnt) -> void* {
+      if (!(mask & field)) return nullptr;
+      void* at = p;
       p += cnt * esz;
-      return ee;
+      return at;
     };
-    if (e == cudaSuccess && (mask & PFLB_FIELD_U)) e = put_d(mom, n * d->dim);
-    if (e == cudaSuccess && (mask & PFLB_FIELD_RHO)) e = put_d(mom + n * d->dim, n);
-    if (e == cudaSuccess && (mask & PFLB_FIELD_PH)) e = put_d(mom + n * (d->dim + 1), n);
-    if (mom) cudaFreeAsync(mom, d->stream);
+    void* u = take(PFLB_FIELD_U, n * d->dim);
+    void* rho = take(PFLB_FIELD_RHO, n);
+    void* ph = take(PFLB_FIELD_PH, n);
+    e = d->L->moments(d->B, d->cur, u, rho, ph, esz == 8, d->stream);
   }
   if (e == cudaSuccess && (mask & PFLB_FIELD_G)) {
     Weights W;
@@ -726,9 +724,9 @@ int pflb_get_fields(pflb_domain* d, unsigned mask, void* dst, size_t bytes, int 
     e = cudaMemcpyAsync(dst, out, need * esz, cudaMemcpyDeviceToHost, d->stream);
   if (where == PFLB_HOST && out) cudaFreeAsync(out, d->stream);
   CK(d, e);
-  CK(d, cudaStreamSynchronize(d->stream));
   DevScalars h;
-  CK(d, cudaMemcpy(&h, d->B.scal, sizeof(h), cudaMemcpyDeviceToHost));
+  CK(d, cudaMemcpyAsync(&h, d->B.scal, sizeof(h), cudaMemcpyDeviceToHost, d->stream));
+  CK(d, cudaStreamSynchronize(d->stream));
   if (h.status != 0) return fail(d, h.status, "%s", status_message(h.status));
   return PFLB_OK;
 }
@@ -816,9 +814,15 @@ int pflb_set_state(pflb_domain* d, const void* src, size_t bytes, int where) {
   if (bytes < state_bytes(d)) return fail(d, PFLB_ERR_ARG, "source too small");
   if (where != PFLB_HOST && where != PFLB_DEVICE) return fail(d, PFLB_ERR_ARG, "bad where");
   CK(d, cudaSetDevice(d->desc.device));
-  StateHeader h;
-  if (where == PFLB_HOST) std::memcpy(&h, src, sizeof(h));
-  else CK(d, cudaMemcpy(&h, src, sizeof(h), cudaMemcpyDeviceToHost));
+  // the header and, for the step count, the scalars behind it
+  struct Front {
+    StateHeader h;
+    DevScalars sc;
+  } front;
+  static_assert(sizeof(Front) == sizeof(StateHeader) + sizeof(DevScalars), "packed front");
+  if (where == PFLB_HOST) std::memcpy(&front, src, sizeof(front));
+  else CK(d, cudaMemcpy(&front, src, sizeof(front), cudaMemcpyDeviceToHost));
+  const StateHeader& h = front.h;
   if (std::memcmp(h.magic, "PFLBSTv3", 8) != 0 || h.dim != d->dim || h.nx != d->desc.nx ||
       h.ny != d->desc.ny || h.nz != d->desc.nz || h.precision != d->desc.precision ||
       h.K != d->K || h.Ts_field != d->desc.Ts_field || h.N != d->N)
@@ -833,10 +837,7 @@ int pflb_set_state(pflb_domain* d, const void* src, size_t bytes, int where) {
   });
   if (rc != PFLB_OK) return rc;
   // the step count of the restored state (a moving solid's phase field)
-  DevScalars sc;
-  if (where == PFLB_HOST) std::memcpy(&sc, in + sizeof(h), sizeof(sc));
-  else CK(d, cudaMemcpy(&sc, in + sizeof(h), sizeof(sc), cudaMemcpyDeviceToHost));
-  if (d->L) CK(d, d->L->set_step(d->B, sc.step, d->stream));
+  if (d->L) CK(d, d->L->set_step(d->B, front.sc.step, d->stream));
   return PFLB_OK;
 }
 

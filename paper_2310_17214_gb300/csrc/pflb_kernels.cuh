@@ -2171,10 +2171,11 @@ init_kernel(const Params<Real, K> P, const State<Real, Store> S, const Real* __r
 
 // --------------------------------------------------- moments (get_fields)
 // u, rho and sum g that the next step sees (pull + boundary rules + drag).
-template <int DIM, int K, class Real, class Store>
+// Written in the caller's type Out; a null output is skipped.
+template <int DIM, int K, class Real, class Store, class Out>
 __global__ void __launch_bounds__(BLOCK)
-moments_kernel(const Params<Real, K> P, const State<Real, Store> S, double* __restrict__ u_out,
-               double* __restrict__ rho_out, double* __restrict__ ph_out) {
+moments_kernel(const Params<Real, K> P, const State<Real, Store> S, Out* __restrict__ u_out,
+               Out* __restrict__ rho_out, Out* __restrict__ ph_out) {
   using L = Lattice<DIM>;
   constexpr int Q = L::Q;
   constexpr int KK = Params<Real, K>::KK;
@@ -2211,9 +2212,10 @@ moments_kernel(const Params<Real, K> P, const State<Real, Store> S, double* __re
   }
   Real sg = 0;
   for (int i = 0; i < Q; ++i) sg += gin[i];
-  for (int a = 0; a < DIM; ++a) u_out[(size_t)a * P.N + c] = double(u[a]);
-  rho_out[c] = double(rho);
-  ph_out[c] = double(sg);
+  if (u_out)
+    for (int a = 0; a < DIM; ++a) u_out[(size_t)a * P.N + c] = Out(u[a]);
+  if (rho_out) rho_out[c] = Out(rho);
+  if (ph_out) ph_out[c] = Out(sg);
 }
 
 // ------------------------------------------------- diagnostics (on demand)

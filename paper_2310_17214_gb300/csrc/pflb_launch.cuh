@@ -93,7 +93,9 @@ struct Launcher {
                            cudaStream_t st) = 0;
   // nsteps fused steps; `cur` flips once per step
   virtual cudaError_t step(Buffers& B, int& cur, int nsteps, cudaStream_t st) = 0;
-  virtual cudaError_t moments(const Buffers& B, int cur, double* u, double* rho, double* ph,
+  // u, rho, P_h of the current state into arrays of doubles (f64) or floats; null
+  // outputs are skipped
+  virtual cudaError_t moments(const Buffers& B, int cur, void* u, void* rho, void* ph, bool f64,
                               cudaStream_t st) = 0;
   // combine deferred partials of the last step into the scalar state
   virtual cudaError_t finalize(Buffers& B, cudaStream_t st) = 0;
@@ -484,6 +486,7 @@ struct LauncherImpl final : Launcher {
     } else {
       surr = a;
       has_surr = true;
+      ++surr_version;
       return true;
     }
   }
@@ -825,12 +828,67 @@ struct LauncherImpl final : Launcher {
   // after two plain steps every launch argument repeats every second step
   // (the ping-pong buffers, the reduction's parity and block count), and a
   // graph launch of the pair costs one launch instead of one per kernel
-  // (the small domains are launch-bound).  Not for moving solids, whose
-  // phase kernel takes the step number as an argument.
+  // (the small domains are launch-bound).  The graph of each starting parity is
+  // kept for later calls of this domain (capturing and instantiating one takes
+  // about as long as ten steps of a small domain); its arguments are the
+  // domain's own buffers and parameters, which live as long as this object, and
+  // whatever else a launch depends on is compared before a kept graph is used.
+  // Not for moving solids, whose phase kernel takes the step number as an
+  // argument.
   static constexpr int kGraphMinSteps = 32;
   cudaStream_t cap_st = nullptr;  // capture stream, created on first use
+  struct PairGraph {
+    cudaGraphExec_t exec = nullptr;
+    int kernel = -1;
+    long long wait_limit = 0;
+    int surr_version = 0;
+    int pending = 0, last_parity = 0;  // bookkeeping a pair starts from
+    long long last_nb = 0;
+  } pair[2];
+  int surr_version = 0;
   ~LauncherImpl() override {
+    for (PairGraph& g : pair)
+      if (g.exec) cudaGraphExecDestroy(g.exec);
     if (cap_st) cudaStreamDestroy(cap_st);
+  }
+
+  // The graph of two steps from the current bookkeeping; null if capture is
+  // refused (the bookkeeping is as before either way).
+  cudaGraphExec_t pair_graph(Buffers& B, int cur) {
+    PairGraph& G = pair[cur];
+    if (G.exec && G.kernel == resolved() && G.wait_limit == wait_limit &&
+        G.surr_version == surr_version && G.pending == B.pending &&
+        G.last_parity == B.last_parity && G.last_nb == B.last_nb)
+      return G.exec;
+    if (G.exec) cudaGraphExecDestroy(G.exec);
+    G = PairGraph{nullptr, resolved(), wait_limit, surr_version, B.pending, B.last_parity, B.last_nb};
+    if (!cap_st && cudaStreamCreateWithFlags(&cap_st, cudaStreamNonBlocking) != cudaSuccess) {
+      cap_st = nullptr;
+      cudaGetLastError();
+      return nullptr;
+    }
+    const Buffers B0 = B;
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(cap_st, cudaStreamCaptureModeRelaxed);
+    if (e == cudaSuccess) {
+      int c = cur;
+      cudaError_t e1 = one_step(B, c, cap_st);
+      if (e1 == cudaSuccess) e1 = one_step(B, c, cap_st);
+      e = cudaStreamEndCapture(cap_st, &g);
+      if (e == cudaSuccess) e = e1;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&G.exec, g, 0);
+    // a pair has to leave the bookkeeping it started from, or it cannot repeat
+    const bool repeats = B.pending == B0.pending && B.last_parity == B0.last_parity &&
+                         B.last_nb == B0.last_nb;
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess || !repeats) {
+      cudaGetLastError();
+      if (e == cudaSuccess) cudaGraphExecDestroy(G.exec);
+      G.exec = nullptr;
+    }
+    B = B0;
+    return G.exec;
   }
 
   cudaError_t step(Buffers& B, int& cur, int nsteps, cudaStream_t st) override {
@@ -846,45 +904,13 @@ struct LauncherImpl final : Launcher {
         e = one_step(B, cur, st);
         if (e != cudaSuccess) return e;
       }
-      if (!cap_st) {
-        e = cudaStreamCreateWithFlags(&cap_st, cudaStreamNonBlocking);
-        if (e != cudaSuccess) return e;
-      }
-      const int cur0 = cur;
-      const long long nstep0 = B.nstep;
-      const int pending0 = B.pending, parity0 = B.last_parity;
-      const long long last_nb0 = B.last_nb;
-      cudaGraph_t g = nullptr;
-      cudaGraphExec_t x = nullptr;
-      e = cudaStreamBeginCapture(cap_st, cudaStreamCaptureModeRelaxed);
-      if (e == cudaSuccess) {
-        cudaError_t e1 = one_step(B, cur, cap_st);
-        if (e1 == cudaSuccess) e1 = one_step(B, cur, cap_st);
-        e = cudaStreamEndCapture(cap_st, &g);
-        if (e == cudaSuccess) e = e1;
-      }
-      if (e == cudaSuccess) e = cudaGraphInstantiate(&x, g, 0);
-      if (e == cudaSuccess) {
-        // the capture advanced the bookkeeping by the pair the first launch runs
-        const int pairs = (nsteps - n) / 2;
-        for (int q = 0; q < pairs && e == cudaSuccess; ++q) {
+      if (cudaGraphExec_t x = pair_graph(B, cur)) {
+        for (; n + 2 <= nsteps; n += 2) {
           e = cudaGraphLaunch(x, st);
-          if (q > 0) B.nstep += 2;
+          if (e != cudaSuccess) return e;
+          B.nstep += 2;
         }
-        n += 2 * pairs;
-      } else {
-        // capture refused: undo its bookkeeping, step without a graph
-        cudaGetLastError();
-        cur = cur0;
-        B.nstep = nstep0;
-        B.pending = pending0;
-        B.last_parity = parity0;
-        B.last_nb = last_nb0;
-        e = cudaSuccess;
       }
-      if (x) cudaGraphExecDestroy(x);
-      if (g) cudaGraphDestroy(g);
-      if (e != cudaSuccess) return e;
     }
     for (; n < nsteps; ++n) {
       e = one_step(B, cur, st);
@@ -899,9 +925,16 @@ struct LauncherImpl final : Launcher {
     B.pending = 0;
     return cudaGetLastError();
   }
-  cudaError_t moments(const Buffers& B, int cur, double* u, double* rho, double* ph,
+  cudaError_t moments(const Buffers& B, int cur, void* u, void* rho, void* ph, bool f64,
                       cudaStream_t st) override {
-    moments_kernel<DIM, K, Real, Store><<<blocks(), BLOCK, 0, st>>>(P, state(B, cur), u, rho, ph);
+    if (f64)
+      moments_kernel<DIM, K, Real, Store, double><<<blocks(), BLOCK, 0, st>>>(
+          P, state(B, cur), static_cast<double*>(u), static_cast<double*>(rho),
+          static_cast<double*>(ph));
+    else
+      moments_kernel<DIM, K, Real, Store, float><<<blocks(), BLOCK, 0, st>>>(
+          P, state(B, cur), static_cast<float*>(u), static_cast<float*>(rho),
+          static_cast<float*>(ph));
     return cudaGetLastError();
   }
   float g_scale() const override { return float(P.g_scale); }
