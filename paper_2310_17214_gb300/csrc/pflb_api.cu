@@ -1252,7 +1252,8 @@ int pflb_create_batch(pflb_domain** domains, int n, pflb_batch** out) {
                           ((D.ny + batch_ty(cfg) - 1) / batch_ty(cfg));
       if (t > domains[i]->B.slots) return bad(PFLB_ERR_STATE, "reduction slots too few");
       if ((long long)tb[i] + t > (1LL << 30)) return bad(PFLB_ERR_ARG, "batch too large");
-      tb[i + 1] = tb[i] + (int)t;
+      const int run = b->L0->batch_run();  // tiles a block draws at a time
+      tb[i + 1] = tb[i] + (int)((t + run - 1) / run);
     }
     if (cudaMalloc((void**)&b->tile_begin[cfg], (n + 1) * sizeof(int)) != cudaSuccess)
       return bad(PFLB_ERR_OOM, "device allocation failed");

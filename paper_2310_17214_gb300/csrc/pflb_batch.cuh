@@ -3,16 +3,22 @@
 // Every domain keeps its own arrays; the batch holds a device work list with
 // one entry per domain (its lattice-unit parameters, the two ping-pong views
 // of its state, its P0 mode) and, per tile shape, the prefix sums of the
-// domains' tile counts.  A launch is a grid-stride loop over the global tile
-// index: a block finds the tile's domain by binary search, copies that
-// domain's parameters into shared memory when it changes domain, and runs the
-// same per-tile code as the single-domain step.  Tiles are handed out by an
-// atomic counter (one per launch parity; each launch clears the other one
-// for the next launch), so blocks that draw cheap tiles take more of them
-// and no SM idles at the end.  Each domain's reduction
-// slots are its tile indices, and the last tile of a domain to finish
-// combines them at once, so a batch step leaves no deferred work behind and
-// every domain's P0 is current for the next launch.
+// domains' counts of runs of BATCH_RUN consecutive tiles.  A launch is a
+// resident grid that draws runs from an atomic counter (one per launch parity;
+// each launch clears the other one for the next launch), so blocks that draw
+// cheap tiles take more of them and no SM idles at the end.  A block finds a
+// run's domain by binary search, copies that domain's parameters into shared
+// memory when it changes domain, and runs the same per-tile code as the
+// single-domain step.  Each domain's reduction slots are its tile indices.  A
+// block makes a run's slots visible and counts them once, and the block whose
+// count completes a domain combines its slots at once, so a batch step leaves
+// no deferred work behind and every domain's P0 is current for the next launch.
+//
+// Runs of tiles: the blocks advance through the tiles side by side, so with
+// single tiles nearly every draw changed domain (a search, a copy of the
+// parameters, two barriers) and every tile paid a fence.  48 beds: 288 us a step
+// drawing one tile at a time, 257 with runs of 4; runs of 2 and 8 up to 3 %
+// slower than 4.
 #pragma once
 
 #include "pflb_half.cuh"
@@ -30,11 +36,13 @@ template <class Real> struct BatchShape<Real, 2> { using T = Tile<typename VecOf
 __host__ __device__ constexpr int batch_tx(int cfg) { return cfg == 2 ? 64 : 32; }
 __host__ __device__ constexpr int batch_ty(int cfg) { return cfg == 0 ? 8 : (cfg == 1 ? 16 : 4); }
 
+constexpr int BATCH_RUN = 4;
+
 template <int K, class Real, class T_>
 __global__ void __launch_bounds__(T_::NT, (MinBlocks<K, T_>::value))
 batch_step_kernel(const BatchDom<K, Real, Real>* __restrict__ doms,
-                  const int* __restrict__ tile_begin, int ndom, int flip,
-                  unsigned* __restrict__ tile_ctr) {
+                  const int* __restrict__ run_begin, int ndom, int flip,
+                  unsigned* __restrict__ run_ctr) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* pl = reinterpret_cast<Real*>(smem_raw);
   __shared__ double red_sh[96];
@@ -43,23 +51,22 @@ batch_step_kernel(const BatchDom<K, Real, Real>* __restrict__ doms,
   __shared__ int p0c_sh;
   __shared__ int next_sh[2];
 
-  const int total = tile_begin[ndom];
-  unsigned* ctr = tile_ctr + flip;
+  const int total = run_begin[ndom];
   if (threadIdx.x == 0) {
-    if (blockIdx.x == 0) tile_ctr[flip ^ 1] = 0u;  // the next launch's counter
-    next_sh[0] = (int)atomicAdd(ctr, 1u);
+    if (blockIdx.x == 0) run_ctr[flip ^ 1] = 0u;  // the next launch's counter
+    next_sh[0] = (int)atomicAdd(run_ctr + flip, 1u);
   }
   __syncthreads();
-  int cur_dom = -1, par = 0;
-  for (int t = next_sh[0]; t < total; t = next_sh[par]) {
-    // domain of tile t: the last d with tile_begin[d] <= t
+  int dom = -1, par = 0;
+  for (int r = next_sh[0]; r < total; r = next_sh[par]) {
+    // domain of run r: the last d with run_begin[d] <= r
     int lo = 0, hi = ndom - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (__ldg(tile_begin + mid) <= t) lo = mid;
+      if (__ldg(run_begin + mid) <= r) lo = mid;
       else hi = mid - 1;
     }
-    if (lo != cur_dom) {
+    if (lo != dom) {
       __syncthreads();  // the previous tile is done with the shared copies
       const BatchDom<K, Real, Real>& D = doms[lo];
       constexpr int PW = sizeof(Params<Real, K>) / 4;
@@ -71,18 +78,24 @@ batch_step_kernel(const BatchDom<K, Real, Real>* __restrict__ doms,
         p0c_sh = D.p0_closed;
       }
       __syncthreads();
-      cur_dom = lo;
+      dom = lo;
     }
-    // draw the next tile now; the tile's staging barrier publishes it
+    // draw the next run now; a tile's staging barrier publishes it
     par ^= 1;
-    if (threadIdx.x == 0) next_sh[par] = (int)atomicAdd(ctr, 1u);
-    const int lt = t - tile_begin[lo];
-    const int nbx = (Psh.nx + T_::TX - 1) / T_::TX;
-    double sI, sIn, sOut;
-    step_tile<K, Real, T_>(Psh, Ssh, lt % nbx, lt / nbx, pl, red_sh, sI, sIn, sOut);
-    const unsigned nb = (unsigned)(tile_begin[lo + 1] - tile_begin[lo]);
-    publish_partials_at(sI, sIn, sOut, Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0,
-                        Psh.eos_c, Psh.inv_rho_ref, (unsigned)lt, nb, true);
+    if (threadIdx.x == 0) next_sh[par] = (int)atomicAdd(run_ctr + flip, 1u);
+    const int first = (r - __ldg(run_begin + lo)) * BATCH_RUN;
+#pragma unroll 1
+    for (int i = 0; i < BATCH_RUN; ++i) {
+      const int nbx = (Psh.nx + T_::TX - 1) / T_::TX;
+      if (first + i >= nbx * ((Psh.ny + T_::TY - 1) / T_::TY)) break;
+      double sI, sIn, sOut, sF;
+      step_tile<K, Real, T_>(Psh, Ssh, (first + i) % nbx, (first + i) / nbx, pl, red_sh, sI, sIn,
+                             sOut, sF);
+      write_partials(sI, sIn, sOut, Ssh.partials, (unsigned)(first + i));
+    }
+    const int nb = ((Psh.nx + T_::TX - 1) / T_::TX) * ((Psh.ny + T_::TY - 1) / T_::TY);
+    count_partials(Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0, Psh.eos_c,
+                   Psh.inv_rho_ref, (unsigned)min(BATCH_RUN, nb - first), (unsigned)nb);
   }
 }
 

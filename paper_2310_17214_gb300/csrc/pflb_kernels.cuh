@@ -1039,9 +1039,11 @@ __device__ __forceinline__ double warp_sum(V v) {
 // The three sums of a tile (I, and the two fluxes when `bc` holds) with one
 // barrier, grouped exactly as block_sum; results valid in thread 0.  `sh`
 // holds 96 doubles and is free again after the block's next barrier.
+// With `df` a fourth sum (of doubles: the fuel consumed), `sh` then 128 doubles.
 template <class V, class Real>
-__device__ __forceinline__ void block_sum3(V a, Real b, Real c, bool bc, double* sh,
-                                           double& ra, double& rb, double& rc) {
+__device__ __forceinline__ void block_sum4(V a, Real b, Real c, bool bc, double d, bool df,
+                                           double* sh, double& ra, double& rb, double& rc,
+                                           double& rd) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const double wa = warp_sum(a);
   const double wb = bc ? warp_sum(b) : 0.0, wc = bc ? warp_sum(c) : 0.0;
@@ -1050,8 +1052,12 @@ __device__ __forceinline__ void block_sum3(V a, Real b, Real c, bool bc, double*
     sh[32 + wid] = wb;
     sh[64 + wid] = wc;
   }
+  if (df) {
+    d = warp_sum(d);
+    if (lane == 0) sh[96 + wid] = d;
+  }
   __syncthreads();
-  ra = rb = rc = 0.0;
+  ra = rb = rc = rd = 0.0;
   if (wid == 0) {
     const bool in = lane < (int)(blockDim.x >> 5);
     double x = in ? sh[lane] : 0.0, y = in ? sh[32 + lane] : 0.0, z = in ? sh[64 + lane] : 0.0;
@@ -1064,9 +1070,21 @@ __device__ __forceinline__ void block_sum3(V a, Real b, Real c, bool bc, double*
     ra = x;
     rb = bc ? y : 0.0;
     rc = bc ? z : 0.0;
+    if (df) {
+      double f = in ? sh[96 + lane] : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) f += __shfl_down_sync(0xffffffffu, f, o);
+      rd = f;
+    }
   }
 }
 
+template <class V, class Real>
+__device__ __forceinline__ void block_sum3(V a, Real b, Real c, bool bc, double* sh,
+                                           double& ra, double& rb, double& rc) {
+  double none = 0.0, rd;
+  block_sum4(a, b, c, bc, none, false, sh, ra, rb, rc, rd);
+}
 template <class Real>
 __device__ __forceinline__ double block_sum(Real v, double* sh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1100,70 +1118,119 @@ __device__ __forceinline__ double block_sum(Real v, double* sh) {
   return r;
 }
 
-// Combine the per-block partials (I, inlet flux, outlet flux) of one step in
-// a fixed order (lane-strided sums, then a fixed shuffle tree) and update the
-// scalar state: the P0 closure when the domain is closed, the diagnostics and
-// the per-step constants the cells of the next step read.  Run by one warp.
+// The scalar state after a step (or, is_init, of a new one) from its sums, by
+// one thread: the P0 closure when the domain is closed, the diagnostics and the
+// per-step constants the cells of the next step read.  With the inlet feedback
+// (feed_c > 0, Sec. 4.4.1) the fuel the step consumed, phi_f (-omega_k) of its
+// input state, sets the inlet peak speed of the next step, u_in = fuel feed_c /
+// P0, held in [0, 0.3].
+__device__ __forceinline__ void apply_sums(double I, double in, double out, double fuel,
+                                           DevScalars* scal, int p0_closed, bool is_init,
+                                           double init_P0, double eos_c, double inv_rho_ref,
+                                           double feed_c) {
+  double P0, P0p;
+  if (is_init) {
+    P0 = P0p = init_P0;
+    scal->mass = init_P0 * I * eos_c;
+    scal->flux_in = scal->flux_out = 0;
+    scal->flux_in_sum = scal->flux_out_sum = 0;
+    scal->step = 0;
+    scal->status = 0;
+  } else {
+    P0p = scal->P0;
+    P0 = P0p;
+    if (p0_closed) P0 = scal->mass / (I * eos_c);
+    scal->flux_in = in;
+    scal->flux_out = out;
+    scal->flux_in_sum += in;
+    scal->flux_out_sum += out;
+    scal->step += 1;
+    // latch only the first failure (a timeout is not overwritten)
+    if (scal->status == 0 && (!(I == I) || !(P0 == P0) || I <= 0.0)) scal->status = -5;
+  }
+  scal->P0_prev = P0p;
+  scal->P0 = P0;
+  scal->I = I;
+  scal->mass_now = P0 * I * eos_c;
+  scal->dlnP0 = (P0 - P0p) / P0;
+  scal->dP0r = (P0 - P0p) * inv_rho_ref;
+  scal->P0_f = float(P0);
+  scal->dlnP0_f = float(scal->dlnP0);
+  scal->dP0r_f = float(scal->dP0r);
+  if (feed_c > 0.0) {
+    double u = fuel * feed_c / P0;
+    u = u > 0.3 ? 0.3 : (u > 0.0 ? u : 0.0);  // NaN -> 0
+    scal->fuel = fuel;
+    scal->u_in = u;
+    scal->u_in_f = float(u);
+  }
+}
+
+// Sums over the slots b = first, first + stride, ... in that order (I, inlet and
+// outlet flux, fuel), eight slots in flight: a short list waits for memory once.
+__device__ __forceinline__ void sum_slots(const double* partials, unsigned nb, unsigned first,
+                                          unsigned stride, double v[4]) {
+  v[0] = v[1] = v[2] = v[3] = 0.0;
+  for (unsigned b = first; b < nb; b += 8 * stride) {
+    double2 a[8], c[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const double2* p =
+          reinterpret_cast<const double2*>(partials + 4 * (size_t)(b + q * stride));
+      const bool in = b + q * stride < nb;
+      a[q] = in ? __ldcg(p) : make_double2(0.0, 0.0);
+      c[q] = in ? __ldcg(p + 1) : make_double2(0.0, 0.0);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      v[0] += a[q].x;
+      v[1] += a[q].y;
+      v[2] += c[q].x;
+      v[3] += c[q].y;
+    }
+  }
+}
+
+// Combine the per-block partials of one step in a fixed order (strided sums,
+// then a fixed shuffle tree) and update the scalar state: by one warp.
 __device__ __forceinline__ void combine_partials(const double* partials, unsigned nb,
                                                  DevScalars* scal, int p0_closed, bool is_init,
                                                  double init_P0, double eos_c,
-                                                 double inv_rho_ref) {
+                                                 double inv_rho_ref, double feed_c = 0.0) {
   const int lane = threadIdx.x & 31;
-  double v0 = 0, v1 = 0, v2 = 0;
-  unsigned b = lane;
-  for (; b + 96 < nb; b += 128) {
-    const double a0 = __ldcg(partials + 4 * b), a1 = __ldcg(partials + 4 * (b + 32));
-    const double a2 = __ldcg(partials + 4 * (b + 64)), a3 = __ldcg(partials + 4 * (b + 96));
-    const double f0 = __ldcg(partials + 4 * b + 1), f1 = __ldcg(partials + 4 * (b + 32) + 1);
-    const double f2 = __ldcg(partials + 4 * (b + 64) + 1), f3 = __ldcg(partials + 4 * (b + 96) + 1);
-    const double o0 = __ldcg(partials + 4 * b + 2), o1 = __ldcg(partials + 4 * (b + 32) + 2);
-    const double o2 = __ldcg(partials + 4 * (b + 64) + 2), o3 = __ldcg(partials + 4 * (b + 96) + 2);
-    v0 += a0; v0 += a1; v0 += a2; v0 += a3;
-    v1 += f0; v1 += f1; v1 += f2; v1 += f3;
-    v2 += o0; v2 += o1; v2 += o2; v2 += o3;
-  }
-  for (; b < nb; b += 32) {
-    v0 += __ldcg(partials + 4 * b + 0);
-    v1 += __ldcg(partials + 4 * b + 1);
-    v2 += __ldcg(partials + 4 * b + 2);
-  }
+  double v[4];
+  sum_slots(partials, nb, lane, 32, v);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v0 += __shfl_down_sync(0xffffffffu, v0, o);
-    v1 += __shfl_down_sync(0xffffffffu, v1, o);
-    v2 += __shfl_down_sync(0xffffffffu, v2, o);
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+  if (lane == 0)
+    apply_sums(v[0], v[1], v[2], v[3], scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref,
+               feed_c);
+}
+
+// The same for a fixed P0 by a whole block (every thread calls it; `sh` holds
+// 96 doubles and is free again after the block's next barrier): one warp takes
+// 25 us over the 4,096 slots of a 2048 x 512 domain, and as the first block's
+// first warp it held up small launches.
+__device__ __forceinline__ void combine_partials_block(const double* partials, unsigned nb,
+                                                       DevScalars* scal, double eos_c,
+                                                       double inv_rho_ref, double* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double v[4];
+  sum_slots(partials, nb, threadIdx.x, blockDim.x, v);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+    if (lane == 0) sh[32 * k + wid] = v[k];
   }
-  if (lane == 0) {
-    const double I = v0;
-    double P0, P0p;
-    if (is_init) {
-      P0 = P0p = init_P0;
-      scal->mass = init_P0 * I * eos_c;
-      scal->flux_in = scal->flux_out = 0;
-      scal->flux_in_sum = scal->flux_out_sum = 0;
-      scal->step = 0;
-      scal->status = 0;
-    } else {
-      P0p = scal->P0;
-      P0 = P0p;
-      if (p0_closed) P0 = scal->mass / (I * eos_c);
-      scal->flux_in = v1;
-      scal->flux_out = v2;
-      scal->flux_in_sum += v1;
-      scal->flux_out_sum += v2;
-      scal->step += 1;
-      // latch only the first failure (a timeout is not overwritten)
-      if (scal->status == 0 && (!(I == I) || !(P0 == P0) || I <= 0.0)) scal->status = -5;
-    }
-    scal->P0_prev = P0p;
-    scal->P0 = P0;
-    scal->I = I;
-    scal->mass_now = P0 * I * eos_c;
-    scal->dlnP0 = (P0 - P0p) / P0;
-    scal->dP0r = (P0 - P0p) * inv_rho_ref;
-    scal->P0_f = float(P0);
-    scal->dlnP0_f = float(scal->dlnP0);
-    scal->dP0r_f = float(scal->dP0r);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double w[3] = {0.0, 0.0, 0.0};
+    for (unsigned q = 0; q < blockDim.x / 32; ++q)
+      for (int k = 0; k < 3; ++k) w[k] += sh[32 * k + q];
+    apply_sums(w[0], w[1], w[2], 0.0, scal, 0, false, 0.0, eos_c, inv_rho_ref, 0.0);
   }
 }
 
@@ -1173,48 +1240,68 @@ __device__ __forceinline__ void combine_partials(const double* partials, unsigne
 // the ticket; the other warps retire).  With a fixed P0 the combine is
 // deferred: block 0 of the next launch, or the on-demand finalize kernel,
 // does it, and the step ends without a serial tail.
+// Write the sums into slot `bid`.
+__device__ __forceinline__ void write_partials(double sI, double sIn, double sOut,
+                                               double* partials, unsigned bid, double sF = 0.0) {
+  if (threadIdx.x == 0) {
+    partials[4 * bid + 3] = sF;
+    partials[4 * bid + 0] = sI;
+    partials[4 * bid + 1] = sIn;
+    partials[4 * bid + 2] = sOut;
+  }
+}
+// Count `n` slots that this block has written; the block that completes the
+// `nb` slots combines them.  (First warp; the others pass.)
+__device__ __forceinline__ void count_partials(double* partials, unsigned* counter,
+                                               DevScalars* scal, int p0_closed, bool is_init,
+                                               double init_P0, double eos_c, double inv_rho_ref,
+                                               unsigned n, unsigned nb, double feed_c = 0.0) {
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  unsigned last = 0;
+  if (lane == 0) {
+    __threadfence();
+    last = (atomicAdd(counter, n) == nb - n) ? 1u : 0u;
+  }
+  last = __shfl_sync(0xffffffffu, last, 0);
+  if (!last) return;
+  __threadfence();
+  combine_partials(partials, nb, scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref, feed_c);
+  if (lane == 0) *counter = 0u;
+}
 // Publish into slot `bid` of `nb`; `now` combines at the last arrival.
 __device__ __forceinline__ void publish_partials_at(double sI, double sIn, double sOut,
                                                     double* partials, unsigned* counter,
                                                     DevScalars* scal, int p0_closed, bool is_init,
                                                     double init_P0, double eos_c,
                                                     double inv_rho_ref, unsigned bid,
-                                                    unsigned nb, bool now) {
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  unsigned last = 0;
-  if (lane == 0) {
-    partials[4 * bid + 0] = sI;
-    partials[4 * bid + 1] = sIn;
-    partials[4 * bid + 2] = sOut;
-    if (now) {
-      __threadfence();
-      last = (atomicAdd(counter, 1u) == nb - 1) ? 1u : 0u;
-    }
-  }
-  if (!now) return;
-  last = __shfl_sync(0xffffffffu, last, 0);
-  if (!last) return;
-  __threadfence();
-  combine_partials(partials, nb, scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref);
-  if (lane == 0) *counter = 0u;
+                                                    unsigned nb, bool now, double sF = 0.0,
+                                                    double feed_c = 0.0) {
+  write_partials(sI, sIn, sOut, partials, bid, sF);
+  if (now)
+    count_partials(partials, counter, scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref, 1u, nb,
+                   feed_c);
 }
 
 __device__ __forceinline__ void publish_partials(double sI, double sIn, double sOut,
                                                  double* partials, unsigned* counter,
                                                  DevScalars* scal, int p0_closed, bool is_init,
                                                  double init_P0, double eos_c,
-                                                 double inv_rho_ref) {
+                                                 double inv_rho_ref, double sF = 0.0,
+                                                 double feed_c = 0.0) {
   publish_partials_at(sI, sIn, sOut, partials, counter, scal, p0_closed, is_init, init_P0, eos_c,
                       inv_rho_ref,
                       blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z),
-                      gridDim.x * gridDim.y * gridDim.z, p0_closed || is_init);
+                      gridDim.x * gridDim.y * gridDim.z, p0_closed || is_init || feed_c > 0.0, sF,
+                      feed_c);
 }
 
-// On-demand combine of the deferred partials of the last step (one warp).
-static __global__ void finalize_kernel(const double* partials, unsigned nb, DevScalars* scal,
-                                double eos_c, double inv_rho_ref) {
-  combine_partials(partials, nb, scal, 0, false, 0.0, eos_c, inv_rho_ref);
+// On-demand combine of the deferred partials of the last step (one block).
+static __global__ void __launch_bounds__(BLOCK)
+finalize_kernel(const double* partials, unsigned nb, DevScalars* scal, double eos_c,
+                double inv_rho_ref) {
+  __shared__ double sh[96];
+  combine_partials_block(partials, nb, scal, eos_c, inv_rho_ref, sh);
 }
 
 // ------------------------------------------------------------ tiles
@@ -1508,12 +1595,14 @@ struct CellPos {
 // Per cell: (a1) pull + moments + implicit drag, (c) reaction source,
 // (b) FD transport of Y_k, T, Ts, low-Mach divergence, (a) source + BGK
 // collision + store, (d) contribution to the FP64 reduction (returned per
-// cell; fluxes through the inlet / outlet face in fin, fout).  `gin` holds the
+// cell; fluxes through the inlet / outlet face in fin, fout; the fuel consumed is
+// added to `fuel` with the inlet feedback).  `gin` holds the
 // streamed populations (load_pops) and is overwritten.
 template <int DIM, int K, class Real, class V, class Acc>
 __device__ __forceinline__ V cell_update(const Params<Real, K>& P, const State<Real, Real>& S,
                                          const Acc& A, V* __restrict__ gin, const CellPos q,
-                                         Real P0, Real dlnP0, Real dP0r, Real& fin, Real& fout) {
+                                         Real P0, Real dlnP0, Real dP0r, Real& fin, Real& fout,
+                                         double& fuel) {
   using L = Lattice<DIM>;
   constexpr int Q = L::Q;
   constexpr int KK = Params<Real, K>::KK;
@@ -1614,6 +1703,20 @@ __device__ __forceinline__ V cell_update(const Params<Real, K>& P, const State<R
 #pragma unroll
       for (int k = 0; k < K; ++k) om[k] = load_cells<V>(S.src + (size_t)k * P.N + q.c, q.even, q.two);
       omT = load_cells<V>(S.src + (size_t)K * P.N + q.c, q.even, q.two);
+    }
+  }
+
+  if constexpr (K > 0) {
+    if (P.feed) {
+#pragma unroll
+      for (int l = 0; l < LN; ++l) {
+        if ((l == 1 && !q.two) || !(get_lane(phif, l) >= P.phi_min)) continue;
+        Real w = 0;
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+          if (k == P.feed_k) w = get_lane(om[k], l);
+        fuel += double(vmul(get_lane(phif, l), -w));
+      }
     }
   }
 
@@ -1857,7 +1960,7 @@ template <int K, class T_> struct MinBlocks {
 template <int K, class Real, class T_>
 __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<Real, Real>& S,
                                           int bx, int by, Real* pl, double* red_sh, double& sI,
-                                          double& sIn, double& sOut) {
+                                          double& sIn, double& sOut, double& sF) {
   using V = typename T_::V;
   constexpr int Q = Lattice<2>::Q, LN = T_::LN, RPT = T_::RPT, RS = T_::TY / RPT;
   const Real P0 = scal_P0<Real>(S.scal);
@@ -1871,6 +1974,7 @@ __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<
   const bool even = LN == 1 || S.even;
   V accI = splat<V>(Real(0));
   Real accIn = 0, accOut = 0;
+  double fuel = 0.0;
   V g[RPT][Q];
 #pragma unroll
   for (int r = 0; r < RPT; ++r)
@@ -1886,13 +1990,14 @@ __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<
       const PlaneAcc<Real, T_> A{pl, nullptr, nullptr,
                                  (ty + r * RS + 1) * T_::HX + tx + T_::XO};
       Real fi, fo;
-      accI = vadd(accI, cell_update<2, K, Real, V>(P, S, A, g[r], q, P0, dlnP0, dP0r, fi, fo));
+      accI = vadd(accI, cell_update<2, K, Real, V>(P, S, A, g[r], q, P0, dlnP0, dP0r, fi, fo,
+                                                     fuel));
       accIn += fi;
       accOut += fo;
     }
   }
   // (d) block partials in FP64 (one barrier)
-  block_sum3(accI, accIn, accOut, flux_block, red_sh, sI, sIn, sOut);
+  block_sum4(accI, accIn, accOut, flux_block, fuel, K > 0 && P.feed, red_sh, sI, sIn, sOut, sF);
 }
 
 template <int DIM, int K, class Real, class T_>
@@ -1906,18 +2011,19 @@ step_kernel(const __grid_constant__ Params<Real, K> P, const State<Real, Real> S
             const double* __restrict__ prev_partials, unsigned prev_nb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* pl = reinterpret_cast<Real*>(smem_raw);
-  __shared__ double red_sh[96];
+  __shared__ double red_sh[128];
 
-  // deferred combine of the previous step's partials (fixed P0 only): block
-  // 0's first warp does it while the other blocks start on their cells
-  if (prev_partials && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32)
-    combine_partials(prev_partials, prev_nb, S.scal, 0, false, 0.0, P.eos_c, P.inv_rho_ref);
+  // deferred combine of the previous step's partials (fixed P0 only): block 0
+  // does it while the other blocks start on their cells
+  if (prev_partials && blockIdx.x == 0 && blockIdx.y == 0)
+    combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
 
-  double sI, sIn, sOut;
-  step_tile<K, Real, T_>(P, S, blockIdx.x, blockIdx.y, pl, red_sh, sI, sIn, sOut);
-  // deterministic finish by the last block (closed P0) or deferred
+  double sI, sIn, sOut, sF;
+  step_tile<K, Real, T_>(P, S, blockIdx.x, blockIdx.y, pl, red_sh, sI, sIn, sOut, sF);
+  // deterministic finish by the last block (closed P0, inlet feedback) or
+  // deferred
   publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
-                   P.inv_rho_ref);
+                   P.inv_rho_ref, sF, P.feed ? P.feed_c : 0.0);
 }
 
 // Persistent variant of the 2-D step: one grid of resident blocks walks the
@@ -1932,11 +2038,11 @@ step_persistent_kernel(const __grid_constant__ Params<Real, K> P, const State<Re
                        unsigned* __restrict__ tile_ctr, int parity) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* pl = reinterpret_cast<Real*>(smem_raw);
-  __shared__ double red_sh[96];
+  __shared__ double red_sh[128];
   __shared__ int next_sh[2];
 
-  if (prev_partials && blockIdx.x == 0 && threadIdx.x < 32)
-    combine_partials(prev_partials, prev_nb, S.scal, 0, false, 0.0, P.eos_c, P.inv_rho_ref);
+  if (prev_partials && blockIdx.x == 0)
+    combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
 
   const int nbx = (P.nx + T_::TX - 1) / T_::TX;
   const int total = nbx * ((P.ny + T_::TY - 1) / T_::TY);
@@ -1951,10 +2057,11 @@ step_persistent_kernel(const __grid_constant__ Params<Real, K> P, const State<Re
     // draw the next tile now; the tile's staging barrier publishes it
     par ^= 1;
     if (threadIdx.x == 0) next_sh[par] = (int)atomicAdd(ctr, 1u);
-    double sI, sIn, sOut;
-    step_tile<K, Real, T_>(P, S, t % nbx, t / nbx, pl, red_sh, sI, sIn, sOut);
+    double sI, sIn, sOut, sF;
+    step_tile<K, Real, T_>(P, S, t % nbx, t / nbx, pl, red_sh, sI, sIn, sOut, sF);
     publish_partials_at(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0,
-                        P.eos_c, P.inv_rho_ref, (unsigned)t, (unsigned)total, p0_closed != 0);
+                        P.eos_c, P.inv_rho_ref, (unsigned)t, (unsigned)total,
+                        p0_closed != 0 || P.feed, sF, P.feed ? P.feed_c : 0.0);
   }
 }
 
@@ -2001,11 +2108,12 @@ chem_implicit_kernel(const __grid_constant__ Params<Real, K> P, const State<Real
 
 // ------------------------------------------------ inlet feedback
 // Sec. 4.4.1: the inflow of species feed_k is matched to its consumption.
-// After the step kernel of step n, whose inputs (T, Y and the pre-pass
-// increments) are still in place, feed_kernel sums phi_f (-omega_k) of that
-// state over the cells (FP64 block partials, grid-stride over at most
-// kFeedBlocks blocks) and feed_combine_kernel sums the partials in a fixed
-// order and sets the inlet peak speed of step n + 1.
+// The FP32 / FP64 steps sum the consumption with their other reductions
+// (combine_partials).  FP16 storage: after the step kernel of step n, whose
+// inputs (T, Y and the pre-pass increments) are still in place, feed_kernel
+// sums phi_f (-omega_k) of that state over the cells (FP64 block partials,
+// grid-stride over at most kFeedBlocks blocks) and feed_combine_kernel sums
+// the partials in a fixed order and sets the inlet peak speed of step n + 1.
 constexpr int kFeedBlocks = 1024;
 
 template <int K, class Real, class Store>

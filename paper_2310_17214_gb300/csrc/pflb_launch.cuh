@@ -117,9 +117,11 @@ struct Launcher {
   virtual void batch_entry(void* dst, const Buffers& B, int cur) const = 0;
   // resident blocks per SM of the batch kernel for tile shape cfg
   virtual int batch_occupancy(int cfg) const = 0;
-  virtual cudaError_t batch_launch(const void* entries, const int* tile_begin, int ndom, int cfg,
+  virtual cudaError_t batch_launch(const void* entries, const int* run_begin, int ndom, int cfg,
                                    int grid, int flip, unsigned* tile_ctr,
                                    cudaStream_t st) const = 0;
+  // consecutive tiles of one domain that a block of the batch draws at a time
+  virtual int batch_run() const = 0;
   // domains can share a batch when their keys are equal (same kernel)
   virtual int batch_key() const = 0;
   // bound of the kernels' device waits (SM clock cycles)
@@ -681,27 +683,28 @@ struct LauncherImpl final : Launcher {
     }
   }
   template <int CFG>
-  static cudaError_t batch_launch_cfg(const void* entries, const int* tile_begin, int ndom,
+  static cudaError_t batch_launch_cfg(const void* entries, const int* run_begin, int ndom,
                                       int grid, int flip, unsigned* ctr, cudaStream_t st) {
     return with_batch_kernel<CFG>([&](auto kern, int threads, size_t smem) {
       kern<<<grid, threads, smem, st>>>(static_cast<const BatchDom<K, Real, Store>*>(entries),
-                                        tile_begin, ndom, flip, ctr);
+                                        run_begin, ndom, flip, ctr);
       return cudaGetLastError();
     });
   }
-  cudaError_t batch_launch(const void* entries, const int* tile_begin, int ndom, int cfg, int grid,
+  cudaError_t batch_launch(const void* entries, const int* run_begin, int ndom, int cfg, int grid,
                            int flip, unsigned* ctr, cudaStream_t st) const override {
     if constexpr (kBatchable) {
       switch (cfg) {
-        case 0: return batch_launch_cfg<0>(entries, tile_begin, ndom, grid, flip, ctr, st);
-        case 1: return batch_launch_cfg<1>(entries, tile_begin, ndom, grid, flip, ctr, st);
-        case 2: return batch_launch_cfg<2>(entries, tile_begin, ndom, grid, flip, ctr, st);
+        case 0: return batch_launch_cfg<0>(entries, run_begin, ndom, grid, flip, ctr, st);
+        case 1: return batch_launch_cfg<1>(entries, run_begin, ndom, grid, flip, ctr, st);
+        case 2: return batch_launch_cfg<2>(entries, run_begin, ndom, grid, flip, ctr, st);
         default: return cudaErrorInvalidValue;
       }
     } else {
       return cudaErrorNotSupported;
     }
   }
+  int batch_run() const override { return kHalf ? 1 : BATCH_RUN; }
   int batch_key() const override { return kBatchable ? 100 + MODE : -1; }
 
   bool tma_usable(const Buffers& B, int cur) {
@@ -792,7 +795,10 @@ struct LauncherImpl final : Launcher {
         if (e != cudaSuccess) return e;
       }
     }
-    const double* prev = (!p0_closed && B.pending)
+    // closed domains, and the FP32 / FP64 steps with the inlet feedback, combine
+    // their sums in the launch itself
+    const bool in_launch = p0_closed || (!kHalf && P.feed);
+    const double* prev = (!in_launch && B.pending)
                              ? B.partials + (size_t)4 * B.slots * B.last_parity : nullptr;
     const int sel = resolved();
     if (sel == 1 && tma_usable(B, cur)) {
@@ -806,7 +812,7 @@ struct LauncherImpl final : Launcher {
                             : step_tiled(B, cur, st, prev);
       if (e != cudaSuccess) return e;
     }
-    if (P.feed) {
+    if (kHalf && P.feed) {  // the other steps sum the consumption themselves
       e = feed(B, cur, st);
       if (e != cudaSuccess) return e;
     }
@@ -818,7 +824,7 @@ struct LauncherImpl final : Launcher {
       e = phase(B, B.nstep, st);
       if (e != cudaSuccess) return e;
     }
-    B.pending = p0_closed ? 0 : 1;
+    B.pending = in_launch ? 0 : 1;
     B.last_parity = cur;
     cur = 1 - cur;
     return cudaGetLastError();
@@ -920,7 +926,7 @@ struct LauncherImpl final : Launcher {
   }
   cudaError_t finalize(Buffers& B, cudaStream_t st) override {
     if (!B.pending) return cudaSuccess;
-    finalize_kernel<<<1, 32, 0, st>>>(B.partials + (size_t)4 * B.slots * B.last_parity,
+    finalize_kernel<<<1, BLOCK, 0, st>>>(B.partials + (size_t)4 * B.slots * B.last_parity,
                                       (unsigned)B.last_nb, B.scal, P.eos_c, P.inv_rho_ref);
     B.pending = 0;
     return cudaGetLastError();

@@ -58,10 +58,10 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
   constexpr int PLANE = (F_Y0 + K) * T_::HP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* planes = reinterpret_cast<Real*>(smem_raw);  // [3][fields][HP]
-  __shared__ double red_sh[96];
+  __shared__ double red_sh[128];
 
-  if (prev_partials && blockIdx.x == 0 && threadIdx.x < 32)
-    combine_partials(prev_partials, prev_nb, S.scal, 0, false, 0.0, P.eos_c, P.inv_rho_ref);
+  if (prev_partials && blockIdx.x == 0)
+    combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
 
   const Real P0 = scal_P0<Real>(S.scal);
   const Real dlnP0 = scal_dlnP0<Real>(S.scal);
@@ -97,6 +97,7 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
 
   V accI = splat<V>(Real(0));
   Real accIn = 0, accOut = 0;
+  double fuel = 0.0;
   bool flux_block = false;
   while (gi < g_end) {
     const int tile = (int)(gi / P.nz);
@@ -125,7 +126,8 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
         const CellPos q{x + P.nx * (y + P.ny * z), x, y, z, even, x + 1 < P.nx};
         const PlaneAcc<Real, T_> A{pc, pm, pp, h};
         Real fi, fo;
-        accI = vadd(accI, cell_update<3, K, Real, V>(P, S, A, g, q, P0, dlnP0, dP0r, fi, fo));
+        accI = vadd(accI, cell_update<3, K, Real, V>(P, S, A, g, q, P0, dlnP0, dP0r, fi, fo,
+                                                       fuel));
         accIn += fi;
         accOut += fo;
       }
@@ -136,10 +138,10 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
       pp = t;
     }
   }
-  double sI, sIn, sOut;
-  block_sum3(accI, accIn, accOut, flux_block, red_sh, sI, sIn, sOut);
+  double sI, sIn, sOut, sF;
+  block_sum4(accI, accIn, accOut, flux_block, fuel, K > 0 && P.feed, red_sh, sI, sIn, sOut, sF);
   publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
-                   P.inv_rho_ref);
+                   P.inv_rho_ref, sF, P.feed ? P.feed_c : 0.0);
 }
 
 }  // namespace pflb

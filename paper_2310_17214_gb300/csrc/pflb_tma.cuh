@@ -132,7 +132,7 @@ struct TmaLayout {
   // +128 so the base can be rounded up to a 128-byte boundary in the kernel
   static constexpr size_t bar_off = 2 * stage_bytes + der_bytes;
   static constexpr size_t red_off = bar_off + 64;
-  static constexpr size_t flag_off = red_off + 96 * sizeof(double);
+  static constexpr size_t flag_off = red_off + 128 * sizeof(double);
   static constexpr size_t smem_bytes = flag_off + 16 + 128;
 };
 
@@ -308,8 +308,8 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
   const float dlnP0 = scal_dlnP0<float>(S.scal);
   const float dP0r = scal_dP0r<float>(S.scal);
 
-  if (prev_partials && blockIdx.x == 0 && threadIdx.x < 32)
-    combine_partials(prev_partials, prev_nb, S.scal, 0, false, 0.0, P.eos_c, P.inv_rho_ref);
+  if (prev_partials && blockIdx.x == 0)
+    combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
 
   // self-check of the alignment every TMA issue relies on (the same answer
   // in every thread): record it and skip all copies rather than fault
@@ -333,6 +333,7 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
   const int lx = (threadIdx.x % (LY::TX / 2)) * 2, ly = threadIdx.x / (LY::TX / 2);
   float2 accI = splat<float2>(0.f);
   float accIn = 0.f, accOut = 0.f;
+  double fuel = 0.0;
   bool any_flux = false;
   int first = blockIdx.x;
   if (threadIdx.x == 0 && first < n_tiles)
@@ -384,7 +385,7 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
       }
       float fi, fo;
       accI = vadd(accI,
-                  cell_update<2, K, float, float2>(P, S, A, g, q, P0, dlnP0, dP0r, fi, fo));
+                  cell_update<2, K, float, float2>(P, S, A, g, q, P0, dlnP0, dP0r, fi, fo, fuel));
       accIn += fi;
       accOut += fo;
     }
@@ -393,10 +394,10 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
     __syncthreads();
   }
 
-  double sI, sIn, sOut;
-  block_sum3(accI, accIn, accOut, any_flux, red_sh, sI, sIn, sOut);
+  double sI, sIn, sOut, sF;
+  block_sum4(accI, accIn, accOut, any_flux, fuel, K > 0 && P.feed, red_sh, sI, sIn, sOut, sF);
   publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
-                   P.inv_rho_ref);
+                   P.inv_rho_ref, sF, P.feed ? P.feed_c : 0.0);
 }
 
 }  // namespace pflb
