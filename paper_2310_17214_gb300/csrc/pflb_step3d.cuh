@@ -124,7 +124,7 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
       if (in_xy) {
         if (!PRE) load_pops<3, K, Real, V>(P, S, x, y, z, g);
         const CellPos q{x + P.nx * (y + P.ny * z), x, y, z, even, x + 1 < P.nx};
-        const PlaneAcc<Real, T_> A{pc, pm, pp, h};
+        const PlaneAcc<Real, T_> A{pc, pm, pp, h, nullptr};
         Real fi, fo;
         accI = vadd(accI, cell_update<3, K, Real, V>(P, S, A, g, q, P0, dlnP0, dP0r, fi, fo,
                                                        fuel));

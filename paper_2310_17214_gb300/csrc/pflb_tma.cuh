@@ -163,6 +163,8 @@ struct TmaAcc {
   __device__ __forceinline__ float2 c(int f) const {
     return *reinterpret_cast<const float2*>(at(f, 0, 0));
   }
+  __device__ __forceinline__ bool has_src() const { return false; }
+  __device__ __forceinline__ float2 increment(int) const { return make_float2(0.f, 0.f); }
   __device__ __forceinline__ float2 n(int f, int a, int s, float2 own) const {
     if (a == 1) return *reinterpret_cast<const float2*>(at(f, 0, s));
     const float v = *at(f, s < 0 ? -1 : 2, 0);
