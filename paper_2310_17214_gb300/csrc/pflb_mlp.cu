@@ -31,6 +31,34 @@ struct pflb_mlp {
 
 namespace {
 
+// Programmatic dependent launch: a kernel launched that way may start while the
+// kernel before it in the stream is finishing.  pdl_wait holds it until that
+// kernel has completed and its writes are visible (nothing is read or written
+// before); pdl_trigger lets the kernel after this one start once every block
+// has called it or ended.  Both do nothing in an ordinary launch.  A training step
+// is two short kernels that wait for each other; started this way they hide
+// their launches and prologues (a step of 8,192 rows: 25 -> 20 us with the
+// changes beside it).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem,
+                             cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 constexpr int TW = 4;                // warps per block in the training kernel
 constexpr int TROWS = 16 * TW;       // rows per block and iteration
 constexpr int HLD = 72;              // row stride of the BF16 tiles: ldmatrix without conflicts
@@ -210,6 +238,16 @@ __device__ __forceinline__ void back_dx(const SmemNet& s, const uint32_t* a, con
   }
 }
 
+// Asynchronous 16-byte copies of NV vectors by the block.
+template <int NV>
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  for (int i = threadIdx.x; i < NV; i += TW * 32)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     static_cast<unsigned>(__cvta_generic_to_shared(dst)) + 16u * i),
+                 "l"(static_cast<const char*>(src) + 16 * (size_t)i)
+                 : "memory");
+}
+
 // Forward + backward of mini-batch rows: the block's part of the gradient of
 // the mean squared error (scaled by inv_norm = 1 / (rows x 6)) and of the loss,
 // into slot blockIdx.x.
@@ -220,21 +258,22 @@ __device__ __forceinline__ void back_dx(const SmemNet& s, const uint32_t* a, con
 // gradient per block goes to memory; update_kernel sums them in a fixed order
 // (with a shared-memory and a global atomic per element and tile instead, and
 // the network loaded one dependent word at a time, a mini-batch of 8,192 rows
-// took 73 us, and takes 25).  What is left is latency: a few hundred dependent
+// took 73 us, and takes 20).  What is left is latency: a few hundred dependent
 // tensor-core and tanh steps of one wave of blocks, twice a launch.
 __global__ void __launch_bounds__(TW * 32, 1)
 grad_kernel(Net net, const float* __restrict__ X, const float* __restrict__ Y, long long n,
             float inv_norm, float* __restrict__ part, double* __restrict__ loss) {
   extern __shared__ __align__(16) unsigned char smem[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem);
-  load_vec16<NPAD * 2 / 16, TW * 32>(reinterpret_cast<uint4*>(S.net.wf),
-                                     reinterpret_cast<const uint4*>(net.wf));
-  load_vec16<NPAD * 2 / 16, TW * 32>(reinterpret_cast<uint4*>(S.net.wb),
-                                     reinterpret_cast<const uint4*>(net.wb));
-  load_vec16<NPB * 4 / 16, TW * 32>(reinterpret_cast<uint4*>(S.net.bias),
-                                    reinterpret_cast<const uint4*>(net.bias));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   for (int i = lane; i < NPB; i += 32) S.db[warp][i] = 0.f;
+  pdl_wait();  // the parameters of the update before
+  pdl_trigger();
+  // the network, every copy in flight at once
+  copy16<NPAD * 2 / 16>(S.net.wf, net.wf);
+  copy16<NPAD * 2 / 16>(S.net.wb, net.wb);
+  copy16<NPB * 4 / 16>(S.net.bias, net.bias);
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   float w1[2][4] = {}, w2[8][4] = {}, w3[8][4] = {}, w4[1][4] = {};
   float lsum = 0.f;
@@ -348,10 +387,10 @@ __device__ __forceinline__ Place place_of(int i) {
           poff(l) + in * pdim(l + 1) + o};
 }
 
-// Sum of the blocks' partial gradients (fixed order: four slices of the
+// Sum of the blocks' partial gradients (fixed order: eight slices of the
 // blocks, then the slices) and, with ADAM, the parameter update and its copies
 // in the network's layouts, with the loss of the mini-batch summed beside.
-constexpr int UP = 64, US = 4;  // parameters and slices per block
+constexpr int UP = 32, US = 8;  // parameters and slices per block
 template <bool ADAM>
 __global__ void __launch_bounds__(UP * US)
 update_kernel(const float* __restrict__ part, int nb, const double* __restrict__ block_loss,
@@ -362,15 +401,18 @@ update_kernel(const float* __restrict__ part, int nb, const double* __restrict__
   __shared__ float sh[US][UP];
   const int q = threadIdx.x % UP, s = threadIdx.x / UP, i = blockIdx.x * UP + q;
   float sum = 0.f;
+  pdl_wait();
+  pdl_trigger();
   if (i < NPARAM) {
     const int b0 = nb * s / US, b1 = nb * (s + 1) / US;
-#pragma unroll 8
+#pragma unroll 16
     for (int b = b0; b < b1; ++b) sum += part[(size_t)b * NPARAM + i];
   }
   sh[s][q] = sum;
   __syncthreads();
   if (s == 0 && i < NPARAM) {
-    const float gi = (sh[0][q] + sh[1][q]) + (sh[2][q] + sh[3][q]);
+    const float gi = ((sh[0][q] + sh[1][q]) + (sh[2][q] + sh[3][q])) +
+                     ((sh[4][q] + sh[5][q]) + (sh[6][q] + sh[7][q]));
     if constexpr (!ADAM) {
       grad[i] = gi;
     } else {
@@ -461,8 +503,8 @@ Net net_of(const pflb_mlp* m) { return Net{m->wf, m->wb, m->bias, m->theta}; }
 // The partial gradients of n rows; returns their number.
 int launch_grad(pflb_mlp* m, const float* X, const float* Y, long long n) {
   const int nb = (int)std::min<long long>((n + TROWS - 1) / TROWS, MAX_PART);
-  grad_kernel<<<nb, TW * 32, sizeof(TrainSmem), m->stream>>>(
-      net_of(m), X, Y, n, 1.f / (float)(n * 6), m->part, m->loss + 1);
+  launch_dependent(grad_kernel, dim3(nb), TW * 32, sizeof(TrainSmem), m->stream, net_of(m), X,
+                   Y, n, 1.f / (float)(n * 6), m->part, m->loss + 1);
   return nb;
 }
 
@@ -575,9 +617,9 @@ int pflb_mlp_train(pflb_mlp* m, const float* X, const float* Y, long long n, int
     m->t += 1;
     const float c1 = 1.f / (1.f - powf(0.9f, (float)m->t));
     const float c2 = 1.f / (1.f - powf(0.999f, (float)m->t));
-    update_kernel<true><<<(NPARAM + UP - 1) / UP, UP * US, 0, m->stream>>>(
-        m->part, nblk, m->loss + 1, m->loss, nullptr, m->theta, m->m, m->v, m->wf, m->wb, m->bias,
-        lr, c1, c2);
+    launch_dependent(update_kernel<true>, dim3((NPARAM + UP - 1) / UP), UP * US, 0, m->stream,
+                     m->part, nblk, m->loss + 1, m->loss, (float*)nullptr, m->theta, m->m,
+                     m->v, m->wf, m->wb, m->bias, lr, c1, c2);
     if (last && last_loss) {
       double l = 0;
       cudaMemcpyAsync(&l, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream);
