@@ -131,23 +131,51 @@ __device__ __forceinline__ void layer_fwd(const __nv_bfloat16* wf, const float* 
   }
 }
 
-// The same for two 16-row tiles sharing each B fragment.
+// The same for two 16-row tiles sharing each B fragment, n-tile j.
 template <int L>
-__device__ __forceinline__ void layer_fwd2(const __nv_bfloat16* wf, const float* bias,
-                                           const uint32_t* a0, const uint32_t* a1,
-                                           float acc0[][4], float acc1[][4]) {
-  constexpr int IN = pdim(L), OUT = pdim(L + 1);
+__device__ __forceinline__ void tile_fwd2(const __nv_bfloat16* wf, const float* bias, int j,
+                                          const uint32_t* a0, const uint32_t* a1, float c0[4],
+                                          float c1[4]) {
   const int t = threadIdx.x & 3;
   const float* b = bias + pboff(L);
+  c0[0] = c0[2] = c1[0] = c1[2] = b[8 * j + 2 * t];
+  c0[1] = c0[3] = c1[1] = c1[3] = b[8 * j + 2 * t + 1];
 #pragma unroll
-  for (int j = 0; j < OUT / 8; ++j) {
-    acc0[j][0] = acc0[j][2] = acc1[j][0] = acc1[j][2] = b[8 * j + 2 * t];
-    acc0[j][1] = acc0[j][3] = acc1[j][1] = acc1[j][3] = b[8 * j + 2 * t + 1];
+  for (int kk = 0; kk < pdim(L) / 16; ++kk) {
+    const uint2 w = b_frag<L>(wf, j, kk);
+    mma16816(c0, a0 + 4 * kk, w.x, w.y);
+    mma16816(c1, a1 + 4 * kk, w.x, w.y);
+  }
+}
+
+// A hidden layer for two 16-row tiles: r = A fragments of tanh(a W + b).  The
+// tanh of n-tile j - 1 is issued behind the products of n-tile j, and an n-tile
+// is packed as soon as it is activated: 32 tanh a lane behind a whole layer's
+// products left the tensor pipe idle meanwhile.  The pre-pass is bound by the
+// two together (2^20 cells, ncu: transcendental unit 62 % of 70 us, tensor pipe
+// 49 %): a surrogate step of 2048 x 512 cells 146.4 -> 143.2 us.  Without effect
+// on top: 20 or 24 warps per SM in place of 16 (151 to 157 us, spills), the next
+// cells' inputs copied ahead (143.2).
+template <int L>
+__device__ __forceinline__ void hidden2(const __nv_bfloat16* wf, const float* bias,
+                                        const uint32_t* a0, const uint32_t* a1, uint32_t* r0,
+                                        uint32_t* r1) {
+  float c0[2][4], c1[2][4];
 #pragma unroll
-    for (int kk = 0; kk < IN / 16; ++kk) {
-      const uint2 w = b_frag<L>(wf, j, kk);
-      mma16816(acc0[j], a0 + 4 * kk, w.x, w.y);
-      mma16816(acc1[j], a1 + 4 * kk, w.x, w.y);
+  for (int j = 0; j <= 8; ++j) {
+    if (j < 8) tile_fwd2<L>(wf, bias, j, a0, a1, c0[j & 1], c1[j & 1]);
+    if (j > 0) {
+      float* u = c0[(j - 1) & 1];
+      float* v = c1[(j - 1) & 1];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        u[e] = fast_tanh(u[e]);
+        v[e] = fast_tanh(v[e]);
+      }
+      r0[2 * (j - 1)] = pack_bf16(u[0], u[1]);
+      r0[2 * (j - 1) + 1] = pack_bf16(u[2], u[3]);
+      r1[2 * (j - 1)] = pack_bf16(v[0], v[1]);
+      r1[2 * (j - 1) + 1] = pack_bf16(v[2], v[3]);
     }
   }
 }
@@ -189,26 +217,13 @@ constexpr int XLD = 24;
 // padding).
 __device__ __forceinline__ void forward32(const SmemFwd& s, const __nv_bfloat16* x,
                                           float out0[4], float out1[4]) {
-  uint32_t a0[16], a1[16];
+  uint32_t a0[16], a1[16], b0[16], b1[16];
   x_frags(x, XLD, a0);
   x_frags(x + 16 * XLD, XLD, a1);
-  float c0[8][4], c1[8][4];
-  layer_fwd2<0>(s.wf, s.bias, a0, a1, c0, c1);
-  to_a<true>(c0, a0);
-  to_a<true>(c1, a1);
-  layer_fwd2<1>(s.wf, s.bias, a0, a1, c0, c1);
-  to_a<true>(c0, a0);
-  to_a<true>(c1, a1);
-  layer_fwd2<2>(s.wf, s.bias, a0, a1, c0, c1);
-  to_a<true>(c0, a0);
-  to_a<true>(c1, a1);
-  float o0[1][4], o1[1][4];
-  layer_fwd2<3>(s.wf, s.bias, a0, a1, o0, o1);
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    out0[e] = o0[0][e];
-    out1[e] = o1[0][e];
-  }
+  hidden2<0>(s.wf, s.bias, a0, a1, b0, b1);
+  hidden2<1>(s.wf, s.bias, b0, b1, a0, a1);
+  hidden2<2>(s.wf, s.bias, a0, a1, b0, b1);
+  tile_fwd2<3>(s.wf, s.bias, 0, b0, b1, out0, out1);
 }
 
 }  // namespace mlp
