@@ -19,12 +19,11 @@ namespace half_store {
 // on GB300 for the single-domain step: 32 x 8 with one row per thread is
 // fastest (two rows spill at the 64-register cap); the prefetch helps the
 // FP16-stored path.  The batched step lets its autotuner pick among shapes.
-// 3-D blocks march over ZC planes.
+// 3-D blocks march over a run of planes.
 template <int DIM, int TXv = 32, int RPTv = 1> struct Tile {
   static constexpr int RPT = RPTv;
   static constexpr bool PREFETCH = DIM == 2;
   static constexpr int TX = TXv, TY = (256 / TXv) * RPT;
-  static constexpr int ZC = DIM == 3 ? 16 : 1;
   static constexpr int HX = TX + 2, HY = TY + 2, HP = HX * HY;
   static constexpr int NPL = DIM == 3 ? 3 : 1;  // staged planes
 };
@@ -812,13 +811,13 @@ template <int DIM, class Real, class Store> struct MinBlocks {
       sizeof(Real) == 8 ? (DIM == 3 ? 1 : 2) : (DIM == 2 ? 4 : (IsHalf<Store>::value ? 2 : 3));
 };
 
-// One tile of the fused step (tile (bx, by) of the xy grid, z-chunk bz in
-// 3-D): stages the tile's planes in `planes` (shared memory), updates its
+// One tile of the fused step (tile (bx, by) of the xy grid, planes z_begin to
+// z_end in 3-D): stages the tile's planes in `planes` (shared memory), updates its
 // cells and returns the block sums of the reduction in thread 0 (I, inlet
 // flux, outlet flux).  Every thread of the block calls it.
 template <int DIM, int K, class Real, class Store, class T_ = Tile<DIM>>
 __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<Real, Store>& S,
-                                          int bx, int by, int bz,
+                                          int bx, int by, int z_begin, int z_end,
                                           Plane<Real, K, T_::HP, n_mom<DIM, Store>()>* planes,
                                           double* red_sh,
                                           double& sI, double& sIn, double& sOut) {
@@ -831,8 +830,6 @@ __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<
   const int x = x0 + tx, y = y0 + ty;
   const int h = (ty + 1) * T_::HX + (tx + 1);
   const bool in_xy = x < P.nx && y < P.ny;
-  const int z_begin = bz * T_::ZC;
-  const int z_end = DIM == 3 ? min(z_begin + T_::ZC, P.nz) : 1;
   const bool flux_block = (x0 == 0 && P.bc[0] == BC_INLET) ||
                           (x0 + T_::TX >= P.nx && P.bc[1] == BC_OUTLET);
 
@@ -910,7 +907,7 @@ __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<
 template <int DIM, int K, class Real, class Store>
 __global__ void __launch_bounds__(BLOCK, MinBlocks<DIM, Real, Store>::value)
 step_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
-            const double* __restrict__ prev_partials, unsigned prev_nb) {
+            const double* __restrict__ prev_partials, unsigned prev_nb, int chunk) {
   using T_ = Tile<DIM>;
   using PL = Plane<Real, K, T_::HP, n_mom<DIM, Store>()>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -919,13 +916,20 @@ step_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
 
   // deferred combine of the previous step's partials (fixed P0 only): block
   // 0's first warp does it while the other blocks start on their cells
-  if (prev_partials && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 &&
-      threadIdx.x < 32)
+  if (prev_partials && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32)
     combine_partials(prev_partials, prev_nb, S.scal, 0, false, 0.0, P.eos_c, P.inv_rho_ref);
 
   double sI, sIn, sOut;
-  half_store::step_tile<DIM, K, Real, Store, T_>(P, S, blockIdx.x, blockIdx.y, blockIdx.z, planes, red_sh,
-                                     sI, sIn, sOut);
+  int bx = blockIdx.x, by = blockIdx.y, z0 = 0, z1 = 1;
+  if constexpr (DIM == 3) {
+    const int gx = (P.nx + T_::TX - 1) / T_::TX;
+    const ZRun r = z_run(blockIdx.x, gx * ((P.ny + T_::TY - 1) / T_::TY), P.nz, chunk);
+    bx = r.tile % gx;
+    by = r.tile / gx;
+    z0 = r.z_begin;
+    z1 = r.z_end;
+  }
+  half_store::step_tile<DIM, K, Real, Store, T_>(P, S, bx, by, z0, z1, planes, red_sh, sI, sIn, sOut);
   // deterministic finish by the last block (closed P0) or deferred
   publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
                    P.inv_rho_ref);
@@ -965,7 +969,7 @@ step_persistent_kernel(const Params<Real, K> P, const State<Real, Store> S, int 
     par ^= 1;
     if (threadIdx.x == 0) next_sh[par] = (int)atomicAdd(ctr, 1u);
     double sI, sIn, sOut;
-    half_store::step_tile<DIM, K, Real, Store, T_>(P, S, t % nbx, t / nbx, 0, planes, red_sh, sI, sIn,
+    half_store::step_tile<DIM, K, Real, Store, T_>(P, S, t % nbx, t / nbx, 0, 1, planes, red_sh, sI, sIn,
                                        sOut);
     publish_partials_at(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0,
                         P.eos_c, P.inv_rho_ref, (unsigned)t, (unsigned)total, p0_closed != 0);
@@ -1294,7 +1298,7 @@ batch_step_kernel(const BatchDom<K, Real, Store>* __restrict__ doms,
     const int lt = t - tile_begin[lo];
     const int nbx = (Psh.nx + T_::TX - 1) / T_::TX;
     double sI, sIn, sOut;
-    half_store::step_tile<2, K, Real, Store, T_>(Psh, Ssh, lt % nbx, lt / nbx, 0, planes, red_sh, sI, sIn,
+    half_store::step_tile<2, K, Real, Store, T_>(Psh, Ssh, lt % nbx, lt / nbx, 0, 1, planes, red_sh, sI, sIn,
                                      sOut);
     const unsigned nb = (unsigned)(tile_begin[lo + 1] - tile_begin[lo]);
     publish_partials_at(sI, sIn, sOut, Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0,

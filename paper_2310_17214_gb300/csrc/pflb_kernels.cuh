@@ -1304,6 +1304,45 @@ finalize_kernel(const double* partials, unsigned nb, DevScalars* scal, double eo
   combine_partials_block(partials, nb, scal, eos_c, inv_rho_ref, sh);
 }
 
+// ------------------------------------------------ runs of planes (3-D)
+// Chunks of c planes (per tile) of the decreasing-size schedule that has
+// reached plane zc: three quarters of what is left in the first class, the
+// rest of it in the last (c <= 4).
+__host__ __device__ inline int chunk_count(int nz, int zc, int c) {
+  const int left = nz - zc;
+  return c <= 4 ? (left + c - 1) / c : left * 3 / 4 / c;
+}
+__host__ __device__ inline int chunks_per_tile(int nz, int c) {
+  int n = 0, zc = 0;
+  for (;; c = c > 4 ? c / 2 : c) {
+    const int k = chunk_count(nz, zc, c);
+    n += k;
+    zc += k * c;
+    if (c <= 4) return n;
+  }
+}
+
+// The run of planes of block b, which takes long chunks first and shorter ones
+// last in launch order; chunk < 0: chunks of -chunk planes all along.
+struct ZRun { int tile, z_begin, z_end; };
+__device__ __forceinline__ ZRun z_run(int b, int tiles, int nz, int chunk) {
+  if (chunk < 0) {
+    const int z = b / tiles * -chunk;
+    return {b % tiles, z, min(z - chunk, nz)};
+  }
+  int zc = 0, c = chunk;
+#pragma unroll 1
+  for (;; c = c > 4 ? c / 2 : c) {
+    const int n = chunk_count(nz, zc, c);  // chunks of c planes per tile
+    if (b < n * tiles || c <= 4) {
+      zc += b / tiles * c;
+      return {b % tiles, zc, min(zc + c, nz)};
+    }
+    b -= n * tiles;
+    zc += n * c;
+  }
+}
+
 // ------------------------------------------------------------ tiles
 // A block owns TX x TY cells of a plane; a thread owns LN neighbouring cells
 // in x (two in FP32 compute, one in FP64) in each of RPT rows.

@@ -373,15 +373,35 @@ struct LauncherImpl final : Launcher {
   }
   int blocks() const { return (P.N + BLOCK - 1) / BLOCK; }
   // tiles of the staged step: 32 x step_ty() cells; in 3-D a block takes a run of
-  // at most kChunk planes
+  // planes (z_run)
   using V = typename VecOf<Real>::V;
   static constexpr bool kHalf = MODE == MODE_FP16;
-  static constexpr int kChunk = kHalf ? 16 : 32;
+  static constexpr int kChunk = 32;
   using HalfTile = half_store::Tile<DIM>;
   dim3 step_grid() {
     const unsigned gx = (P.nx + 31) / 32, gy = (P.ny + step_ty() - 1) / step_ty();
-    if (DIM == 3 && kHalf) return dim3(gx, gy, (P.nz + kChunk - 1) / kChunk);
-    return DIM == 3 ? dim3(gx * gy * chunks_per_tile(P.nz, kChunk)) : dim3(gx, gy);
+    if (DIM == 2) return dim3(gx, gy);
+    const int c = kHalf ? half_chunk() : kChunk;
+    return dim3(gx * gy * (c > 0 ? chunks_per_tile(P.nz, c) : (P.nz - c - 1) / -c));
+  }
+  // Runs of planes of the FP16-stored 3-D step (256 threads, two blocks per SM),
+  // by the planes a resident block has to do.  Below eight, the shortest equal
+  // runs that all fit in one wave (64^3: 47 us a step; shrinking ones from eight
+  // 68, equal ones of sixteen 114); else runs that shrink from eight (160 x 96 x
+  // 96, 19 planes: 186; 251 equal ones of sixteen, 281 shrinking from 32), from
+  // sixteen at 32 planes and more (256 x 128 x 128, 54 planes: 437; 457 from
+  // eight, 491 from 32, 493 equal ones of sixteen).  A closed domain keeps equal
+  // runs of sixteen: its FP32 partial sums set P0, and FP16 residuals amplify a
+  // last bit of it.
+  int half_chunk() {
+    const long long tiles = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
+    const long long resident = 2LL * sm_count();
+    if (p0_closed) return -16;
+    if (tiles * P.nz >= 32 * resident) return 16;
+    if (tiles * P.nz < 8 * resident)
+      for (int c = 1; c <= P.nz; ++c)
+        if (tiles * ((P.nz + c - 1) / c) <= resident) return -c;
+    return 8;
   }
   int sm_count() {
     if (sms == 0) {
@@ -568,24 +588,26 @@ struct LauncherImpl final : Launcher {
     }
   }
 
-  // staged tiles, one block each (in 3-D, FP16 storage: kChunk planes of one)
+  // staged tiles, one block each (in 3-D a run of planes of one)
   cudaError_t step_tiled(Buffers& B, int cur, cudaStream_t st, const double* prev) {
     if constexpr (DIM == 3 && !kHalf) {
       return step_march<false>(B, cur, st, prev, true);
     } else {
       const dim3 grid = step_grid();
       if (step_blocks() > B.slots) return cudaErrorInvalidValue;
-      auto launch = [&](auto kern, int threads, size_t smem) -> cudaError_t {
+      auto launch = [&](auto kern, int threads, size_t smem, auto... chunk) -> cudaError_t {
         const cudaError_t e =
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<grid, threads, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb);
+        kern<<<grid, threads, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb,
+                                      chunk...);
         return cudaGetLastError();
       };
       cudaError_t e;
       if constexpr (kHalf) {
         e = launch(half_store::step_kernel<DIM, K, Real, Store>, BLOCK,
-                   half_store::step_smem_bytes<DIM, K, Real, Store>());
+                   half_store::step_smem_bytes<DIM, K, Real, Store>(),
+                   DIM == 3 ? half_chunk() : 0);
       } else if constexpr (sizeof(Real) == 4) {
         using T_ = Tile<V, 32, 8>;
         e = launch(step_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>());

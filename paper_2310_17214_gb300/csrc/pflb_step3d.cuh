@@ -30,23 +30,6 @@ template <class Real> struct MarchTile {
   static constexpr int MINB = sizeof(Real) == 8 ? 1 : 3;
 };
 
-// Chunks of c planes (per tile) of the decreasing-size schedule that has
-// reached plane zc: three quarters of what is left in the first class, the
-// rest of it in the last (c <= 4).
-__host__ __device__ inline int chunk_count(int nz, int zc, int c) {
-  const int left = nz - zc;
-  return c <= 4 ? (left + c - 1) / c : left * 3 / 4 / c;
-}
-__host__ __device__ inline int chunks_per_tile(int nz, int c) {
-  int n = 0, zc = 0;
-  for (;; c = c > 4 ? c / 2 : c) {
-    const int k = chunk_count(nz, zc, c);
-    n += k;
-    zc += k * c;
-    if (c <= 4) return n;
-  }
-}
-
 template <int K, class Real, bool PRE>
 __global__ void __launch_bounds__(MarchTile<Real>::T::NT, MarchTile<Real>::MINB)
 step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real, Real> S,
@@ -72,21 +55,9 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
   const long long total = (long long)tiles * P.nz;
   long long gi, g_end;
   if (chunk > 0) {
-    // blocks in launch order take long chunks first and shorter ones last
-    int b = blockIdx.x, zc = 0, c = chunk;
-#pragma unroll 1
-    for (;; c = c > 4 ? c / 2 : c) {
-      const int n = chunk_count(P.nz, zc, c);  // chunks of c planes per tile
-      if (b < n * tiles) {
-        const int t = b % tiles;
-        zc += b / tiles * c;
-        gi = (long long)t * P.nz + zc;
-        g_end = gi + min(c, P.nz - zc);
-        break;
-      }
-      b -= n * tiles;
-      zc += n * c;
-    }
+    const ZRun r = z_run(blockIdx.x, tiles, P.nz, chunk);
+    gi = (long long)r.tile * P.nz + r.z_begin;
+    g_end = gi + (r.z_end - r.z_begin);
   } else {
     gi = total * blockIdx.x / gridDim.x;
     g_end = total * (blockIdx.x + 1) / gridDim.x;
