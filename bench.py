@@ -722,7 +722,10 @@ def main():
     achieved = bpc * N / per_launch / 1e9
     workload = workload_name(prob)
     kname = {"fp32": "float,float", "fp32_fp16": "float,__half", "fp64": "double,double"}
-    kernel = f"{KERNEL_FN[tuned['chosen']]} (3-D, K=5, {kname[args.precision]})"
+    fn = KERNEL_FN[tuned["chosen"]]
+    if fn == "step_kernel" and args.precision != "fp32_fp16":  # 3-D tiles in shrinking runs
+        fn = "step3d_march_kernel<prefetch=false>, shrinking runs"
+    kernel = f"{fn} (3-D, K=5, {kname[args.precision]})"
 
     extra = {}
     if not args.quick and rank == 0:
