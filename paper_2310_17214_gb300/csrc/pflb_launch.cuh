@@ -376,14 +376,23 @@ struct LauncherImpl final : Launcher {
   // planes (z_run)
   using V = typename VecOf<Real>::V;
   static constexpr bool kHalf = MODE == MODE_FP16;
-  static constexpr int kChunk = 32;
   using HalfTile = half_store::Tile<DIM>;
   dim3 step_grid() {
     const unsigned gx = (P.nx + 31) / 32, gy = (P.ny + step_ty() - 1) / step_ty();
     if (DIM == 2) return dim3(gx, gy);
-    const int c = kHalf ? half_chunk() : kChunk;
+    const int c = kHalf ? half_chunk() : first_chunk();
     return dim3(gx * gy * (c > 0 ? chunks_per_tile(P.nz, c) : (P.nz - c - 1) / -c));
   }
+  // Planes of the tile columns of a 3-D domain and, FP32 / FP64, the resident
+  // blocks that share them.
+  long long planes() const {
+    return (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8) * P.nz;
+  }
+  long long resident3d() { return (sizeof(Real) == 8 ? 1LL : 3LL) * sm_count(); }
+  // First run of the shrinking runs: 32 planes, sixteen where that is more than a
+  // resident block's share (FP32, 250 x 100 x 100, 23 planes: 177 us a step, 210
+  // from 32; 256 x 128 x 128, 36 planes: 260, 253 from 32).
+  int first_chunk() { return planes() >= 32 * resident3d() ? 32 : 16; }
   // Runs of planes of the FP16-stored 3-D step (256 threads, two blocks per SM),
   // by the planes a resident block has to do.  Below eight, the shortest equal
   // runs that all fit in one wave (64^3: 47 us a step; shrinking ones from eight
@@ -494,8 +503,7 @@ struct LauncherImpl final : Launcher {
   int resolved() {
     if (kernel_sel >= 0) return kernel_sel;
     if (DIM == 2 || kHalf) return 0;
-    const long long planes = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8) * P.nz;
-    return planes < 16LL * sm_count() * (sizeof(Real) == 8 ? 1 : 3) ? 4 : 0;
+    return planes() < 16 * resident3d() ? 4 : 0;
   }
   long long wait_limit = kDefaultWaitCycles;
   void set_wait_limit(long long cycles) override { wait_limit = cycles; }
@@ -557,7 +565,7 @@ struct LauncherImpl final : Launcher {
   }
 
   // 3-D step: the persistent z-march (grid = resident blocks per SM x SMs) or,
-  // with chunked = true, one block per tile and kChunk planes
+  // with chunked = true, one block per shrinking run
   int mgrid[2] = {0, 0};
   template <bool PRE>
   cudaError_t step_march(Buffers& B, int cur, cudaStream_t st, const double* prev, bool chunked) {
@@ -579,7 +587,7 @@ struct LauncherImpl final : Launcher {
         const int nb = chunked ? (int)step_blocks() : grid;
         if (nb > B.slots) return cudaErrorInvalidValue;
         kern<<<nb, T_::NT, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb,
-                                       chunked ? kChunk : 0);
+                                       chunked ? first_chunk() : 0);
         B.last_nb = nb;
       }
       return cudaGetLastError();
