@@ -582,7 +582,9 @@ struct LauncherImpl final : Launcher {
         using T_ = typename MarchTile<Real>::T;
         constexpr size_t smem = step_smem_bytes<3, K, Real, T_>();
         auto kern = step3d_march_kernel<K, Real, PRE>;
-        const cudaError_t e = resident_grid(kern, T_::NT, smem, grid, B.slots);
+        // no more blocks than planes of the tile columns, so that none is without
+        const cudaError_t e =
+            resident_grid(kern, T_::NT, smem, grid, std::min(B.slots, planes()));
         if (e != cudaSuccess) return e;
         const int nb = chunked ? (int)step_blocks() : grid;
         if (nb > B.slots) return cudaErrorInvalidValue;

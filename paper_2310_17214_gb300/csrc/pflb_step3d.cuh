@@ -43,8 +43,12 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
   Real* planes = reinterpret_cast<Real*>(smem_raw);  // [3][fields][HP]
   __shared__ double red_sh[128];
 
-  if (prev_partials && blockIdx.x == 0)
+  if (prev_partials && blockIdx.x == 0) {
     combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
+    // the block's own sums go to red_sh next; a block without planes meets no
+    // other barrier before them
+    __syncthreads();
+  }
 
   const Real P0 = scal_P0<Real>(S.scal);
   const Real dlnP0 = scal_dlnP0<Real>(S.scal);
