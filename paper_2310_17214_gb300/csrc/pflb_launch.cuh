@@ -426,6 +426,10 @@ struct LauncherImpl final : Launcher {
   // SM: the height whose tiles spread best, counting an SM's tiles times the
   // pipe work of one (a staged cell costs about a quarter of an update).  A
   // 128 x 64 channel has 32 tiles of 8 rows, on as many SMs, or 128 of 2 rows.
+  // A lower tile is left out where its tiles exceed most_tiles, the partial slots
+  // of a caller that cannot size them by the tile (131072 x 10 cells: 8,192 tiles
+  // of 8 rows, 20,480 of 2).
+  long long most_tiles = 1LL << 40;
   int ty_cached = 0;
   int step_ty() {
     if (DIM == 3 || sizeof(Real) == 4) return 8;
@@ -433,6 +437,7 @@ struct LauncherImpl final : Launcher {
       double best = 0;
       for (int ty = 8; ty >= 2; ty /= 2) {
         const long long tiles = (long long)((P.nx + 31) / 32) * ((P.ny + ty - 1) / ty);
+        if (ty < 8 && tiles > most_tiles) continue;
         const double cost =
             double((tiles + sm_count() - 1) / sm_count()) * (32 * ty + 0.25 * 34 * (ty + 2));
         if (ty_cached == 0 || cost < best) {

@@ -134,6 +134,7 @@ extern "C" int pflb_step_noalloc(const pflb_domain_desc* desc, const pflb_mechan
   cudaError_t e = cudaSuccess;
   long long nblk = 0;
   auto run = [&](auto& L) {
+    L.most_tiles = kMaxBlocks;
     nblk = L.step_blocks();
     if (nblk <= kMaxBlocks) {
       e = L.step(B, cur, 1, st);
