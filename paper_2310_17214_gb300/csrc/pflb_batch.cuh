@@ -94,7 +94,7 @@ batch_step_kernel(const BatchDom<K, Real, Real>* __restrict__ doms,
       write_partials(sI, sIn, sOut, Ssh.partials, (unsigned)(first + i));
     }
     const int nb = ((Psh.nx + T_::TX - 1) / T_::TX) * ((Psh.ny + T_::TY - 1) / T_::TY);
-    count_partials(Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0, Psh.eos_c,
+    count_partials<slots_in_flight(K)>(Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0, Psh.eos_c,
                    Psh.inv_rho_ref, (unsigned)min(BATCH_RUN, nb - first), (unsigned)nb);
   }
 }

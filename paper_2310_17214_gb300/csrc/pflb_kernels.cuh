@@ -1166,71 +1166,96 @@ __device__ __forceinline__ void apply_sums(double I, double in, double out, doub
   }
 }
 
-// Sums over the slots b = first, first + stride, ... in that order (I, inlet and
-// outlet flux, fuel), eight slots in flight: a short list waits for memory once.
-__device__ __forceinline__ void sum_slots(const double* partials, unsigned nb, unsigned first,
-                                          unsigned stride, double v[4]) {
+// Slots of one share of the combine by a block.
+constexpr unsigned SLOT_RUN = 256;
+// Slots that a lane has in flight: eight, so that a short list waits for memory
+// once; four in the kernels without species, whose 64 registers eight would spill.
+__host__ __device__ constexpr int slots_in_flight(int K) { return K == 0 ? 4 : 8; }
+
+// The warp's sums over the shares w0, w0 + nw, ... of the slots (I, inlet and
+// outlet flux and, FUEL, the fuel); valid in lane 0.  A lane adds every 32nd slot
+// of a share in order, F of them in flight.  Only the slots that there are cost an
+// addition: the FP64 pipe takes a warp's instruction every 16 cycles, and 32
+// additions by every warp of a block were 1.5 to 3 us of it whatever the list.
+template <bool FUEL, int F>
+__device__ __forceinline__ void sum_slots(const double* partials, unsigned nb, unsigned w0,
+                                          unsigned nw, double v[4]) {
+  const unsigned lane = threadIdx.x & 31;
   v[0] = v[1] = v[2] = v[3] = 0.0;
-  for (unsigned b = first; b < nb; b += 8 * stride) {
-    double2 a[8], c[8];
+  for (unsigned w = w0; w * SLOT_RUN < nb; w += nw) {
+#pragma unroll 1
+    for (unsigned s = w * SLOT_RUN; s < min(nb, (w + 1) * SLOT_RUN); s += 32 * F) {
+      double2 a[F], c[F];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const double2* p =
-          reinterpret_cast<const double2*>(partials + 4 * (size_t)(b + q * stride));
-      const bool in = b + q * stride < nb;
-      a[q] = in ? __ldcg(p) : make_double2(0.0, 0.0);
-      c[q] = in ? __ldcg(p + 1) : make_double2(0.0, 0.0);
-    }
+      for (int q = 0; q < F; ++q) {
+        const unsigned b = s + 32 * q + lane;
+        const double* p = partials + 4 * (size_t)b;
+        a[q] = c[q] = make_double2(0.0, 0.0);
+        if (b < nb) {
+          a[q] = __ldcg(reinterpret_cast<const double2*>(p));
+          if constexpr (FUEL) c[q] = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+          else c[q].x = __ldcg(p + 2);
+        }
+      }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      v[0] += a[q].x;
-      v[1] += a[q].y;
-      v[2] += c[q].x;
-      v[3] += c[q].y;
+      for (int q = 0; q < F; ++q) {
+        if (s + 32 * q >= nb) break;
+        v[0] += a[q].x;
+        v[1] += a[q].y;
+        v[2] += c[q].x;
+        if constexpr (FUEL) v[3] += c[q].y;
+      }
     }
   }
+#pragma unroll
+  for (int k = 0; k < (FUEL ? 4 : 3); ++k)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
 }
 
 // Combine the per-block partials of one step in a fixed order (strided sums,
 // then a fixed shuffle tree) and update the scalar state: by one warp.
+template <int F>
 __device__ __forceinline__ void combine_partials(const double* partials, unsigned nb,
                                                  DevScalars* scal, int p0_closed, bool is_init,
                                                  double init_P0, double eos_c,
                                                  double inv_rho_ref, double feed_c = 0.0) {
-  const int lane = threadIdx.x & 31;
   double v[4];
-  sum_slots(partials, nb, lane, 32, v);
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-  if (lane == 0)
+  if (feed_c > 0.0) sum_slots<true, F>(partials, nb, 0, 1, v);
+  else sum_slots<false, F>(partials, nb, 0, 1, v);
+  if ((threadIdx.x & 31) == 0)
     apply_sums(v[0], v[1], v[2], v[3], scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref,
                feed_c);
 }
 
 // The same for a fixed P0 by a whole block (every thread calls it; `sh` holds
 // 96 doubles and is free again after the block's next barrier): one warp takes
-// 25 us over the 4,096 slots of a 2048 x 512 domain, and as the first block's
-// first warp it held up small launches.
+// 25 us over the 4,096 slots of a 2048 x 512 domain.  Up to SLOT_RUN slots are
+// left to the first warp; beyond, eight warps' shares are dealt to the warps that
+// there are, so that the sums are the same bits under every block size.
+template <int F>
 __device__ __forceinline__ void combine_partials_block(const double* partials, unsigned nb,
                                                        DevScalars* scal, double eos_c,
                                                        double inv_rho_ref, double* sh) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  double v[4];
-  sum_slots(partials, nb, threadIdx.x, blockDim.x, v);
+  const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (nb <= SLOT_RUN) {
+    if (wid == 0) combine_partials<F>(partials, nb, scal, 0, false, 0.0, eos_c, inv_rho_ref);
+    return;
+  }
+#pragma unroll 1
+  for (unsigned w = wid; w < 8 && w * SLOT_RUN < nb; w += blockDim.x / 32) {
+    double v[4];
+    sum_slots<false, F>(partials, nb, w, 8, v);
+    if (lane == 0)
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (lane == 0) sh[32 * k + wid] = v[k];
+      for (int k = 0; k < 3; ++k) sh[32 * k + w] = v[k];
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double w[3] = {0.0, 0.0, 0.0};
-    for (unsigned q = 0; q < blockDim.x / 32; ++q)
-      for (int k = 0; k < 3; ++k) w[k] += sh[32 * k + q];
-    apply_sums(w[0], w[1], w[2], 0.0, scal, 0, false, 0.0, eos_c, inv_rho_ref, 0.0);
+    double u[3] = {0.0, 0.0, 0.0};
+    for (unsigned q = 0; q < 8 && q * SLOT_RUN < nb; ++q)
+      for (int k = 0; k < 3; ++k) u[k] += sh[32 * k + q];
+    apply_sums(u[0], u[1], u[2], 0.0, scal, 0, false, 0.0, eos_c, inv_rho_ref, 0.0);
   }
 }
 
@@ -1238,7 +1263,7 @@ __device__ __forceinline__ void combine_partials_block(const double* partials, u
 // need P0 of the next step before it starts, so the warp that draws the last
 // arrival ticket combines at once (lane 0 fences its own writes before taking
 // the ticket; the other warps retire).  With a fixed P0 the combine is
-// deferred: block 0 of the next launch, or the on-demand finalize kernel,
+// deferred: the first block of the next launch, or the on-demand finalize kernel,
 // does it, and the step ends without a serial tail.
 // Write the sums into slot `bid`.
 __device__ __forceinline__ void write_partials(double sI, double sIn, double sOut,
@@ -1252,6 +1277,7 @@ __device__ __forceinline__ void write_partials(double sI, double sIn, double sOu
 }
 // Count `n` slots that this block has written; the block that completes the
 // `nb` slots combines them.  (First warp; the others pass.)
+template <int F>
 __device__ __forceinline__ void count_partials(double* partials, unsigned* counter,
                                                DevScalars* scal, int p0_closed, bool is_init,
                                                double init_P0, double eos_c, double inv_rho_ref,
@@ -1266,10 +1292,11 @@ __device__ __forceinline__ void count_partials(double* partials, unsigned* count
   last = __shfl_sync(0xffffffffu, last, 0);
   if (!last) return;
   __threadfence();
-  combine_partials(partials, nb, scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref, feed_c);
+  combine_partials<F>(partials, nb, scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref, feed_c);
   if (lane == 0) *counter = 0u;
 }
 // Publish into slot `bid` of `nb`; `now` combines at the last arrival.
+template <int F>
 __device__ __forceinline__ void publish_partials_at(double sI, double sIn, double sOut,
                                                     double* partials, unsigned* counter,
                                                     DevScalars* scal, int p0_closed, bool is_init,
@@ -1279,29 +1306,33 @@ __device__ __forceinline__ void publish_partials_at(double sI, double sIn, doubl
                                                     double feed_c = 0.0) {
   write_partials(sI, sIn, sOut, partials, bid, sF);
   if (now)
-    count_partials(partials, counter, scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref, 1u, nb,
-                   feed_c);
+    count_partials<F>(partials, counter, scal, p0_closed, is_init, init_P0, eos_c, inv_rho_ref, 1u,
+                      nb, feed_c);
 }
 
+template <int F>
 __device__ __forceinline__ void publish_partials(double sI, double sIn, double sOut,
                                                  double* partials, unsigned* counter,
                                                  DevScalars* scal, int p0_closed, bool is_init,
                                                  double init_P0, double eos_c,
                                                  double inv_rho_ref, double sF = 0.0,
                                                  double feed_c = 0.0) {
-  publish_partials_at(sI, sIn, sOut, partials, counter, scal, p0_closed, is_init, init_P0, eos_c,
-                      inv_rho_ref,
-                      blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z),
-                      gridDim.x * gridDim.y * gridDim.z, p0_closed || is_init || feed_c > 0.0, sF,
-                      feed_c);
+  publish_partials_at<F>(sI, sIn, sOut, partials, counter, scal, p0_closed, is_init, init_P0, eos_c,
+                         inv_rho_ref, blockIdx.x, gridDim.x, p0_closed || is_init || feed_c > 0.0,
+                         sF, feed_c);
 }
 
-// On-demand combine of the deferred partials of the last step (one block).
+// On-demand combine of the deferred partials of the last step (one block), to
+// the same bits as the next step's: by the block, or by its first warp (FP16
+// storage).
 static __global__ void __launch_bounds__(BLOCK)
 finalize_kernel(const double* partials, unsigned nb, DevScalars* scal, double eos_c,
-                double inv_rho_ref) {
+                double inv_rho_ref, int one_warp) {
   __shared__ double sh[96];
-  combine_partials_block(partials, nb, scal, eos_c, inv_rho_ref, sh);
+  if (!one_warp)
+    combine_partials_block<8>(partials, nb, scal, eos_c, inv_rho_ref, sh);
+  else if (threadIdx.x < 32)
+    combine_partials<8>(partials, nb, scal, 0, false, 0.0, eos_c, inv_rho_ref);
 }
 
 // ------------------------------------------------ runs of planes (3-D)
@@ -2094,25 +2125,46 @@ constexpr size_t step_smem_bytes() {
                          (DIM == 2 && K > 0 ? (K + 1) * T_::TX * T_::TY : 0));
 }
 
+// The previous step's deferred partials (fixed P0 only) are combined by the first
+// block, which with `lead` = 1 does nothing else: the launch then has one block
+// more than tiles, and no tile waits for the combine.  FP32: always so (in front of
+// its tile the combine made steps of up to 608 tiles, one wave, 2 to 4 us longer:
+// a 128 x 64 channel 10.9 us, 7.7 so; 400 x 200 bed 12.9, 10.0; several waves
+// equal); without species at compile time, as both forms in one kernel spill.
+// FP64: while an SM is left for it (a 128 x 64 channel 19.0 us a step, 18.0 so);
+// beyond, it moves tiles among the SMs, which the FP64 pipe bounds (400 x 160 bed, 260 tiles:
+// 97.7 us with the combine in front of the first tile, 102.4 in a block of its own).
+template <int K, class Real>
+__host__ __device__ constexpr bool always_lead() { return K == 0 && sizeof(Real) == 4; }
+
 template <int K, class Real, class T_>
 __global__ void __launch_bounds__(T_::NT, (MinBlocks<K, T_>::value))
 step_kernel(const __grid_constant__ Params<Real, K> P, const State<Real, Real> S, int p0_closed,
-            const double* __restrict__ prev_partials, unsigned prev_nb) {
+            const double* __restrict__ prev_partials, unsigned prev_nb, int lead) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* pl = reinterpret_cast<Real*>(smem_raw);
   __shared__ double red_sh[128];
+  constexpr int F = slots_in_flight(K);
 
-  // deferred combine of the previous step's partials (fixed P0 only): block 0
-  // does it while the other blocks start on their cells
-  if (prev_partials && blockIdx.x == 0 && blockIdx.y == 0)
-    combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
-
+  int b = blockIdx.x, nb = gridDim.x;
+  if (prev_partials) {
+    constexpr int CF = always_lead<K, Real>() ? F : 8;
+    if (b == 0) {
+      combine_partials_block<CF>(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
+      if (always_lead<K, Real>() || lead) return;
+    }
+    const int off = always_lead<K, Real>() ? 1 : lead;
+    b -= off;
+    nb -= off;
+  }
+  const int gx = (P.nx + T_::TX - 1) / T_::TX;
   double sI, sIn, sOut, sF;
-  step_tile<K, Real, T_>(P, S, blockIdx.x, blockIdx.y, pl, red_sh, sI, sIn, sOut, sF);
+  step_tile<K, Real, T_>(P, S, b % gx, b / gx, pl, red_sh, sI, sIn, sOut, sF);
   // deterministic finish by the last block (closed P0, inlet feedback) or
   // deferred
-  publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
-                   P.inv_rho_ref, sF, P.feed ? P.feed_c : 0.0);
+  publish_partials_at<F>(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0,
+                         P.eos_c, P.inv_rho_ref, (unsigned)b, (unsigned)nb,
+                         p0_closed || (K > 0 && P.feed), sF, K > 0 && P.feed ? P.feed_c : 0.0);
 }
 
 // Persistent variant of the 2-D step: one grid of resident blocks walks the
@@ -2131,7 +2183,8 @@ step_persistent_kernel(const __grid_constant__ Params<Real, K> P, const State<Re
   __shared__ int next_sh[2];
 
   if (prev_partials && blockIdx.x == 0)
-    combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
+    combine_partials_block<slots_in_flight(K)>(prev_partials, prev_nb, S.scal, P.eos_c,
+                                               P.inv_rho_ref, red_sh);
 
   const int nbx = (P.nx + T_::TX - 1) / T_::TX;
   const int total = nbx * ((P.ny + T_::TY - 1) / T_::TY);
@@ -2148,9 +2201,10 @@ step_persistent_kernel(const __grid_constant__ Params<Real, K> P, const State<Re
     if (threadIdx.x == 0) next_sh[par] = (int)atomicAdd(ctr, 1u);
     double sI, sIn, sOut, sF;
     step_tile<K, Real, T_>(P, S, t % nbx, t / nbx, pl, red_sh, sI, sIn, sOut, sF);
-    publish_partials_at(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0,
-                        P.eos_c, P.inv_rho_ref, (unsigned)t, (unsigned)total,
-                        p0_closed != 0 || P.feed, sF, P.feed ? P.feed_c : 0.0);
+    publish_partials_at<slots_in_flight(K)>(
+        sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c, P.inv_rho_ref,
+        (unsigned)t, (unsigned)total, p0_closed || (K > 0 && P.feed), sF,
+        K > 0 && P.feed ? P.feed_c : 0.0);
   }
 }
 
@@ -2362,8 +2416,8 @@ init_kernel(const Params<Real, K> P, const State<Real, Store> S, const Real* __r
     acc = (Real(1) - S.phi[c]) / (T * invMw);
   }
   const double s = block_sum<Real>(acc, red_sh);
-  publish_partials(s, 0.0, 0.0, S.partials, S.counter, S.scal, 0, true, P0_init, P.eos_c,
-                   P.inv_rho_ref);
+  publish_partials<8>(s, 0.0, 0.0, S.partials, S.counter, S.scal, 0, true, P0_init, P.eos_c,
+                      P.inv_rho_ref);
 }
 
 // --------------------------------------------------- moments (get_fields)

@@ -379,7 +379,7 @@ struct LauncherImpl final : Launcher {
   using HalfTile = half_store::Tile<DIM>;
   dim3 step_grid() {
     const unsigned gx = (P.nx + 31) / 32, gy = (P.ny + step_ty() - 1) / step_ty();
-    if (DIM == 2) return dim3(gx, gy);
+    if (DIM == 2) return dim3(gx * gy);
     const int c = kHalf ? half_chunk() : first_chunk();
     return dim3(gx * gy * (c > 0 ? chunks_per_tile(P.nz, c) : (P.nz - c - 1) / -c));
   }
@@ -608,14 +608,18 @@ struct LauncherImpl final : Launcher {
     if constexpr (DIM == 3 && !kHalf) {
       return step_march<false>(B, cur, st, prev, true);
     } else {
-      const dim3 grid = step_grid();
+      dim3 grid = step_grid();
       if (step_blocks() > B.slots) return cudaErrorInvalidValue;
-      auto launch = [&](auto kern, int threads, size_t smem, auto... chunk) -> cudaError_t {
+      // one block more for the previous step's combine (see step_kernel)
+      const bool lead =
+          DIM == 2 && prev && (sizeof(Real) == 4 || (long long)grid.x < sm_count());
+      if (lead) ++grid.x;
+      auto launch = [&](auto kern, int threads, size_t smem, int last) -> cudaError_t {
         const cudaError_t e =
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         kern<<<grid, threads, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb,
-                                      chunk...);
+                                          last);
         return cudaGetLastError();
       };
       cudaError_t e;
@@ -625,15 +629,17 @@ struct LauncherImpl final : Launcher {
                    DIM == 3 ? half_chunk() : 0);
       } else if constexpr (sizeof(Real) == 4) {
         using T_ = Tile<V, 32, 8>;
-        e = launch(step_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>());
+        e = launch(step_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>(), lead);
       } else {
         using T8 = Tile<V, 32, 8>;
         using T4 = Tile<V, 32, 4>;
         using T2 = Tile<V, 32, 2>;
         const int ty = step_ty();
-        e = ty == 8 ? launch(step_kernel<K, Real, T8>, T8::NT, step_smem_bytes<2, K, Real, T8>())
-            : ty == 4 ? launch(step_kernel<K, Real, T4>, T4::NT, step_smem_bytes<2, K, Real, T4>())
-                      : launch(step_kernel<K, Real, T2>, T2::NT, step_smem_bytes<2, K, Real, T2>());
+        auto at = [&](auto t) {
+          using T_ = decltype(t);
+          return launch(step_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>(), lead);
+        };
+        e = ty == 8 ? at(T8()) : ty == 4 ? at(T4()) : at(T2());
       }
       if (e == cudaSuccess) B.last_nb = step_blocks();
       return e;
@@ -964,7 +970,8 @@ struct LauncherImpl final : Launcher {
   cudaError_t finalize(Buffers& B, cudaStream_t st) override {
     if (!B.pending) return cudaSuccess;
     finalize_kernel<<<1, BLOCK, 0, st>>>(B.partials + (size_t)4 * B.slots * B.last_parity,
-                                      (unsigned)B.last_nb, B.scal, P.eos_c, P.inv_rho_ref);
+                                         (unsigned)B.last_nb, B.scal, P.eos_c, P.inv_rho_ref,
+                                         kHalf ? 1 : 0);
     B.pending = 0;
     return cudaGetLastError();
   }

@@ -44,7 +44,8 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
   __shared__ double red_sh[128];
 
   if (prev_partials && blockIdx.x == 0) {
-    combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
+    combine_partials_block<slots_in_flight(K)>(prev_partials, prev_nb, S.scal, P.eos_c,
+                                               P.inv_rho_ref, red_sh);
     // the block's own sums go to red_sh next; a block without planes meets no
     // other barrier before them
     __syncthreads();
@@ -115,8 +116,9 @@ step3d_march_kernel(const __grid_constant__ Params<Real, K> P, const State<Real,
   }
   double sI, sIn, sOut, sF;
   block_sum4(accI, accIn, accOut, flux_block, fuel, K > 0 && P.feed, red_sh, sI, sIn, sOut, sF);
-  publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
-                   P.inv_rho_ref, sF, P.feed ? P.feed_c : 0.0);
+  publish_partials<slots_in_flight(K)>(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed,
+                                       false, 0.0, P.eos_c, P.inv_rho_ref, sF,
+                                       K > 0 && P.feed ? P.feed_c : 0.0);
 }
 
 }  // namespace pflb

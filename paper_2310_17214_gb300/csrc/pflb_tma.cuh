@@ -311,7 +311,8 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
   const float dP0r = scal_dP0r<float>(S.scal);
 
   if (prev_partials && blockIdx.x == 0)
-    combine_partials_block(prev_partials, prev_nb, S.scal, P.eos_c, P.inv_rho_ref, red_sh);
+    combine_partials_block<slots_in_flight(K)>(prev_partials, prev_nb, S.scal, P.eos_c,
+                                               P.inv_rho_ref, red_sh);
 
   // self-check of the alignment every TMA issue relies on (the same answer
   // in every thread): record it and skip all copies rather than fault
@@ -398,8 +399,9 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
 
   double sI, sIn, sOut, sF;
   block_sum4(accI, accIn, accOut, any_flux, fuel, K > 0 && P.feed, red_sh, sI, sIn, sOut, sF);
-  publish_partials(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
-                   P.inv_rho_ref, sF, P.feed ? P.feed_c : 0.0);
+  publish_partials<slots_in_flight(K)>(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed,
+                                       false, 0.0, P.eos_c, P.inv_rho_ref, sF,
+                                       K > 0 && P.feed ? P.feed_c : 0.0);
 }
 
 }  // namespace pflb

@@ -4,7 +4,12 @@ first block of the next launch (fixed P0).
 One plane: a 24 x 160 x 1 lattice has 20 tile-planes of 32 x 8 cells and 40
 partial slots, fewer planes than the resident grid of the z-march.
 
-Bars: the suite's, FP64 1e-10 and FP32 1e-4 relative to the oracle's scalars."""
+Reading the scalars combines the last step's sums at once instead of in the next
+launch: to the same bits, under every block size of the step (FP64 tiles of 2,
+4 and 8 rows, the z-march) and beside more than one share of 256 slots.
+
+Bars: the suite's, FP64 1e-10 and FP32 1e-4 relative to the oracle's scalars; the
+moment of reading moves no bit."""
 import numpy as np
 import pytest
 
@@ -47,3 +52,21 @@ def test_one_plane_scalars_match_oracle(precision, bar, kernel):
         assert all(r != 0.0 for r in ref)
         assert np.all(np.abs(np.subtract(got, ref)) <= bar * np.abs(ref)), (n, got, ref)
     d.close()
+
+
+@pytest.mark.parametrize("shape", [(2, 128, 64, 1), (2, 300, 120, 1), (2, 600, 500, 1),
+                                   (3, 40, 24, 20)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32_fp16"])
+def test_reading_the_scalars_moves_no_bit(precision, shape):
+    p, f = problem(*shape)
+    seen = []
+    for read in (False, True):
+        d = domain(p, f, precision)
+        for _ in range(20):
+            d.step(1)
+            if read:
+                d.scalars()
+        dg = d.diagnostics()
+        seen.append((d.scalars(), dg["flux_in_total"], dg["flux_out_total"]))
+        d.close()
+    assert seen[0] == seen[1]
