@@ -1078,7 +1078,9 @@ struct pflb_batch {
   void* entries = nullptr;        // device work list [n][entry_bytes]
   unsigned* tile_ctr = nullptr;   // tile counters, one per launch parity
   std::vector<unsigned char> host_entries;
-  int* tile_begin[BATCH_SHAPES] = {};  // device prefix sums per tile shape
+  std::vector<int> tiles[BATCH_SHAPES];  // tiles of each domain per tile shape
+  int* run_begin = nullptr;       // device prefix sums of the domains' runs of `run` tiles
+  int run = 1;
   int occ[BATCH_SHAPES] = {};
   int sms = 0;
   int cfg = 0, bps = 0, grid = 0;
@@ -1104,6 +1106,20 @@ int batch_grid(const pflb_batch* b, int cfg, int bps) {
   const int occ = b->occ[cfg];
   const int per = bps > 0 ? std::min(bps, occ) : occ;
   return std::max(1, per * b->sms);
+}
+
+// The grid of a tile shape, the runs that suit it and their prefix sums.
+cudaError_t batch_configure(pflb_batch* b, int cfg, int bps) {
+  b->cfg = cfg;
+  b->bps = bps;
+  b->grid = batch_grid(b, cfg, bps);
+  const std::vector<int>& t = b->tiles[cfg];
+  b->run = b->L0->batch_run(t.data(), (int)t.size(), b->grid);
+  std::vector<int> begin(t.size() + 1, 0);
+  for (size_t i = 0; i < t.size(); ++i) begin[i + 1] = begin[i] + (t[i] + b->run - 1) / b->run;
+  const cudaError_t e = cudaMemcpyAsync(b->run_begin, begin.data(), begin.size() * sizeof(int),
+                                        cudaMemcpyHostToDevice, b->stream);
+  return e == cudaSuccess ? cudaStreamSynchronize(b->stream) : e;
 }
 
 // Rebuild the work list when a domain was stepped on its own since the last
@@ -1158,7 +1174,7 @@ int batch_finish(pflb_batch* b, int nsteps) {
 }
 
 cudaError_t batch_launch_one(pflb_batch* b, int flip) {
-  return b->L0->batch_launch(b->entries, b->tile_begin[b->cfg], (int)b->doms.size(), b->cfg,
+  return b->L0->batch_launch(b->entries, b->run_begin, b->run, (int)b->doms.size(), b->cfg,
                              b->grid, flip, b->tile_ctr, b->stream);
 }
 
@@ -1241,31 +1257,24 @@ int pflb_create_batch(pflb_domain** domains, int n, pflb_batch** out) {
       cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess)
     return bad(PFLB_ERR_CUDA, "stream creation failed");
   if (cudaMalloc(&b->entries, b->host_entries.size()) != cudaSuccess ||
+      cudaMalloc((void**)&b->run_begin, (n + 1) * sizeof(int)) != cudaSuccess ||
       cudaMalloc((void**)&b->tile_ctr, 2 * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(b->tile_ctr, 0, 2 * sizeof(unsigned)) != cudaSuccess)
     return bad(PFLB_ERR_OOM, "device allocation failed");
   for (int cfg = 0; cfg < BATCH_SHAPES; ++cfg) {
-    std::vector<int> tb(n + 1, 0);
+    long long total = 0;
     for (int i = 0; i < n; ++i) {
       const pflb_domain_desc& D = domains[i]->desc;
       const long long t = (long long)((D.nx + batch_tx(cfg) - 1) / batch_tx(cfg)) *
                           ((D.ny + batch_ty(cfg) - 1) / batch_ty(cfg));
       if (t > domains[i]->B.slots) return bad(PFLB_ERR_STATE, "reduction slots too few");
-      if ((long long)tb[i] + t > (1LL << 30)) return bad(PFLB_ERR_ARG, "batch too large");
-      const int run = b->L0->batch_run();  // tiles a block draws at a time
-      tb[i + 1] = tb[i] + (int)((t + run - 1) / run);
+      if ((total += t) > (1LL << 30)) return bad(PFLB_ERR_ARG, "batch too large");
+      b->tiles[cfg].push_back((int)t);
     }
-    if (cudaMalloc((void**)&b->tile_begin[cfg], (n + 1) * sizeof(int)) != cudaSuccess)
-      return bad(PFLB_ERR_OOM, "device allocation failed");
-    if (cudaMemcpy(b->tile_begin[cfg], tb.data(), (n + 1) * sizeof(int),
-                   cudaMemcpyHostToDevice) != cudaSuccess)
-      return bad(PFLB_ERR_CUDA, "upload failed");
     b->occ[cfg] = b->L0->batch_occupancy(cfg);
     if (b->occ[cfg] < 1) return bad(PFLB_ERR_CUDA, "batch kernel has no occupancy");
   }
-  b->cfg = 0;
-  b->bps = 0;
-  b->grid = batch_grid(b, 0, 0);
+  if (batch_configure(b, 0, 0) != cudaSuccess) return bad(PFLB_ERR_CUDA, "upload failed");
   *out = b;
   return PFLB_OK;
 }
@@ -1289,9 +1298,8 @@ int pflb_batch_set_config(pflb_batch* b, int tile, int blocks_per_sm) {
   if (cudaStreamSynchronize(b->stream) != cudaSuccess)
     return bfail(b, PFLB_ERR_CUDA, "synchronise failed");
   drop_graphs(b);
-  b->cfg = tile;
-  b->bps = blocks_per_sm;
-  b->grid = batch_grid(b, tile, blocks_per_sm);
+  if (batch_configure(b, tile, blocks_per_sm) != cudaSuccess)
+    return bfail(b, PFLB_ERR_CUDA, "upload failed");
   return PFLB_OK;
 }
 
@@ -1369,8 +1377,7 @@ int pflb_batch_destroy(pflb_batch* b) {
   cudaSetDevice(b->device);
   if (b->stream) cudaStreamSynchronize(b->stream);
   drop_graphs(b);
-  for (int* p : b->tile_begin)
-    if (p) cudaFree(p);
+  if (b->run_begin) cudaFree(b->run_begin);
   if (b->entries) cudaFree(b->entries);
   if (b->tile_ctr) cudaFree(b->tile_ctr);
   if (b->ev) cudaEventDestroy(b->ev);

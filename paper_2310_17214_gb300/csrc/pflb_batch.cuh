@@ -3,7 +3,7 @@
 // Every domain keeps its own arrays; the batch holds a device work list with
 // one entry per domain (its lattice-unit parameters, the two ping-pong views
 // of its state, its P0 mode) and, per tile shape, the prefix sums of the
-// domains' counts of runs of BATCH_RUN consecutive tiles.  A launch is a
+// domains' counts of runs of consecutive tiles.  A launch is a
 // resident grid that draws runs from an atomic counter (one per launch parity;
 // each launch clears the other one for the next launch), so blocks that draw
 // cheap tiles take more of them and no SM idles at the end.  A block finds a
@@ -16,9 +16,8 @@
 //
 // Runs of tiles: the blocks advance through the tiles side by side, so with
 // single tiles nearly every draw changed domain (a search, a copy of the
-// parameters, two barriers) and every tile paid a fence.  48 beds: 288 us a step
-// drawing one tile at a time, 257 with runs of 4; runs of 2 and 8 up to 3 %
-// slower than 4.
+// parameters, two barriers) and every tile paid a fence.  The length of the runs
+// follows the work there is (LauncherImpl::batch_run).
 #pragma once
 
 #include "pflb_half.cuh"
@@ -36,12 +35,13 @@ template <class Real> struct BatchShape<Real, 2> { using T = Tile<typename VecOf
 __host__ __device__ constexpr int batch_tx(int cfg) { return cfg == 2 ? 64 : 32; }
 __host__ __device__ constexpr int batch_ty(int cfg) { return cfg == 0 ? 8 : (cfg == 1 ? 16 : 4); }
 
+// most tiles of a run
 constexpr int BATCH_RUN = 4;
 
 template <int K, class Real, class T_>
 __global__ void __launch_bounds__(T_::NT, (MinBlocks<K, T_>::value))
 batch_step_kernel(const BatchDom<K, Real, Real>* __restrict__ doms,
-                  const int* __restrict__ run_begin, int ndom, int flip,
+                  const int* __restrict__ run_begin, int run, int ndom, int flip,
                   unsigned* __restrict__ run_ctr) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* pl = reinterpret_cast<Real*>(smem_raw);
@@ -83,9 +83,9 @@ batch_step_kernel(const BatchDom<K, Real, Real>* __restrict__ doms,
     // draw the next run now; a tile's staging barrier publishes it
     par ^= 1;
     if (threadIdx.x == 0) next_sh[par] = (int)atomicAdd(run_ctr + flip, 1u);
-    const int first = (r - __ldg(run_begin + lo)) * BATCH_RUN;
+    const int first = (r - __ldg(run_begin + lo)) * run;
 #pragma unroll 1
-    for (int i = 0; i < BATCH_RUN; ++i) {
+    for (int i = 0; i < run; ++i) {
       const int nbx = (Psh.nx + T_::TX - 1) / T_::TX;
       if (first + i >= nbx * ((Psh.ny + T_::TY - 1) / T_::TY)) break;
       double sI, sIn, sOut, sF;
@@ -94,8 +94,9 @@ batch_step_kernel(const BatchDom<K, Real, Real>* __restrict__ doms,
       write_partials(sI, sIn, sOut, Ssh.partials, (unsigned)(first + i));
     }
     const int nb = ((Psh.nx + T_::TX - 1) / T_::TX) * ((Psh.ny + T_::TY - 1) / T_::TY);
-    count_partials<slots_in_flight(K)>(Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0, Psh.eos_c,
-                   Psh.inv_rho_ref, (unsigned)min(BATCH_RUN, nb - first), (unsigned)nb);
+    count_partials<slots_in_flight(K)>(Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0,
+                                       Psh.eos_c, Psh.inv_rho_ref, (unsigned)min(run, nb - first),
+                                       (unsigned)nb);
   }
 }
 

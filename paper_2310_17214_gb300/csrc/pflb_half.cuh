@@ -1263,7 +1263,7 @@ template <> struct BatchShape<2> { using T = Tile<2, 64, 1>; };
 template <int K, class Real, class Store, class T_>
 __global__ void __launch_bounds__(BLOCK, (T_::RPT > 1 ? 3 : 4))
 batch_step_kernel(const BatchDom<K, Real, Store>* __restrict__ doms,
-                  const int* __restrict__ tile_begin, int ndom, int flip,
+                  const int* __restrict__ tile_begin, int /* run: 1 */, int ndom, int flip,
                   unsigned* __restrict__ tile_ctr) {
   using PL = Plane<Real, K, T_::HP, n_mom<2, Store>()>;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -117,11 +117,12 @@ struct Launcher {
   virtual void batch_entry(void* dst, const Buffers& B, int cur) const = 0;
   // resident blocks per SM of the batch kernel for tile shape cfg
   virtual int batch_occupancy(int cfg) const = 0;
-  virtual cudaError_t batch_launch(const void* entries, const int* run_begin, int ndom, int cfg,
-                                   int grid, int flip, unsigned* tile_ctr,
+  virtual cudaError_t batch_launch(const void* entries, const int* run_begin, int run, int ndom,
+                                   int cfg, int grid, int flip, unsigned* tile_ctr,
                                    cudaStream_t st) const = 0;
-  // consecutive tiles of one domain that a block of the batch draws at a time
-  virtual int batch_run() const = 0;
+  // consecutive tiles of one domain that a block draws at a time, of n domains of
+  // tiles[i] tiles on a grid of `grid` blocks
+  virtual int batch_run(const int* tiles, int n, int grid) const = 0;
   // domains can share a batch when their keys are equal (same kernel)
   virtual int batch_key() const = 0;
   // bound of the kernels' device waits (SM clock cycles)
@@ -726,28 +727,48 @@ struct LauncherImpl final : Launcher {
     }
   }
   template <int CFG>
-  static cudaError_t batch_launch_cfg(const void* entries, const int* run_begin, int ndom,
+  static cudaError_t batch_launch_cfg(const void* entries, const int* run_begin, int run, int ndom,
                                       int grid, int flip, unsigned* ctr, cudaStream_t st) {
     return with_batch_kernel<CFG>([&](auto kern, int threads, size_t smem) {
       kern<<<grid, threads, smem, st>>>(static_cast<const BatchDom<K, Real, Store>*>(entries),
-                                        run_begin, ndom, flip, ctr);
+                                        run_begin, run, ndom, flip, ctr);
       return cudaGetLastError();
     });
   }
-  cudaError_t batch_launch(const void* entries, const int* run_begin, int ndom, int cfg, int grid,
-                           int flip, unsigned* ctr, cudaStream_t st) const override {
+  cudaError_t batch_launch(const void* entries, const int* run_begin, int run, int ndom, int cfg,
+                           int grid, int flip, unsigned* ctr, cudaStream_t st) const override {
     if constexpr (kBatchable) {
       switch (cfg) {
-        case 0: return batch_launch_cfg<0>(entries, run_begin, ndom, grid, flip, ctr, st);
-        case 1: return batch_launch_cfg<1>(entries, run_begin, ndom, grid, flip, ctr, st);
-        case 2: return batch_launch_cfg<2>(entries, run_begin, ndom, grid, flip, ctr, st);
+        case 0: return batch_launch_cfg<0>(entries, run_begin, run, ndom, grid, flip, ctr, st);
+        case 1: return batch_launch_cfg<1>(entries, run_begin, run, ndom, grid, flip, ctr, st);
+        case 2: return batch_launch_cfg<2>(entries, run_begin, run, ndom, grid, flip, ctr, st);
         default: return cudaErrorInvalidValue;
       }
     } else {
       return cudaErrorNotSupported;
     }
   }
-  int batch_run() const override { return kHalf ? 1 : BATCH_RUN; }
+  // FP32: of 1, 2 and BATCH_RUN tiles the run whose rounds of the grid, each as long
+  // as the run and a sixth of a tile for the draw, take the least.  Runs of four all
+  // along: 5 beds of 297 tiles 40 us a step, 17.6 in single draws, 24.7 in twos; 20
+  // beds of 4,120 tiles 51.2 / 50.4 / 46.9 in runs of 1 / 2 / 4; 48 beds of 34,279
+  // tiles 297 / 261 / 266.  FP64: single draws, as a tile is long beside a draw (48
+  // beds of 2,384 tiles 314 / 320 / 316; 1 bed of 91 tiles 51 / 87 / 152).
+  int batch_run(const int* tiles, int n, int grid) const override {
+    if (kHalf || sizeof(Real) == 8) return 1;
+    int best = 1;
+    double least = 0.0;
+    for (int run = 1; run <= BATCH_RUN; run *= 2) {
+      long long runs = 0;
+      for (int i = 0; i < n; ++i) runs += (tiles[i] + run - 1) / run;
+      const double t = double((runs + grid - 1) / grid) * (run + 1.0 / 6.0);
+      if (run == 1 || t < least) {
+        best = run;
+        least = t;
+      }
+    }
+    return best;
+  }
   int batch_key() const override { return kBatchable ? 100 + MODE : -1; }
 
   bool tma_usable(const Buffers& B, int cur) {
