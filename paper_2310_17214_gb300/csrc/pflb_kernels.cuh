@@ -479,38 +479,35 @@ __device__ __forceinline__ bool solve_pivoted(LA (*A)[n], LA* r) {
 // a J x J system (two reactions: 2 x 2) in place of the (K + 1) x (K + 1) one.
 //
 // FP64 domains do everything in FP64.  FP32 domains (LA = float) keep state,
-// rates and right-hand side in FP64 and take the Jacobian, the solve and the
-// update test in FP32: a direction off by about cond(A) x 6e-8 of itself still
+// rates and right-hand side in FP64, form the factors of the Jacobian (powers,
+// products before a factor, rate and heat derivatives, 1 / cp) in FP64 and
+// narrow them, and take their products, the matrix, the solve and the update
+// test in FP32: a direction off by about cond(A) x 6e-8 of itself still
 // contracts, and the iteration stops where the FP64 right-hand side puts the
 // root.  The FP64 pipe bounds this pre-pass (one warp instruction every 16
 // cycles per SM, conversions and comparisons included), so the FP32 part takes
 // its own copies of the constants, signs are tested on the bit pattern, and
 // what an iteration needs only if another follows is left to that one (most
 // cells are cold and take one).  2048 x 512 cells of the two-step bed, FP32
-// domain, a step: 1.28 ms with the 7 x 7 system, 1.20 with the 2 x 2 one, 0.74
-// so.
+// domain, a step: 1.28 ms with the 7 x 7 system, 0.81 so (0.74 with the factors
+// formed in FP32).
 
 // Power C^o of a concentration for the reaction orders that occur (1, 2, 1/2:
-// multiplications and a square root), pow() otherwise; the second form also
-// gives d = dC^o/dC for C > 0.
-template <class R>
-__device__ __forceinline__ R conc_power(R C, R o) {
-  if (o == R(1)) return C;
-  if (o == R(2)) return C * C;
-  if (o == R(0.5)) return sqrt(C);
-  return pow(C, o);
-}
-template <class R>
-__device__ __forceinline__ R conc_power(R C, R o, R& d) {
-  if (o == R(1)) { d = R(1); return C; }
-  if (o == R(2)) { d = R(2) * C; return C * C; }
+// multiplications and a square root), pow() otherwise,
+// with d = dC^o/dC for C > 0, in the precision LA of the Jacobian.
+template <class R, class LA>
+__device__ __forceinline__ R conc_power(R C, R o, LA& d) {
+  if (o == R(1)) { d = LA(1); return C; }
+  if (o == R(2)) { d = LA(2) * LA(C); return C * C; }
   if (o == R(0.5)) {
     const R s = sqrt(C);
-    d = s > R(0) ? R(0.5) / s : R(0);
+    d = s > R(0) ? LA(0.5) / LA(s) : LA(0);
     return s;
   }
-  d = C > R(0) ? o * R(pow(C, o - R(1))) : R(0);
-  return pow(C, o);
+  const R p = pow(C, o);
+  if constexpr (sizeof(R) == sizeof(LA)) d = C > R(0) ? o * R(pow(C, o - R(1))) : LA(0);
+  else d = C > R(0) ? LA(o * p / C) : LA(0);
+  return p;
 }
 
 // Rate constants of reaction j at T; k_r = 0 for an irreversible reaction.  FP32
@@ -547,14 +544,13 @@ __device__ __forceinline__ void rate_constants(const Chem32<K>& c, int j, float 
 }
 
 // One Newton iteration's rates: q_j in Real, its derivatives dq_j/dT (qT) and
-// along the reactions (Q[j][i]) in LA.  C_k = rho Y_k / M_k (in Real and in LA)
-// and dC_k = rho / M_k are 0 where Y_k <= 0.  Species of order 0 are skipped
-// (the orders are uniform).
+// along the reactions (Q[j][i]) in LA, from factors in Real.  C_k = rho Y_k / M_k
+// and dC_k = rho / M_k are 0 where Y_k <= 0.  Species of order 0 are skipped (the
+// orders are uniform).
 template <int K, int J, class Real, class LA, class Chem, class ChemL>
 __device__ __forceinline__ void reaction_rates(const Chem& c, const ChemL& cl, const Real* C,
-                                               const LA* CL, const LA* dC, Real T, Real invT,
-                                               Real* q, LA* qT, LA (*Q)[J]) {
-  const LA iT = LA(invT);
+                                               const LA* dC, Real T, Real invT, Real* q, LA* qT,
+                                               LA (*Q)[J]) {
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     q[j] = Real(0);
@@ -564,52 +560,47 @@ __device__ __forceinline__ void reaction_rates(const Chem& c, const ChemL& cl, c
     if (!c.active(j)) continue;
     Real kk[2];
     rate_constants<K>(c, j, T, invT, kk[0], kk[1]);
+    Real dl = vmul(vfma(c.EaR[j], invT, c.b[j]), invT);  // d ln k / dT, forward
+    Real dT = Real(0);
 #pragma unroll
     for (int dir = 0; dir < 2; ++dir) {
       if (dir == 1 && !c.rev[j]) break;
-      const Real k0 = dir == 0 ? kk[0] : -kk[1];
-      // d ln k / dT of this direction
-      LA dl = vmul(vfma(cl.EaR[j], iT, cl.b[j]), iT);
-      if (dir == 1) dl = vfma(-vfma(cl.dH_R[j], iT, cl.dn[j]), iT, dl);
+      if (dir == 1) dl = vfma(-vfma(c.dH_R[j], invT, c.dn[j]), invT, dl);
       // prefix / suffix products: the product without factor k, no division
-      LA Pw[K], pre[K], Dp[K], prodL = LA(k0), suf = LA(1);
-      Real prod = k0;
+      LA Pw[K], pre[K], Dp[K], suf = LA(1);
+      Real prod = dir == 0 ? kk[0] : -kk[1];
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        const auto o = dir == 0 ? cl.order[j][k] : cl.rorder[j][k];
-        if (o == LA(0)) continue;
-        pre[k] = prodL;
-        Pw[k] = conc_power(CL[k], o, Dp[k]);
-        prodL = vmul(prodL, Pw[k]);
-        if constexpr (sizeof(Real) != sizeof(LA))
-          prod = vmul(prod, conc_power(C[k], dir == 0 ? c.order[j][k] : c.rorder[j][k]));
+        const Real o = dir == 0 ? c.order[j][k] : c.rorder[j][k];
+        if (o == Real(0)) continue;
+        pre[k] = LA(prod);
+        const Real p = conc_power(C[k], o, Dp[k]);
+        Pw[k] = LA(p);
+        prod = vmul(prod, p);
       }
-      if constexpr (sizeof(Real) == sizeof(LA)) prod = prodL;
       q[j] = vadd(q[j], prod);
-      qT[j] = vfma(prodL, dl, qT[j]);
+      dT = vfma(prod, dl, dT);
 #pragma unroll
       for (int k = K - 1; k >= 0; --k) {
-        const auto o = dir == 0 ? cl.order[j][k] : cl.rorder[j][k];
-        if (o == LA(0)) continue;
+        const Real o = dir == 0 ? c.order[j][k] : c.rorder[j][k];
+        if (o == Real(0)) continue;
         const LA d = vmul(vmul(pre[k], suf), vmul(Dp[k], dC[k]));
         suf = vmul(suf, Pw[k]);
 #pragma unroll
         for (int i = 0; i < J; ++i) Q[j][i] = vfma(d, cl.Ms[i][k], Q[j][i]);
       }
     }
+    qT[j] = LA(dT);
   }
 }
 
 // The system of one iteration (see above): matrix A, right-hand side r and the
-// row a of dT.  h0 = h / rho in LA, rhs_j = hr q_j - xi_j, R.
+// row a of dT.  hr = h / rho, icp = 1 / cp, w = hr (sum_j H_j q_j) / cp^2,
+// rhs_j = hr q_j - xi_j, R.
 template <int K, int J, class LA, class ChemL>
-__device__ __forceinline__ void reaction_system(const ChemL& cl, LA hr, LA icp, const LA* q,
+__device__ __forceinline__ void reaction_system(const ChemL& cl, LA hr, LA icp, LA w,
                                                 const LA* rhs, const LA* qT, const LA (*Q)[J], LA R,
                                                 LA (*A)[J], LA* r, LA* a) {
-  LA Hq = LA(0);
-#pragma unroll
-  for (int j = 0; j < J; ++j) Hq = vfma(cl.H[j], q[j], Hq);
-  const LA w = vmul(vmul(hr, Hq), vmul(icp, icp));
 #pragma unroll
   for (int i = 0; i < J; ++i) a[i] = vfma(-w, cl.cM[i], vmul(cl.H[i], icp));
 #pragma unroll
@@ -620,6 +611,12 @@ __device__ __forceinline__ void reaction_system(const ChemL& cl, LA hr, LA icp, 
       A[j][i] = vfma(-hr, vfma(-qT[j], a[i], Q[j][i]), LA(i == j ? 1 : 0));
   }
 }
+
+// The least LA not below a threshold x: a value in LA is below it when it is
+// below x.
+template <class LA> __device__ __forceinline__ LA threshold(double x);
+template <> __device__ __forceinline__ double threshold<double>(double x) { return x; }
+template <> __device__ __forceinline__ float threshold<float>(double x) { return __double2float_ru(x); }
 
 // z > 0 by its bits (a comparison would go through the FP64 pipe)
 __device__ __forceinline__ bool positive(double z) { return __double_as_longlong(z) > 0; }
@@ -642,7 +639,7 @@ __device__ __forceinline__ void chem_be_newton(const Chem64<K>& c, const ChemL& 
 #pragma unroll 1
     for (int sub = 0; sub < nsub && ok == 0; ++sub) {
       const double Ts = vadd(T0, accT);
-      const LA tolT = LA(1e-13) * LA(Ts);
+      const LA tolT = threshold<LA>(1e-13 * Ts), tolY = threshold<LA>(1e-13);
       double xi[J], T = Ts, z[K];
 #pragma unroll
       for (int j = 0; j < J; ++j) xi[j] = 0.0;
@@ -651,35 +648,34 @@ __device__ __forceinline__ void chem_be_newton(const Chem64<K>& c, const ChemL& 
       ok = -1;
 #pragma unroll 1
       for (int it = 0; it < 30; ++it) {
-        double Cc[K], q[J], R = 0.0;
-        LA CL[K], dC[K], zL[K], cpL = LA(0), qT[J], Q[J][J], A[J][J], r[J], a[J], qL[J], rhs[J];
+        double C[K], q[J], R = 0.0, cp = 0.0, Hq = 0.0;
+        LA dC[K], qT[J], Q[J][J], A[J][J], r[J], a[J], rhs[J];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-          const bool pos = positive(z[k]);
-          zL[k] = LA(z[k]);
-          dC[k] = pos ? LA(rho) * cl.invM[k] : LA(0);
-          CL[k] = vmul(zL[k], dC[k]);
-          if constexpr (sizeof(LA) != 8) {
-            Cc[k] = 0.0;
-            if (c.used & (1 << k)) Cc[k] = pos ? vmul(z[k], vmul(rho, c.invM[k])) : 0.0;
+          C[k] = 0.0;
+          dC[k] = LA(0);
+          if ((c.used & (1 << k)) && positive(z[k])) {
+            const double d = vmul(rho, c.invM[k]);
+            dC[k] = LA(d);
+            C[k] = vmul(z[k], d);
           }
-          cpL = vfma(zL[k], cl.cp[k], cpL);
+          cp = vfma(z[k], c.cp[k], cp);
         }
-        reaction_rates<K, J, double, LA>(c, cl, Cc, CL, dC, T, 1.0 / T, q, qT, Q);
+        reaction_rates<K, J, double, LA>(c, cl, C, dC, T, 1.0 / T, q, qT, Q);
+        const double icp = 1.0 / cp;
         if (it > 0) {  // R = 0 in the first iteration
-          double cp = 0.0, Hxi = 0.0;
-#pragma unroll
-          for (int k = 0; k < K; ++k) cp = vfma(z[k], c.cp[k], cp);
+          double Hxi = 0.0;
 #pragma unroll
           for (int j = 0; j < J; ++j) Hxi = vfma(c.H[j], xi[j], Hxi);
-          R = vsub(vsub(Ts, T), Hxi / cp);
+          R = vfma(-Hxi, icp, vsub(Ts, T));
         }
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-          qL[j] = LA(q[j]);
+          Hq = vfma(c.H[j], q[j], Hq);
           rhs[j] = LA(vfma(hr, q[j], -xi[j]));
         }
-        reaction_system<K, J, LA>(cl, hrL, LA(1) / cpL, qL, rhs, qT, Q, LA(R), A, r, a);
+        const double w = vmul(vmul(hr, Hq), vmul(icp, icp));
+        reaction_system<K, J, LA>(cl, hrL, LA(icp), LA(w), rhs, qT, Q, LA(R), A, r, a);
         if (!solve_pivoted<J, LA>(A, r)) break;
         LA ar = LA(0);
 #pragma unroll
@@ -699,7 +695,7 @@ __device__ __forceinline__ void chem_be_newton(const Chem64<K>& c, const ChemL& 
           for (int j = 0; j < J; ++j) e = vfma(cl.Ms[j][k], r[j], e);
           e = fabs(e);
           if (!(e == e)) bad = true;
-          if (!(e < LA(1e-13))) done = false;
+          if (!(e < tolY)) done = false;
         }
         if (bad || !positive(T)) break;
         if (done) { ok = 0; break; }
@@ -760,7 +756,7 @@ __device__ __forceinline__ void chem_be_newton32(const Chem32<K>& c, float T0, c
       for (int it = 0; it < 30; ++it) {
         const float T = vadd(Ts, dTs);
         if (!(T > 0.f)) break;
-        float Cc[K], dC[K], q[J], rhs[J], qT[J], Q[J][J], A[J][J], r[J], a[J], cp = 0.f;
+        float Cc[K], dC[K], q[J], rhs[J], qT[J], Q[J][J], A[J][J], r[J], a[J], cp = 0.f, Hq = 0.f;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
           const float z = vadd(vadd(Y0[k], acc[k]), d[k]);
@@ -768,16 +764,18 @@ __device__ __forceinline__ void chem_be_newton32(const Chem32<K>& c, float T0, c
           Cc[k] = vmul(z, dC[k]);
           cp = vfma(z, c.cp[k], cp);
         }
-        reaction_rates<K, J, float, float>(c, c, Cc, Cc, dC, T, 1.f / T, q, qT, Q);
+        reaction_rates<K, J, float, float>(c, c, Cc, dC, T, 1.f / T, q, qT, Q);
         const float icp = 1.f / cp;
         float Hxi = 0.f;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
           Hxi = vfma(c.H[j], xi[j], Hxi);
+          Hq = vfma(c.H[j], q[j], Hq);
           rhs[j] = vfma(hr, q[j], -xi[j]);
         }
         const float R = vfma(-Hxi, icp, -dTs);
-        reaction_system<K, J, float>(c, hr, icp, q, rhs, qT, Q, R, A, r, a);
+        const float w = vmul(vmul(hr, Hq), vmul(icp, icp));
+        reaction_system<K, J, float>(c, hr, icp, w, rhs, qT, Q, R, A, r, a);
         if (!solve_pivoted<J, float>(A, r)) break;
         float dTn = R;
 #pragma unroll
