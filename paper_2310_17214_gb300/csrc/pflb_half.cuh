@@ -5,7 +5,9 @@
 // of the residual, 7e-5 of the velocity after 40 steps of the 2-D bed), so this
 // path keeps its own operation order: a run reproduces the runs it has to be
 // compared with, checkpoints written earlier included.  The FP32 / FP64 path
-// (two cells per thread in FP32, written-out rounding) is in pflb_kernels.cuh.
+// (two cells per thread in FP32, written-out rounding) is in pflb_kernels.cuh;
+// what does not touch that order (the lattices, the packed operations, the
+// reductions, the runs of planes) is shared with it.
 #pragma once
 
 #include "pflb_kernels.cuh"
@@ -13,46 +15,24 @@
 namespace pflb {
 namespace half_store {
 
+using Real = float;
+using Store = __half;
+
 // Tile shape: TX x (256 / TX) RPT cells per plane, 256 threads; in 2-D every
-// thread can own RPT rows and issues the population loads of its cells before
-// the staging barrier (PREFETCH), so the two load phases overlap.  Measured
-// on GB300 for the single-domain step: 32 x 8 with one row per thread is
-// fastest (two rows spill at the 64-register cap); the prefetch helps the
-// FP16-stored path.  The batched step lets its autotuner pick among shapes.
-// 3-D blocks march over a run of planes.
+// thread can own RPT rows and issues the population loads of its inner cells
+// before the staging barrier, so the two load phases overlap.  The single-domain
+// step takes 32 x 8 with one row per thread (two rows spill at the 64-register
+// cap); the batched step lets its autotuner pick among shapes.  3-D blocks march
+// over a run of planes.
 template <int DIM, int TXv = 32, int RPTv = 1> struct Tile {
   static constexpr int RPT = RPTv;
-  static constexpr bool PREFETCH = DIM == 2;
   static constexpr int TX = TXv, TY = (256 / TXv) * RPT;
   static constexpr int HX = TX + 2, HY = TY + 2, HP = HX * HY;
   static constexpr int NPL = DIM == 3 ? 3 : 1;  // staged planes
 };
 
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  uint64_t d;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)),
-      "l"(f2_bits(c)));
-  return f2_of(d);
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-  uint64_t d;
-  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
-  return f2_of(d);
-}
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-  uint64_t d;
-  asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
-  return f2_of(d);
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  uint64_t d;
-  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
-  return f2_of(d);
-}
-__device__ __forceinline__ float2 splat2(float a) { return make_float2(a, a); }
-
 // Viscosity: Sutherland (Sec. 4, eq. muT) or constant, lattice units.
-template <class Real, int K>
+template <int K>
 __device__ __forceinline__ Real viscosity(const Params<Real, K>& P, Real T) {
   if (!P.sutherland) return P.mu_lat;
   Real t = T * P.inv_suth_T;
@@ -67,7 +47,7 @@ __device__ __forceinline__ Real viscosity(const Params<Real, K>& P, Real T) {
 // Phi_kj = (1 + sqrt(mu_k / mu_j) (M_j / M_k)^(1/4))^2 / (sqrt(8) sqrt(1 + M_k / M_j)),
 // lambda = (sum_k X_k lambda_k + 1 / sum_k X_k / lambda_k) / 2 with
 // lambda_k = mu_k (1.32 cv_k + 1.77 R / M_k).
-template <class Real, int K>
+template <int K>
 __device__ __forceinline__ void transport(const Params<Real, K>& P, Real T, const Real* Y,
                                           Real invMw, Real cp, Real& mu, Real& lam) {
   if constexpr (K > 0) {
@@ -105,7 +85,7 @@ __device__ __forceinline__ void transport(const Params<Real, K>& P, Real T, cons
   lam = mu * cp * P.inv_Pr;
 }
 
-template <class Real, int K>
+template <int K>
 __device__ __forceinline__ Real mixture_invMw(const Params<Real, K>& P, const Real* Y) {
   if constexpr (K == 0) {
     return Real(1) / P.M0;
@@ -117,7 +97,7 @@ __device__ __forceinline__ Real mixture_invMw(const Params<Real, K>& P, const Re
   }
 }
 
-template <class Real, int K>
+template <int K>
 __device__ __forceinline__ Real mixture_cp(const Params<Real, K>& P, const Real* Y) {
   if constexpr (K == 0) {
     return P.cp0;
@@ -131,7 +111,7 @@ __device__ __forceinline__ Real mixture_cp(const Params<Real, K>& P, const Real*
 
 // Explicit Arrhenius rates (Sec. 3.2.2 eq. 8, Sec. 3.3 eq. 9), per lattice
 // step per rho_ref: om[k] = omega_k dt / rho_ref, omT likewise (J/kg).
-template <class Real, int K>
+template <int K>
 __device__ __forceinline__ void rates(const Params<Real, K>& P, Real T, const Real* Y, Real rho,
                                       Real invT, Real* om, Real& omT) {
 #pragma unroll
@@ -175,7 +155,7 @@ __device__ __forceinline__ void rates(const Params<Real, K>& P, Real T, const Re
 
 // First-order part w_i (P + 3 c_i . j) of direction i at the source cell
 // (global index src, offset (dx, dy, dz) from the pulling cell).
-template <int DIM, class Real, class MA>
+template <int DIM, class MA>
 __device__ __forceinline__ Real first_order(const MA& A, int i, int src, int dx, int dy, int dz) {
   using L = Lattice<DIM>;
   Real cj = 0;
@@ -187,7 +167,7 @@ __device__ __forceinline__ Real first_order(const MA& A, int i, int src, int dx,
   return Real(L::w(i)) * (A.mom(0, src, dx, dy, dz) + Real(3) * cj);
 }
 
-template <class Real, int K>
+template <int K>
 __device__ __forceinline__ Real inlet_u(const Params<Real, K>& P, Real u, const int xyz[3],
                                         int dim) {
   if (P.inlet_parabolic != 1) return u;
@@ -201,19 +181,17 @@ __device__ __forceinline__ Real inlet_u(const Params<Real, K>& P, Real u, const 
 }
 
 // The cell's own post-collision population of direction ib (bounce-back).
-template <int DIM, class Real, class Store, int K, class MA>
+template <int DIM, int K, class MA>
 __device__ __forceinline__ Real own_pop(const Params<Real, K>& P, const State<Real, Store>& S,
                                         int c, int ib, const MA& mom) {
   const Real r = Codec<Store, Real>::raw(S.g_in + (size_t)ib * P.N + c);
-  if constexpr (IsHalf<Store>::value)
-    return Codec<Store, Real>::dec(r, Real(Lattice<DIM>::w(ib)) * P.g_inv_scale,
-                                   half_store::first_order<DIM, Real>(mom, ib, c, 0, 0, 0));
-  else return r;
+  return Codec<Store, Real>::dec(r, Real(Lattice<DIM>::w(ib)) * P.g_inv_scale,
+                                 half_store::first_order<DIM>(mom, ib, c, 0, 0, 0));
 }
 
 // Half-way bounce-back with the wall velocity for the directions entering
 // through face F, when the cell lies on it (on) and it is a wall.
-template <int DIM, int F, class Real, class Store, int K, class MA>
+template <int DIM, int F, int K, class MA>
 __device__ __forceinline__ void wall_pops(const Params<Real, K>& P, const State<Real, Store>& S,
                                           int c, bool on, Real rho_c, Real* gin, const MA& mom) {
   using L = Lattice<DIM>;
@@ -225,7 +203,7 @@ __device__ __forceinline__ void wall_pops(const Params<Real, K>& P, const State<
     Real cu = 0;
 #pragma unroll
     for (int b = 0; b < DIM; ++b) cu += Real(L::c(i, b)) * P.wall_u[F][b];
-    gin[i] = half_store::own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom) +
+    gin[i] = half_store::own_pop<DIM>(P, S, c, L::opp(i), mom) +
              Real(2) * Real(L::w(i)) * rho_c * cu;
   }
 }
@@ -240,12 +218,11 @@ __device__ __forceinline__ void wall_pops(const Params<Real, K>& P, const State<
 // (moving walls add 2 w rho c.u_w), the inlet as a moving wall with the inlet
 // velocity and inlet density, the outlet as anti-bounce-back at P_h = 0 with
 // wall velocity uw.
-template <int DIM, class Real, class Store, int K, class MA>
+template <int DIM, int K, class MA>
 __device__ __forceinline__ void pull(const Params<Real, K>& P, const State<Real, Store>& S, int c,
                                      const int xyz[3], Real rho_c, Real rho_in, const Real* uw,
                                      Real* gin, const MA& mom) {
   using L = Lattice<DIM>;
-  constexpr bool FO = IsHalf<Store>::value;  // residual storage: add the first-order part
   // cells off every domain face: fixed offsets from the cell (the common case)
   const bool inner = xyz[0] > 0 && xyz[0] < P.nx - 1 && xyz[1] > 0 && xyz[1] < P.ny - 1 &&
                      (DIM == 2 || (xyz[2] > 0 && xyz[2] < P.nz - 1));
@@ -256,10 +233,8 @@ __device__ __forceinline__ void pull(const Params<Real, K>& P, const State<Real,
       const int cx = L::c(i, 0), cy = L::c(i, 1), cz = DIM == 3 ? L::c(i, 2) : 0;
       const int src = c - cx - cy * sy - cz * sz;
       const Real r = Codec<Store, Real>::raw(S.g_in + (size_t)i * P.N + src);
-      if constexpr (FO)
-        gin[i] = Codec<Store, Real>::dec(r, Real(L::w(i)) * P.g_inv_scale,
-                                         half_store::first_order<DIM, Real>(mom, i, src, -cx, -cy, -cz));
-      else gin[i] = r;
+      gin[i] = Codec<Store, Real>::dec(r, Real(L::w(i)) * P.g_inv_scale,
+                                       half_store::first_order<DIM>(mom, i, src, -cx, -cy, -cz));
     }
     return;
   }
@@ -284,10 +259,8 @@ __device__ __forceinline__ void pull(const Params<Real, K>& P, const State<Real,
     const int src = sx + P.nx * (sy + P.ny * sz);
     const Real r = Codec<Store, Real>::raw(S.g_in + (size_t)i * P.N + src);
     // a periodic source: the staged halo holds its image at the same offset
-    if constexpr (FO)
-      gin[i] = Codec<Store, Real>::dec(r, Real(L::w(i)) * P.g_inv_scale,
-                                       half_store::first_order<DIM, Real>(mom, i, src, -cx, -cy, -cz));
-    else gin[i] = r;
+    gin[i] = Codec<Store, Real>::dec(r, Real(L::w(i)) * P.g_inv_scale,
+                                     half_store::first_order<DIM>(mom, i, src, -cx, -cy, -cz));
   }
   // non-periodic faces the cell lies on
   const bool f0 = x == 0 && !per0, f1 = x == P.nx - 1 && !per1;
@@ -305,7 +278,7 @@ __device__ __forceinline__ void pull(const Params<Real, K>& P, const State<Real,
       Real cu = 0;
 #pragma unroll
       for (int a = 0; a < DIM; ++a) cu += Real(L::c(i, a)) * uw[a];
-      gin[i] = -half_store::own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom) +
+      gin[i] = -half_store::own_pop<DIM>(P, S, c, L::opp(i), mom) +
                Real(L::w(i)) * (pb2 + rho_c * (Real(3) * cu * cu - uu));
     }
   }
@@ -315,7 +288,7 @@ __device__ __forceinline__ void pull(const Params<Real, K>& P, const State<Real,
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
       if (L::c(i, 0) != 1) continue;
-      gin[i] = half_store::own_pop<DIM, Real, Store>(P, S, c, L::opp(i), mom) +
+      gin[i] = half_store::own_pop<DIM>(P, S, c, L::opp(i), mom) +
                Real(2) * Real(L::w(i)) * rho_in * ui;
     }
   }
@@ -331,29 +304,24 @@ __device__ __forceinline__ void pull(const Params<Real, K>& P, const State<Real,
 }
 
 // ------------------------------------------------ staged tile (smem)
-// Fields per staged cell: T, phi_s, rho, kappa_T = phi_f lambda, mu, f_D
-// (diffusivity factor), Ts, phi_f rho f_D, then Y_k.
-enum { F_T = 0, F_PHI, F_RHO, F_KT, F_MU, F_FD, F_TS, F_RF, F_Y0 };
-
-template <class Real, int K, int HP, int NM = 0>
+// Fields per staged cell as in the other step, then the moments (P, j).
+template <int DIM, int K, int HP>
 struct Plane {
-  Real f[F_Y0 + K + NM][HP];  // NM moment fields (P, j) after the species
+  Real f[F_Y0 + K + DIM + 1][HP];
 };
 
 // Stage plane z (may be -1 or nz: ghost plane) of the block's tile with its
 // xy halo.  Out-of-domain halo cells follow the ghost rules: periodic faces
 // wrap; otherwise the adjacent cell's values, with the inlet state (T_in,
 // Y_in) on the inlet face and the wall temperature on a wall that has one.
-template <int DIM, class Real, class Store, int K, int HP, class T_ = Tile<DIM>,
-          int NM = n_mom<DIM, Store>()>
+template <int DIM, int K, class T_>
 __device__ __forceinline__ void stage_plane(const Params<Real, K>& P, const State<Real, Store>& S,
-                                            Plane<Real, K, HP, NM>& pl, int x0, int y0, int z,
+                                            Plane<DIM, K, T_::HP>& pl, int x0, int y0, int z,
                                             Real P0) {
-  static_assert(T_::HP == HP, "plane and tile shape disagree");
   // tiles whose halo lies inside the lattice need no ghost rules
   const bool inner = x0 >= 1 && y0 >= 1 && x0 + T_::TX < P.nx && y0 + T_::TY < P.ny &&
                      (DIM == 2 || (z >= 0 && z < P.nz));
-  for (int h = threadIdx.x; h < HP; h += blockDim.x) {
+  for (int h = threadIdx.x; h < T_::HP; h += blockDim.x) {
     const int hx = h % T_::HX, hy = h / T_::HX;
     int q[3] = {x0 - 1 + hx, y0 - 1 + hy, z};
     int ghost_face = -1;
@@ -411,38 +379,34 @@ __device__ __forceinline__ void stage_plane(const Params<Real, K>& P, const Stat
     pl.f[F_RF][h] = phif * rho * fD;
 #pragma unroll
     for (int k = 0; k < K; ++k) pl.f[F_Y0 + k][h] = Y[k];
-    if constexpr (NM > 0) {
 #pragma unroll
-      for (int a = 0; a < NM; ++a) pl.f[F_Y0 + K + a][h] = __ldg(S.M_in + (size_t)a * P.N + c);
-    }
+    for (int a = 0; a <= DIM; ++a) pl.f[F_Y0 + K + a][h] = __ldg(S.M_in + (size_t)a * P.N + c);
   }
 }
 
 // Staged-plane accessor: own and neighbour values of the staged fields and
-// properties (the populations come from global memory).
-template <int DIM, class Real, bool PRE = false, class TL = Tile<DIM>, int MF = 0,
-          bool STASH = false>
+// properties.  2-D: the populations may be in registers already (pre); 3-D: the
+// pulled populations wait in shared memory (st).  MF: the first moment field.
+template <int DIM, class TL, int MF>
 struct PlaneAcc {
   static constexpr int HP = TL::HP;
-  static constexpr bool has_pops = PRE;  // populations prefetched into registers
-  static constexpr bool kStash = STASH;  // pulled populations wait in shared memory
+  static constexpr bool has_pops = DIM == 2;
+  static constexpr bool kStash = DIM == 3;
   const Real* __restrict__ cen;
   const Real* __restrict__ zm;
   const Real* __restrict__ zp;
   int h;
   const Real* pre;
   bool pv;  // pre holds this cell's populations
-  Real* st; // stash, [Q][BLOCK] (STASH)
+  Real* st; // stash, [Q][BLOCK]
   __device__ __forceinline__ Real c(int f) const { return cen[f * HP + h]; }
   __device__ __forceinline__ Real n(int f, int a, int s) const {
     if (a == 0) return cen[f * HP + h + s];
     if (a == 1) return cen[f * HP + h + s * TL::HX];
     return (s < 0 ? zm : zp)[f * HP + h];
   }
-  template <class Store>
-  __device__ __forceinline__ Real pop(int i, Real) const { return PRE ? pre[i] : Real(0); }
-  // moment a of the staged cell at offset (dx, dy, dz) (FP16 storage; MF is
-  // the first moment field, src the cell's global index, unused here)
+  __device__ __forceinline__ Real pop(int i) const { return has_pops ? pre[i] : Real(0); }
+  // moment a of the staged cell at offset (dx, dy, dz)
   __device__ __forceinline__ Real mom(int a, int, int dx, int dy, int dz) const {
     const Real* p = dz < 0 ? zm : (dz > 0 ? zp : cen);
     return p[(MF + a) * HP + h + dx + dy * TL::HX];
@@ -454,7 +418,7 @@ struct PlaneAcc {
 // Per cell: (a1) pull + moments + implicit drag, (c) reaction source,
 // (b) FD transport of Y_k, T, Ts, low-Mach divergence, (a) source + BGK
 // collision + store, (d) contribution to the FP64 reduction.
-template <int DIM, int K, class Real, class Store, class Acc>
+template <int DIM, int K, class Acc>
 __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const State<Real, Store>& S,
                                             const Acc& A, int c, const int xyz[3], Real P0,
                                             Real dlnP0, Real dP0r, Real& fin, Real& fout) {
@@ -481,8 +445,10 @@ __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const Stat
   const Real invT = fdiv(Real(1), T0);
 
   // cells on a non-periodic face (their pull takes the boundary rules)
-  bool edge = (xyz[0] == 0 && P.bc[0] != BC_PERIODIC) || (xyz[0] == P.nx - 1 && P.bc[1] != BC_PERIODIC) ||
-              (xyz[1] == 0 && P.bc[2] != BC_PERIODIC) || (xyz[1] == P.ny - 1 && P.bc[3] != BC_PERIODIC);
+  bool edge = (xyz[0] == 0 && P.bc[0] != BC_PERIODIC) ||
+              (xyz[0] == P.nx - 1 && P.bc[1] != BC_PERIODIC) ||
+              (xyz[1] == 0 && P.bc[2] != BC_PERIODIC) ||
+              (xyz[1] == P.ny - 1 && P.bc[3] != BC_PERIODIC);
   if (DIM == 3)
     edge = edge || (xyz[2] == 0 && P.bc[4] != BC_PERIODIC) ||
            (xyz[2] == P.nz - 1 && P.bc[5] != BC_PERIODIC);
@@ -495,7 +461,6 @@ __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const Stat
     for (int k = 0; k < K; ++k) Yin[k] = P.Y_in[k];
     rho_in = fdiv(P0 * P.eos_cr, P.T_in * half_store::mixture_invMw(P, Yin));
   }
-  constexpr bool FO = IsHalf<Store>::value;  // FP16 residual storage
   Real gin[Q];
   Real u[3] = {0, 0, 0}, uw[3] = {0, 0, 0}, mraw[3] = {0, 0, 0};
   const bool outlet_cell = P.bc[1] == BC_OUTLET && xyz[0] == P.nx - 1;
@@ -504,12 +469,11 @@ __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const Stat
     if (Acc::has_pops && A.pv) {  // populations prefetched for this cell
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        // prefetched values are raw stored numbers (scaled residuals with FP16)
-        gin[i] = A.template pop<Store>(i, Real(L::w(i)) * P.g_inv_scale);
-        if constexpr (FO)
-          gin[i] = Codec<Store, Real>::dec(gin[i], Real(L::w(i)) * P.g_inv_scale,
-                                           half_store::first_order<DIM, Real>(A, i, 0, -L::c(i, 0), -L::c(i, 1),
-                                                                  DIM == 3 ? -L::c(i, 2) : 0));
+        // prefetched values are the scaled residuals as stored
+        gin[i] = Codec<Store, Real>::dec(
+            A.pop(i), Real(L::w(i)) * P.g_inv_scale,
+            half_store::first_order<DIM>(A, i, 0, -L::c(i, 0), -L::c(i, 1),
+                                         DIM == 3 ? -L::c(i, 2) : 0));
       }
     } else {
       half_store::pull<DIM>(P, S, c, xyz, rho, rho_in, uw, gin, A);
@@ -573,36 +537,38 @@ __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const Stat
       fm[a] = Real(0.5) * (rf0 + at(F_RF, a, -1));
       fp[a] = Real(0.5) * (rf0 + at(F_RF, a, +1));
     }
-    // FP32: species in pairs with packed f32x2 arithmetic; the last one of an
-    // odd count (and every species in FP64) one at a time
-    constexpr int KP = sizeof(Real) == 4 ? (K / 2) * 2 : 0;
+    // species in pairs with packed f32x2 arithmetic, the last one of an odd count
+    // by itself
+    constexpr int KP = (K / 2) * 2;
     if constexpr (KP > 0) {
-      float2 sx2[3] = {half_store::splat2(0.f), half_store::splat2(0.f), half_store::splat2(0.f)}, sYm2 = half_store::splat2(0.f);
-      const float2 prf = half_store::splat2(-phif * rho), pf = half_store::splat2(phif), ip = half_store::splat2(iphr);
+      const float2 zero = splat<float2>(0.f);
+      float2 sx2[3] = {zero, zero, zero}, sYm2 = zero;
+      const float2 prf = splat<float2>(-phif * rho), pf = splat<float2>(phif);
+      const float2 ip = splat<float2>(iphr);
 #pragma unroll
       for (int k = 0; k < KP; k += 2) {
         const float2 y0 = make_float2(Y0[k], Y0[k + 1]);
-        float2 adv = half_store::splat2(0.f), dif = half_store::splat2(0.f), cen = half_store::splat2(0.f);
+        float2 adv = zero, dif = zero, cen = zero;
 #pragma unroll
         for (int a = 0; a < DIM; ++a) {
-          const float2 dm = half_store::sub2(y0, make_float2(at(F_Y0 + k, a, -1), at(F_Y0 + k + 1, a, -1)));
-          const float2 dp = half_store::sub2(make_float2(at(F_Y0 + k, a, +1), at(F_Y0 + k + 1, a, +1)), y0);
-          adv = half_store::fma2(half_store::splat2(u[a]), u[a] > 0.f ? dm : dp, adv);
-          dif = half_store::fma2(half_store::splat2(fp[a]), dp, dif);
-          dif = half_store::fma2(half_store::splat2(-fm[a]), dm, dif);
-          const float2 sd = half_store::add2(dp, dm);
-          cen = half_store::fma2(half_store::splat2(u[a]), sd, cen);
-          sx2[a] = half_store::fma2(make_float2(P.cpD[k], P.cpD[k + 1]), sd, sx2[a]);
+          const float2 dm = vsub(y0, make_float2(at(F_Y0 + k, a, -1), at(F_Y0 + k + 1, a, -1)));
+          const float2 dp = vsub(make_float2(at(F_Y0 + k, a, +1), at(F_Y0 + k + 1, a, +1)), y0);
+          adv = vfma(splat<float2>(u[a]), u[a] > 0.f ? dm : dp, adv);
+          dif = vfma(splat<float2>(fp[a]), dp, dif);
+          dif = vfma(splat<float2>(-fm[a]), dm, dif);
+          const float2 sd = vadd(dp, dm);
+          cen = vfma(splat<float2>(u[a]), sd, cen);
+          sx2[a] = vfma(make_float2(P.cpD[k], P.cpD[k + 1]), sd, sx2[a]);
         }
-        float2 dY = half_store::fma2(prf, adv, half_store::fma2(make_float2(P.Dlat[k], P.Dlat[k + 1]), dif,
-                                        half_store::mul2(pf, make_float2(om[k], om[k + 1]))));
-        dY = fluid_on ? half_store::mul2(dY, ip) : half_store::splat2(0.f);
-        const float2 yn = half_store::add2(y0, dY);
+        float2 dY = vfma(prf, adv, vfma(make_float2(P.Dlat[k], P.Dlat[k + 1]), dif,
+                                        vmul(pf, make_float2(om[k], om[k + 1]))));
+        dY = fluid_on ? vmul(dY, ip) : splat<float2>(0.f);
+        const float2 yn = vadd(y0, dY);
         Yn[k] = yn.x;
         Yn[k + 1] = yn.y;
         // material increment: the step's increment plus u.grad Y_k (central)
-        const float2 dm2 = fluid_on ? half_store::fma2(half_store::splat2(0.5f), cen, dY) : half_store::splat2(0.f);
-        sYm2 = half_store::fma2(make_float2(P.invM[k], P.invM[k + 1]), dm2, sYm2);
+        const float2 dm2 = fluid_on ? vfma(splat<float2>(0.5f), cen, dY) : splat<float2>(0.f);
+        sYm2 = vfma(make_float2(P.invM[k], P.invM[k + 1]), dm2, sYm2);
       }
 #pragma unroll
       for (int a = 0; a < DIM; ++a) sx[a] += sx2[a].x + sx2[a].y;
@@ -726,26 +692,21 @@ __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const Stat
   const Real B = omega * rho3;
   const Real uu15 = Real(1.5) * uu;
   const Real keep = Real(1) - omega;
-  // FP16 storage: the post-collision moments of this cell in closed form
+  // the post-collision moments of this cell in closed form
   // (sum_i w_i e_i = 0, sum_i w_i x_i = u.G, sum_i w_i c_i e_i = u,
   // sum_i w_i c_i x_i = F / 3 on the isotropic lattice); any values would do,
   // since readers add back exactly what is subtracted here, but these leave
   // a residual of second order in u
-  Real Pst = 0, jst[3] = {0, 0, 0};
-  if constexpr (FO) {
-    Pst = keep * sg + A0 + src_w * (uH - uF);
+  const Real Pst = keep * sg + A0 + src_w * (uH - uF);
+  Real jst[3] = {0, 0, 0};
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) jst[a] = keep * mraw[a] + B * u[a] + src_w * CS2 * F[a];
-  }
-  // FP32 updates a direction and its opposite together with packed f32x2
-  // arithmetic (c.u, c.H, c.F of the opposite are the negated ones); the rest
-  // direction, and every direction in FP64, one at a time
-  constexpr bool PAIRS = sizeof(Real) == 4;
+  for (int a = 0; a < DIM; ++a) jst[a] = keep * mraw[a] + B * u[a] + src_w * CS2 * F[a];
+  // a direction and its opposite are updated together with packed f32x2
+  // arithmetic (c.u, c.H, c.F of the opposite are the negated ones), the rest
+  // direction by itself
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
-    if constexpr (PAIRS) {
-      if (L::opp(i) < i) continue;  // done with its opposite
-    }
+    if (L::opp(i) < i) continue;  // done with its opposite
     Real cu = 0, cH = 0, cF = 0, cj = 0;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
@@ -754,40 +715,37 @@ __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const Stat
     }
     Real gi = gin[i];
     if constexpr (Acc::kStash) gi = A.st[i * BLOCK + threadIdx.x];
-    if constexpr (PAIRS) {
-      if (i > 0) {
-        const int j = L::opp(i);
-        Real gj = gin[j];
-        if constexpr (Acc::kStash) gj = A.st[j * BLOCK + threadIdx.x];
-        const float2 cu2 = make_float2(cu, -cu);
-        const float2 e = half_store::fma2(cu2, half_store::fma2(cu2, half_store::splat2(4.5f), half_store::splat2(3.f)), half_store::splat2(-uu15));
-        const float2 x = half_store::fma2(half_store::sub2(make_float2(cH, -cH), half_store::splat2(uH)), e,
-                              half_store::sub2(make_float2(cF, -cF), half_store::splat2(uF)));
-        float2 t = half_store::fma2(half_store::splat2(B), e, half_store::splat2(A0));
-        t = half_store::fma2(half_store::splat2(src_w), x, t);
-        const float w = float(L::w(i));
-        float2 g = half_store::fma2(half_store::splat2(keep), make_float2(gi, gj), half_store::mul2(half_store::splat2(w), t));
-        if constexpr (FO)
-          g = half_store::sub2(g, half_store::mul2(half_store::splat2(w), half_store::fma2(half_store::splat2(3.f), make_float2(cj, -cj), half_store::splat2(Pst))));
-        Codec<Store, Real>::store(S.g_out + (size_t)i * P.N + c, g.x,
-                                  P.g_scale * Real(1.0 / L::w(i)));
-        Codec<Store, Real>::store(S.g_out + (size_t)j * P.N + c, g.y,
-                                  P.g_scale * Real(1.0 / L::w(j)));
-        continue;
-      }
+    if (i > 0) {
+      const int j = L::opp(i);
+      Real gj = gin[j];
+      if constexpr (Acc::kStash) gj = A.st[j * BLOCK + threadIdx.x];
+      const float2 cu2 = make_float2(cu, -cu);
+      const float2 e = vfma(cu2, vfma(cu2, splat<float2>(4.5f), splat<float2>(3.f)),
+                            splat<float2>(-uu15));
+      const float2 x = vfma(vsub(make_float2(cH, -cH), splat<float2>(uH)), e,
+                            vsub(make_float2(cF, -cF), splat<float2>(uF)));
+      float2 t = vfma(splat<float2>(B), e, splat<float2>(A0));
+      t = vfma(splat<float2>(src_w), x, t);
+      const float w = float(L::w(i));
+      float2 g = vfma(splat<float2>(keep), make_float2(gi, gj), vmul(splat<float2>(w), t));
+      g = vsub(g, vmul(splat<float2>(w), vfma(splat<float2>(3.f), make_float2(cj, -cj),
+                                              splat<float2>(Pst))));
+      Codec<Store, Real>::store(S.g_out + (size_t)i * P.N + c, g.x,
+                                P.g_scale * Real(1.0 / L::w(i)));
+      Codec<Store, Real>::store(S.g_out + (size_t)j * P.N + c, g.y,
+                                P.g_scale * Real(1.0 / L::w(j)));
+      continue;
     }
     const Real w = Real(L::w(i));
     const Real e = cu * (Real(3) + Real(4.5) * cu) - uu15;
     const Real x = (cH - uH) * e + (cF - uF);
     Real g = keep * gi + w * (A0 + B * e + src_w * x);
-    if constexpr (FO) g -= w * (Pst + Real(3) * cj);
+    g -= w * (Pst + Real(3) * cj);
     Codec<Store, Real>::store(S.g_out + (size_t)i * P.N + c, g, P.g_scale * Real(1.0 / L::w(i)));
   }
-  if constexpr (FO) {
-    S.M_out[c] = Pst;
+  S.M_out[c] = Pst;
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) S.M_out[(size_t)(1 + a) * P.N + c] = jst[a];
-  }
+  for (int a = 0; a < DIM; ++a) S.M_out[(size_t)(1 + a) * P.N + c] = jst[a];
 
   S.T_out[c] = Tn;
 #pragma unroll
@@ -802,23 +760,18 @@ __device__ __forceinline__ Real cell_update(const Params<Real, K>& P, const Stat
   return phif * fdiv(Real(1), Tn * half_store::mixture_invMw(P, Yn)) + Real(0) * Ph;
 }
 
-// Resident blocks per SM requested from the register allocator: 2-D FP32 /
-// FP16 storage at <= 64 registers (4 blocks), 3-D FP32 at <= 80 (3 blocks),
-// 3-D FP16 storage, whose decode holds the source cells' moments, at <= 128
-// (2 blocks); FP64 is bound by the FP64 pipe and keeps the registers it needs.
-template <int DIM, class Real, class Store> struct MinBlocks {
-  static constexpr int value =
-      sizeof(Real) == 8 ? (DIM == 3 ? 1 : 2) : (DIM == 2 ? 4 : (IsHalf<Store>::value ? 2 : 3));
-};
+// Resident blocks per SM asked of the register allocator: 4 in 2-D (64
+// registers); 2 in 3-D, whose decode holds the source cells' moments (128).
+template <int DIM> constexpr int min_blocks() { return DIM == 2 ? 4 : 2; }
 
 // One tile of the fused step (tile (bx, by) of the xy grid, planes z_begin to
 // z_end in 3-D): stages the tile's planes in `planes` (shared memory), updates its
 // cells and returns the block sums of the reduction in thread 0 (I, inlet
 // flux, outlet flux).  Every thread of the block calls it.
-template <int DIM, int K, class Real, class Store, class T_ = Tile<DIM>>
+template <int DIM, int K, class T_ = Tile<DIM>>
 __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<Real, Store>& S,
                                           int bx, int by, int z_begin, int z_end,
-                                          Plane<Real, K, T_::HP, n_mom<DIM, Store>()>* planes,
+                                          Plane<DIM, K, T_::HP>* planes,
                                           double* red_sh,
                                           double& sI, double& sIn, double& sOut) {
   const Real P0 = scal_P0<Real>(S.scal);
@@ -842,23 +795,18 @@ __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<
     Real pre[RPT][L::Q];
     bool pv[RPT];
 #pragma unroll
-    for (int r = 0; r < RPT; ++r) pv[r] = false;
-    if constexpr (T_::PREFETCH) {
+    for (int r = 0; r < RPT; ++r) {
+      const int yr = y0 + ty + r * RS;
+      pv[r] = x > 0 && x < P.nx - 1 && yr > 0 && yr < P.ny - 1;
+      if (pv[r]) {
+        const int c = x + P.nx * yr;
 #pragma unroll
-      for (int r = 0; r < RPT; ++r) {
-        const int yr = y0 + ty + r * RS;
-        const bool inner = x > 0 && x < P.nx - 1 && yr > 0 && yr < P.ny - 1;
-        pv[r] = inner;
-        if (inner) {
-          const int c = x + P.nx * yr;
-#pragma unroll
-          for (int i = 0; i < L::Q; ++i)
-            pre[r][i] = Codec<Store, Real>::raw(
-                S.g_in + (size_t)i * P.N + c - L::c(i, 0) - L::c(i, 1) * P.nx);
-        }
+        for (int i = 0; i < L::Q; ++i)
+          pre[r][i] = Codec<Store, Real>::raw(
+              S.g_in + (size_t)i * P.N + c - L::c(i, 0) - L::c(i, 1) * P.nx);
       }
     }
-    half_store::stage_plane<DIM, Real, Store, K, T_::HP, T_>(P, S, planes[0], x0, y0, 0, P0);
+    half_store::stage_plane<DIM, K, T_>(P, S, planes[0], x0, y0, 0, P0);
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < RPT; ++r) {
@@ -868,31 +816,29 @@ __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<
         const int xyz[3] = {x, yr, 0};
         const int hr = (ty + r * RS + 1) * T_::HX + (tx + 1);
         Real fi, fo;
-        const PlaneAcc<DIM, Real, T_::PREFETCH, T_, F_Y0 + K> A{&planes[0].f[0][0], nullptr,
-                                                                nullptr, hr, pre[r], pv[r],
-                                                                nullptr};
-        accI += half_store::cell_update<DIM, K, Real, Store>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
+        const PlaneAcc<DIM, T_, F_Y0 + K> A{&planes[0].f[0][0], nullptr, nullptr, hr, pre[r],
+                                            pv[r], nullptr};
+        accI += half_store::cell_update<DIM, K>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
         accIn += fi;
         accOut += fo;
       }
     }
   } else {
     // ring of three staged planes: slot (z mod 3)
-    half_store::stage_plane<DIM, Real, Store, K, T_::HP, T_>(P, S, planes[(z_begin + 2) % 3], x0, y0,
+    half_store::stage_plane<DIM, K, T_>(P, S, planes[(z_begin + 2) % 3], x0, y0,
                                                  z_begin - 1, P0);
-    half_store::stage_plane<DIM, Real, Store, K, T_::HP, T_>(P, S, planes[z_begin % 3], x0, y0, z_begin, P0);
+    half_store::stage_plane<DIM, K, T_>(P, S, planes[z_begin % 3], x0, y0, z_begin, P0);
     for (int z = z_begin; z < z_end; ++z) {
-      half_store::stage_plane<DIM, Real, Store, K, T_::HP, T_>(P, S, planes[(z + 1) % 3], x0, y0, z + 1, P0);
+      half_store::stage_plane<DIM, K, T_>(P, S, planes[(z + 1) % 3], x0, y0, z + 1, P0);
       __syncthreads();
       if (in_xy) {
         const int c = x + P.nx * (y + P.ny * z);
         const int xyz[3] = {x, y, z};
         Real fi, fo;
-        const PlaneAcc<DIM, Real, false, T_, F_Y0 + K, true> A{
-            &planes[z % 3].f[0][0], &planes[(z + 2) % 3].f[0][0],
-            &planes[(z + 1) % 3].f[0][0], h, nullptr, false,
-            reinterpret_cast<Real*>(planes + T_::NPL)};
-        accI += half_store::cell_update<DIM, K, Real, Store>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
+        const PlaneAcc<DIM, T_, F_Y0 + K> A{
+            &planes[z % 3].f[0][0], &planes[(z + 2) % 3].f[0][0], &planes[(z + 1) % 3].f[0][0], h,
+            nullptr, false, reinterpret_cast<Real*>(planes + T_::NPL)};
+        accI += half_store::cell_update<DIM, K>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
         accIn += fi;
         accOut += fo;
       }
@@ -904,12 +850,12 @@ __device__ __forceinline__ void step_tile(const Params<Real, K>& P, const State<
   block_sum3<Real>(accI, accIn, accOut, flux_block, red_sh, sI, sIn, sOut);
 }
 
-template <int DIM, int K, class Real, class Store>
-__global__ void __launch_bounds__(BLOCK, MinBlocks<DIM, Real, Store>::value)
+template <int DIM, int K>
+__global__ void __launch_bounds__(BLOCK, min_blocks<DIM>())
 step_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
             const double* __restrict__ prev_partials, unsigned prev_nb, int chunk) {
   using T_ = Tile<DIM>;
-  using PL = Plane<Real, K, T_::HP, n_mom<DIM, Store>()>;
+  using PL = Plane<DIM, K, T_::HP>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PL* planes = reinterpret_cast<PL*>(smem_raw);
   __shared__ double red_sh[96];
@@ -941,10 +887,10 @@ step_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
     z0 = r.z_begin;
     z1 = r.z_end;
   }
-  half_store::step_tile<DIM, K, Real, Store, T_>(P, S, bx, by, z0, z1, planes, red_sh, sI, sIn, sOut);
+  half_store::step_tile<DIM, K, T_>(P, S, bx, by, z0, z1, planes, red_sh, sI, sIn, sOut);
   // deterministic finish by the last block (closed P0) or deferred
-  publish_partials_at<4>(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0, P.eos_c,
-                         P.inv_rho_ref, (unsigned)b, (unsigned)nb, p0_closed);
+  publish_partials_at<4>(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0,
+                         P.eos_c, P.inv_rho_ref, (unsigned)b, (unsigned)nb, p0_closed);
 }
 
 // Persistent variant of the 2-D step: one grid of resident blocks walks the
@@ -952,13 +898,13 @@ step_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
 // clears the other one for the next step), so no block waits for a second
 // wave and cheap tiles do not leave SMs idle.  Reduction slots are the tile
 // indices, as in step_kernel.
-template <int DIM, int K, class Real, class Store, class T_>
-__global__ void __launch_bounds__(BLOCK, (sizeof(Real) == 8 ? 2 : (T_::RPT > 1 ? 3 : 4)))
+template <int DIM, int K, class T_>
+__global__ void __launch_bounds__(BLOCK, (T_::RPT > 1 ? 3 : 4))
 step_persistent_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
                        const double* __restrict__ prev_partials, unsigned prev_nb,
                        unsigned* __restrict__ tile_ctr, int parity) {
   static_assert(DIM == 2, "the persistent step walks 2-D tiles");
-  using PL = Plane<Real, K, T_::HP, n_mom<DIM, Store>()>;
+  using PL = Plane<DIM, K, T_::HP>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PL* planes = reinterpret_cast<PL*>(smem_raw);
   __shared__ double red_sh[96];
@@ -981,7 +927,7 @@ step_persistent_kernel(const Params<Real, K> P, const State<Real, Store> S, int 
     par ^= 1;
     if (threadIdx.x == 0) next_sh[par] = (int)atomicAdd(ctr, 1u);
     double sI, sIn, sOut;
-    half_store::step_tile<DIM, K, Real, Store, T_>(P, S, t % nbx, t / nbx, 0, 1, planes, red_sh, sI, sIn,
+    half_store::step_tile<DIM, K, T_>(P, S, t % nbx, t / nbx, 0, 1, planes, red_sh, sI, sIn,
                                        sOut);
     publish_partials_at<4>(sI, sIn, sOut, S.partials, S.counter, S.scal, p0_closed, false, 0.0,
                         P.eos_c, P.inv_rho_ref, (unsigned)t, (unsigned)total, p0_closed != 0);
@@ -989,9 +935,9 @@ step_persistent_kernel(const Params<Real, K> P, const State<Real, Store> S, int 
 }
 
 // staged planes, and in 3-D the stash of the pulled populations
-template <int DIM, int K, class Real, class Store, class T_ = Tile<DIM>>
+template <int DIM, int K, class T_ = Tile<DIM>>
 constexpr size_t step_smem_bytes() {
-  return sizeof(Plane<Real, K, T_::HP, n_mom<DIM, Store>()>) * T_::NPL +
+  return sizeof(Plane<DIM, K, T_::HP>) * T_::NPL +
          (DIM == 3 ? sizeof(Real) * Lattice<DIM>::Q * BLOCK : 0);
 }
 
@@ -1003,17 +949,17 @@ __host__ __device__ constexpr int march_field(int f) {
        : f == F_TS ? G_TS : f == F_RF ? G_RF : G_Y0 + (f - F_Y0);
 }
 
-template <int K, class Store>
-__host__ __device__ constexpr int march_nf() { return G_Y0 + K + n_mom<3, Store>(); }
+template <int K>
+__host__ __device__ constexpr int march_nf() { return G_Y0 + K + 4; }  // species, moments
 
-template <int K, class Real, class Store>
+template <int K>
 constexpr size_t march_smem_bytes() {
-  return sizeof(Real) * (3 * march_nf<K, Store>() * Tile<3>::HP + Lattice<3>::Q * BLOCK);
+  return sizeof(Real) * (3 * march_nf<K>() * Tile<3>::HP + Lattice<3>::Q * BLOCK);
 }
 
 // Accessor of cell_update over the march's staged planes; mu and f_D are the
 // cell's own values.
-template <class Real, int K, bool PRE>
+template <int K, bool PRE>
 struct MarchAcc {
   using TL = Tile<3>;
   static constexpr int HP = TL::HP;
@@ -1038,8 +984,7 @@ struct MarchAcc {
     if (a == 1) return cen[g + h + s * TL::HX];
     return (s < 0 ? zm : zp)[g + h];
   }
-  template <class S_>
-  __device__ __forceinline__ Real pop(int i, Real) const { return PRE ? pre[i] : Real(0); }
+  __device__ __forceinline__ Real pop(int i) const { return PRE ? pre[i] : Real(0); }
   __device__ __forceinline__ Real mom(int a, int, int dx, int dy, int dz) const {
     const Real* p = dz < 0 ? zm : (dz > 0 ? zp : cen);
     return p[(G_Y0 + K + a) * HP + h + dx + dy * TL::HX];
@@ -1048,13 +993,12 @@ struct MarchAcc {
 
 // Stage plane z (may be -1 or nz: ghost plane) of the tile at (x0, y0) with
 // its xy halo into `pl` ([NF][HP]), with the ghost rules of stage_plane.
-template <class Real, class Store, int K>
+template <int K>
 __device__ __forceinline__ void march_stage(const Params<Real, K>& P, const State<Real, Store>& S,
                                             Real* __restrict__ pl, int x0, int y0, int z,
                                             Real P0) {
   using T_ = Tile<3>;
   constexpr int HP = T_::HP;
-  constexpr int NM = n_mom<3, Store>();
   const bool inner = x0 >= 1 && y0 >= 1 && x0 + T_::TX < P.nx && y0 + T_::TY < P.ny && z >= 0 &&
                      z < P.nz;
   for (int h = threadIdx.x; h < HP; h += blockDim.x) {
@@ -1113,18 +1057,16 @@ __device__ __forceinline__ void march_stage(const Params<Real, K>& P, const Stat
     pl[G_RF * HP + h] = phif * rho * fD;
 #pragma unroll
     for (int k = 0; k < K; ++k) pl[(G_Y0 + k) * HP + h] = Y[k];
-    if constexpr (NM > 0) {
 #pragma unroll
-      for (int a = 0; a < NM; ++a)
-        pl[(G_Y0 + K + a) * HP + h] = __ldg(S.M_in + (size_t)a * P.N + c);
-    }
+    for (int a = 0; a < 4; ++a)
+      pl[(G_Y0 + K + a) * HP + h] = __ldg(S.M_in + (size_t)a * P.N + c);
   }
 }
 
 // The 19 pulls of cell (x, y, z) with periodic faces wrapped; false (and
 // nothing loaded) for a cell on a non-periodic face, whose pull needs the
 // boundary rules.
-template <class Real, class Store, int K>
+template <int K>
 __device__ __forceinline__ bool march_prefetch(const Params<Real, K>& P,
                                                const State<Real, Store>& S, int x, int y, int z,
                                                Real* __restrict__ out) {
@@ -1150,21 +1092,14 @@ __device__ __forceinline__ bool march_prefetch(const Params<Real, K>& P,
   return true;
 }
 
-// Resident blocks per SM asked of the register allocator: FP32 storage fits
-// 80 registers (3 blocks); the FP16 decode needs more (2 blocks, no spills).
-template <class Real, class Store, bool PRE> struct MarchBlocks {
-  static constexpr int value =
-      sizeof(Real) == 8 ? 1 : ((PRE || IsHalf<Store>::value) ? 2 : 3);
-};
-
-template <int K, class Real, class Store, bool PRE>
-__global__ void __launch_bounds__(BLOCK, (MarchBlocks<Real, Store, PRE>::value))
+template <int K, bool PRE>
+__global__ void __launch_bounds__(BLOCK, min_blocks<3>())
 step3d_march_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_closed,
                     const double* __restrict__ prev_partials, unsigned prev_nb) {
   using T_ = Tile<3>;
   using L = Lattice<3>;
   constexpr int HP = T_::HP;
-  constexpr int NF = march_nf<K, Store>();
+  constexpr int NF = march_nf<K>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* planes = reinterpret_cast<Real*>(smem_raw);  // [3][NF][HP]
   __shared__ double red_sh[96];
@@ -1197,19 +1132,19 @@ step3d_march_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_
                  (x0 + T_::TX >= P.nx && P.bc[1] == BC_OUTLET);
 
     __syncthreads();  // the previous column is done with the planes
-    half_store::march_stage<Real, Store, K>(P, S, planes + ((z_begin + 2) % 3) * NF * HP, x0, y0,
+    half_store::march_stage<K>(P, S, planes + ((z_begin + 2) % 3) * NF * HP, x0, y0,
                                 z_begin - 1, P0);
-    half_store::march_stage<Real, Store, K>(P, S, planes + (z_begin % 3) * NF * HP, x0, y0, z_begin, P0);
+    half_store::march_stage<K>(P, S, planes + (z_begin % 3) * NF * HP, x0, y0, z_begin, P0);
     Real pre[L::Q], nxt[L::Q];
     bool have = false, have_nxt = false;
     if constexpr (PRE) {
-      if (in_xy) have = half_store::march_prefetch<Real, Store, K>(P, S, x, y, z_begin, pre);
+      if (in_xy) have = half_store::march_prefetch<K>(P, S, x, y, z_begin, pre);
     }
     for (int z = z_begin; z < z_end; ++z) {
-      half_store::march_stage<Real, Store, K>(P, S, planes + ((z + 1) % 3) * NF * HP, x0, y0, z + 1, P0);
+      half_store::march_stage<K>(P, S, planes + ((z + 1) % 3) * NF * HP, x0, y0, z + 1, P0);
       if constexpr (PRE) {
         have_nxt = in_xy && z + 1 < z_end &&
-                   half_store::march_prefetch<Real, Store, K>(P, S, x, y, z + 1, nxt);
+                   half_store::march_prefetch<K>(P, S, x, y, z + 1, nxt);
       }
       __syncthreads();
       if (in_xy) {
@@ -1227,16 +1162,17 @@ step3d_march_kernel(const Params<Real, K> P, const State<Real, Store> S, int p0_
             Real Yo[K], lam0;
 #pragma unroll
             for (int k = 0; k < K; ++k) Yo[k] = cen[(G_Y0 + k) * HP + h];
-            half_store::transport(P, T0, Yo, half_store::mixture_invMw(P, Yo), half_store::mixture_cp(P, Yo), mu0, lam0);
+            half_store::transport(P, T0, Yo, half_store::mixture_invMw(P, Yo),
+                                  half_store::mixture_cp(P, Yo), mu0, lam0);
           }
         }
-        const MarchAcc<Real, K, PRE> A{cen, planes + ((z + 2) % 3) * NF * HP,
+        const MarchAcc<K, PRE> A{cen, planes + ((z + 2) % 3) * NF * HP,
                                        planes + ((z + 1) % 3) * NF * HP, h, mu0, fD,
                                        pre, PRE && have, planes + 3 * NF * HP};
         // a cell that prefetched nothing lies on a non-periodic face: the
         // update pulls with the boundary rules there
         Real fi, fo;
-        accI += half_store::cell_update<3, K, Real, Store>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
+        accI += half_store::cell_update<3, K>(P, S, A, c, xyz, P0, dlnP0, dP0r, fi, fo);
         accIn += fi;
         accOut += fo;
       }
@@ -1260,12 +1196,12 @@ template <> struct BatchShape<0> { using T = Tile<2, 32, 1>; };
 template <> struct BatchShape<1> { using T = Tile<2, 32, 2>; };
 template <> struct BatchShape<2> { using T = Tile<2, 64, 1>; };
 
-template <int K, class Real, class Store, class T_>
+template <int K, class T_>
 __global__ void __launch_bounds__(BLOCK, (T_::RPT > 1 ? 3 : 4))
 batch_step_kernel(const BatchDom<K, Real, Store>* __restrict__ doms,
                   const int* __restrict__ tile_begin, int /* run: 1 */, int ndom, int flip,
                   unsigned* __restrict__ tile_ctr) {
-  using PL = Plane<Real, K, T_::HP, n_mom<2, Store>()>;
+  using PL = Plane<2, K, T_::HP>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PL* planes = reinterpret_cast<PL*>(smem_raw);
   __shared__ double red_sh[96];
@@ -1310,7 +1246,7 @@ batch_step_kernel(const BatchDom<K, Real, Store>* __restrict__ doms,
     const int lt = t - tile_begin[lo];
     const int nbx = (Psh.nx + T_::TX - 1) / T_::TX;
     double sI, sIn, sOut;
-    half_store::step_tile<2, K, Real, Store, T_>(Psh, Ssh, lt % nbx, lt / nbx, 0, 1, planes, red_sh, sI, sIn,
+    half_store::step_tile<2, K, T_>(Psh, Ssh, lt % nbx, lt / nbx, 0, 1, planes, red_sh, sI, sIn,
                                      sOut);
     const unsigned nb = (unsigned)(tile_begin[lo + 1] - tile_begin[lo]);
     publish_partials_at<4>(sI, sIn, sOut, Ssh.partials, Ssh.counter, Ssh.scal, p0c_sh, false, 0.0,

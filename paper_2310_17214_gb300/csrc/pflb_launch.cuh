@@ -578,8 +578,8 @@ struct LauncherImpl final : Launcher {
     if constexpr (DIM == 3) {
       int& grid = mgrid[PRE ? 1 : 0];
       if constexpr (kHalf) {
-        constexpr size_t smem = half_store::march_smem_bytes<K, Real, Store>();
-        auto kern = half_store::step3d_march_kernel<K, Real, Store, PRE>;
+        constexpr size_t smem = half_store::march_smem_bytes<K>();
+        auto kern = half_store::step3d_march_kernel<K, PRE>;
         const cudaError_t e = resident_grid(kern, BLOCK, smem, grid, B.slots);
         if (e != cudaSuccess) return e;
         kern<<<grid, BLOCK, smem, st>>>(P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb);
@@ -625,8 +625,8 @@ struct LauncherImpl final : Launcher {
       };
       cudaError_t e;
       if constexpr (kHalf) {
-        e = launch(half_store::step_kernel<DIM, K, Real, Store>, BLOCK,
-                   half_store::step_smem_bytes<DIM, K, Real, Store>(),
+        e = launch(half_store::step_kernel<DIM, K>, BLOCK,
+                   half_store::step_smem_bytes<DIM, K>(),
                    DIM == 3 ? half_chunk() : 0);
       } else if constexpr (sizeof(Real) == 4) {
         using T_ = Tile<V, 32, 8>;
@@ -665,8 +665,8 @@ struct LauncherImpl final : Launcher {
       cudaError_t e;
       if constexpr (kHalf) {
         using T_ = half_store::Tile<2, 32, TY / 8>;
-        e = launch(half_store::step_persistent_kernel<2, K, Real, Store, T_>, BLOCK,
-                   half_store::step_smem_bytes<2, K, Real, Store, T_>());
+        e = launch(half_store::step_persistent_kernel<2, K, T_>, BLOCK,
+                   half_store::step_smem_bytes<2, K, T_>());
       } else {
         using T_ = Tile<V, 32, TY>;
         e = launch(step_persistent_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>());
@@ -700,8 +700,8 @@ struct LauncherImpl final : Launcher {
   static auto with_batch_kernel(F f) {
     if constexpr (kHalf) {
       using T_ = typename half_store::BatchShape<CFG>::T;
-      return f(half_store::batch_step_kernel<K, Real, Store, T_>, BLOCK,
-               half_store::step_smem_bytes<2, K, Real, Store, T_>());
+      return f(half_store::batch_step_kernel<K, T_>, BLOCK,
+               half_store::step_smem_bytes<2, K, T_>());
     } else {
       using T_ = typename BatchShape<Real, CFG>::T;
       return f(batch_step_kernel<K, Real, T_>, T_::NT, step_smem_bytes<2, K, Real, T_>());
