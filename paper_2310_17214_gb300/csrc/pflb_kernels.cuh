@@ -82,13 +82,13 @@ template <> struct Lattice<3> {
 template <int K>
 struct Chem64 {
   static constexpr int KK = K > 0 ? K : 1;
-  double A[JMAX], b[JMAX], EaR[JMAX], dH[JMAX], dS[JMAX], dn[JMAX];
+  double A[JMAX], b[JMAX], EaR[JMAX], dn[JMAX];
   int rev[JMAX];
-  double order[JMAX][KK], rorder[JMAX][KK], stoich[JMAX][KK];
+  double order[JMAX][KK], rorder[JMAX][KK];
   double Ms[JMAX][KK];          // M_k s_kj
   double dS_R[JMAX], dH_R[JMAX];  // dS / R, dH / R
-  double M[KK], invM[KK], cp[KK], hf[KK];
-  double p_ref, ln_pref_R, rho_ref, dt;  // ln_pref_R = ln(p_ref / R)
+  double invM[KK], cp[KK];
+  double ln_pref_R, rho_ref, dt;  // ln_pref_R = ln(p_ref / R)
   double H[JMAX], cM[JMAX];  // sum_k hf_k Ms_jk, sum_k cp_k Ms_jk
   double pref_R;             // p_ref / R
   int used;                  // bit k: species k enters a rate
@@ -104,7 +104,7 @@ struct Chem32 {
   int on[JMAX], rev[JMAX];
   float order[JMAX][KK], rorder[JMAX][KK];
   float Ms[JMAX][KK];  // M_k s_kj
-  float invM[KK], cp[KK], hf[KK];
+  float invM[KK], cp[KK];
   float ln_pref_R, dt;
   float H[JMAX], cM[JMAX];
   __device__ __forceinline__ bool active(int j) const { return on[j] != 0; }
@@ -199,8 +199,6 @@ struct DevScalars {
 // order in u).  A reader adds w_i (P + 3 c_i . j) of the source cell back.
 template <class Store> struct IsHalf { static constexpr bool value = false; };
 template <> struct IsHalf<__half> { static constexpr bool value = true; };
-template <int DIM, class Store>
-__host__ __device__ constexpr int n_mom() { return IsHalf<Store>::value ? DIM + 1 : 0; }
 
 template <class Real, class Store>
 struct State {
@@ -235,37 +233,23 @@ struct BatchDom {
 
 // ----------------------------------------------------- storage codecs
 template <class Store, class Real> struct Codec;
-// load: from global memory (read-only path); get: from shared memory.
-// raw: the stored value as a number; dec(raw, w/S, fo): the population from it
-// and the first-order part fo of the source cell (FP16 storage: one FMA, the
-// same on every path that decodes, so all paths round alike).
+// raw: the stored value as a number (read-only path).
 template <> struct Codec<double, double> {
   __device__ static double raw(const double* p) { return __ldg(p); }
-  __device__ static double dec(double r, double, double) { return r; }
-  __device__ static double load(const double* p, double) { return __ldg(p); }
-  __device__ static double get(const double* p, double) { return *p; }
   __device__ static void store(double* p, double v, double) { *p = v; }
 };
 template <> struct Codec<float, float> {
   __device__ static float raw(const float* p) { return __ldg(p); }
-  __device__ static float dec(float r, float, float) { return r; }
-  __device__ static float load(const float* p, float) { return __ldg(p); }
-  __device__ static float get(const float* p, float) { return *p; }
   __device__ static void store(float* p, float v, float) { *p = v; }
 };
 // FP16: residual r_i = g_i - w_i (P + 3 c_i . j), stored as h = r / w * scale
-// (weights folded so every direction has the same range); load/get return
-// r_i, the caller adds the first-order part of the source cell.
+// (weights folded so every direction has the same range).  dec(raw, w/S, fo): the
+// population from it and the first-order part fo of the source cell, one FMA,
+// the same on every path that decodes, so that all paths round alike.
 template <> struct Codec<__half, float> {
   __device__ static float raw(const __half* p) { return __half2float(__ldg(p)); }
   __device__ static float dec(float r, float w_over_scale, float fo) {
     return __fmaf_rn(r, w_over_scale, fo);
-  }
-  __device__ static float load(const __half* p, float w_over_scale) {
-    return __half2float(__ldg(p)) * w_over_scale;
-  }
-  __device__ static float get(const __half* p, float w_over_scale) {
-    return __half2float(*p) * w_over_scale;
   }
   __device__ static void store(__half* p, float v, float scale_over_w) {
     *p = __float2half_rn(v * scale_over_w);

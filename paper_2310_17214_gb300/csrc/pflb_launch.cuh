@@ -214,14 +214,11 @@ Params<Real, K> make_params(const pflb_domain_desc& d, const pflb_mechanism& m, 
     c.A[j] = m.A[j];
     c.b[j] = m.b[j];
     c.EaR[j] = m.EaR[j];
-    c.dH[j] = m.dH[j];
-    c.dS[j] = m.dS[j];
     c.dn[j] = dn;
     c.rev[j] = m.rev[j];
     for (int k = 0; k < K; ++k) {
       c.order[j][k] = m.order[j][k];
       c.rorder[j][k] = m.rorder[j][k];
-      c.stoich[j][k] = m.stoich[j][k];
       c.Ms[j][k] = m.M[k] * m.stoich[j][k];
     }
     c.dS_R[j] = m.dS[j] / R_GAS;
@@ -229,19 +226,16 @@ Params<Real, K> make_params(const pflb_domain_desc& d, const pflb_mechanism& m, 
   }
   P.p_ref_R = Real(K > 0 && m.p_ref > 0 ? m.p_ref / R_GAS : 101325.0 / R_GAS);
   for (int k = 0; k < K; ++k) {
-    P.c64.M[k] = m.M[k];
     P.c64.invM[k] = 1.0 / m.M[k];
     P.c64.cp[k] = m.cp[k];
-    P.c64.hf[k] = m.hf[k];
   }
   for (int j = 0; j < P.J; ++j)
     for (int k = 0; k < K; ++k) {
       P.c64.H[j] += m.hf[k] * P.c64.Ms[j][k];
       P.c64.cM[j] += m.cp[k] * P.c64.Ms[j][k];
     }
-  P.c64.p_ref = m.p_ref > 0 ? m.p_ref : 101325.0;
-  P.c64.ln_pref_R = std::log(P.c64.p_ref / R_GAS);
-  P.c64.pref_R = P.c64.p_ref / R_GAS;
+  P.c64.pref_R = (m.p_ref > 0 ? m.p_ref : 101325.0) / R_GAS;
+  P.c64.ln_pref_R = std::log(P.c64.pref_R);
   for (int j = 0; j < P.J; ++j)
     for (int k = 0; k < K; ++k)
       if (m.order[j][k] != 0.0 || (m.rev[j] && m.rorder[j][k] != 0.0)) P.c64.used |= 1 << k;
@@ -270,7 +264,6 @@ Params<Real, K> make_params(const pflb_domain_desc& d, const pflb_mechanism& m, 
     for (int k = 0; k < K; ++k) {
       f.invM[k] = float(c.invM[k]);
       f.cp[k] = float(c.cp[k]);
-      f.hf[k] = float(c.hf[k]);
     }
     f.ln_pref_R = float(c.ln_pref_R);
     f.dt = float(c.dt);
@@ -775,15 +768,15 @@ struct LauncherImpl final : Launcher {
     if constexpr (!kTmaType) {
       return false;
     } else {
-      using LY = TmaLayout<K, Store>;
+      using LY = TmaLayout<K>;
       if (tma_state < 0) return false;
       if (tma_state == 0) {
         // rows must be whole 16-byte units for every array the boxes read
-        if (P.nx % (16 / (int)sizeof(Store)) != 0 || P.nx % 4 != 0 || !encode_tiled()) {
+        if (P.nx % 4 != 0 || !encode_tiled()) {
           tma_state = -1;
           return false;
         }
-        auto kern = step_tma_kernel<K, Store>;
+        auto kern = step_tma_kernel<K>;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)LY::smem_bytes) != cudaSuccess) {
           tma_state = -1;
@@ -813,8 +806,6 @@ struct LauncherImpl final : Launcher {
         const unsigned long long dY[3] = {nx, ny, (unsigned long long)(K > 0 ? K : 1)};
         const unsigned long long dg[3] = {nx, ny, 9ull};
         const unsigned pb[3] = {(unsigned)LY::PW, (unsigned)LY::PH, 1u};
-        const CUtensorMapDataType gdt = sizeof(Store) == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16
-                                                           : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
         TmaMaps& m = maps[cur];
         const void* Ts = B.Ts[cur] ? B.Ts[cur] : B.T[cur];
         const void* Y = K > 0 ? B.Y[cur] : B.T[cur];
@@ -823,7 +814,7 @@ struct LauncherImpl final : Launcher {
                   encode_map(&m.Ts, Ts, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 2, d2, fb) &&
                   (K > 0 ? encode_map(&m.Y, Y, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 3, dY, fb)
                          : encode_map(&m.Y, Y, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 2, d2, fb)) &&
-                  encode_map(&m.g, B.g[cur], gdt, (int)sizeof(Store), 3, dg, pb);
+                  encode_map(&m.g, B.g[cur], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 3, dg, pb);
         if (!ok) {
           tma_state = -1;
           return false;
@@ -836,11 +827,11 @@ struct LauncherImpl final : Launcher {
 
   cudaError_t step_tma(Buffers& B, int cur, cudaStream_t st, const double* prev) {
     if constexpr (kTmaType) {
-      using LY = TmaLayout<K, Store>;
+      using LY = TmaLayout<K>;
       const int tiles_x = (P.nx + LY::TX - 1) / LY::TX;
       const int n_tiles = tiles_x * ((P.ny + LY::TY - 1) / LY::TY);
       const TmaMaps& m = maps[cur];
-      step_tma_kernel<K, Store><<<tma_grid, LY::NT, LY::smem_bytes, st>>>(
+      step_tma_kernel<K><<<tma_grid, LY::NT, LY::smem_bytes, st>>>(
           P, state(B, cur), p0_closed, prev, (unsigned)B.last_nb, m.T, m.phi, m.Ts, m.Y, m.g,
           tiles_x, n_tiles, wait_limit);
       B.last_nb = tma_grid;

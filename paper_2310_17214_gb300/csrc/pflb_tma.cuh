@@ -1,13 +1,12 @@
-// pflb_tma.cuh -- persistent, TMA-pipelined fused step for 2-D lattices with
-// FP32 compute (FP32 or FP16-stored populations).
+// pflb_tma.cuh -- persistent, TMA-pipelined fused step for 2-D lattices in FP32.
 //
 // Each block walks a strided list of 32 x 8 tiles.  One elected thread issues
 // the tensor-memory-accelerator loads of the NEXT tile into the other half of
 // a double-buffered stage while the block works on the current one:
 //   - T, phi_s, Ts: 2-D boxes of (32 + 2 XL) x 10 cells (tile + halo; the x
-//     start is rounded down to a 16-byte boundary, XL = 16 / sizeof(Real));
+//     start is rounded down to a 16-byte boundary, XL = 4);
 //   - Y_k: one 3-D box (32 + 2 XL) x 10 x K;
-//   - populations: for each direction i the 32 + 2 XLp by 8 window of g_i
+//   - populations: for each direction i the 32 + 2 XL by 8 window of g_i
 //     shifted by -c_iy rows (the -c_ix column shift is an offset into the
 //     box), so the pull of every interior cell reads shared memory.
 // Loads complete on an mbarrier per stage (expect_tx = box bytes, a box that
@@ -106,26 +105,25 @@ struct TmaMapRefs {
 };
 
 // ------------------------------------------------------------ stage layout
-template <int K, class Store>
+template <int K>
 struct TmaLayout {
   static constexpr int TX = 32, TY = 8;
   static constexpr int XL = 4;                        // 16 B of floats
   static constexpr int FW = TX + 2 * XL, FH = TY + 2;  // field box
-  static constexpr int XLP = 16 / (int)sizeof(Store);
-  static constexpr int PW = TX + 2 * XLP, PH = TY;    // population box
+  static constexpr int PW = TX + 2 * XL, PH = TY;     // population box
   static constexpr int Q = 9;
   static constexpr int NRAW = 3 + K;                  // T, phi, Ts, Y_k
   static constexpr int FBOX = FW * FH;                // floats per field box
   static constexpr int FBP = (FBOX * 4 + 127) / 128 * 32;  // 128-byte aligned box slot
   static constexpr int OFF_T = 0, OFF_PHI = FBP, OFF_TS = 2 * FBP, OFF_Y = 3 * FBP;
-  static constexpr int PBOX = PW * PH;                // Stores per population box
+  static constexpr int PBOX = PW * PH;                // floats per population box
   // derived plane: rows start two cells left of the tile, so that a thread's
   // pair of cells is an aligned word of its row
   static constexpr int HX = TX + 4, HP = HX * (TY + 2);
   static constexpr int NT = TX * TY / 2;              // threads, two cells each
   static constexpr int NDER = 5;                      // rho, kT, mu, fD, RF
   static constexpr size_t raw_bytes = ((size_t)(3 * FBP + K * FBOX) * 4 + 127) / 128 * 128;
-  static constexpr size_t pop_bytes = (size_t)Q * PBOX * sizeof(Store);
+  static constexpr size_t pop_bytes = (size_t)Q * PBOX * 4;
   static constexpr size_t stage_bytes = (raw_bytes + pop_bytes + 127) / 128 * 128;
   static constexpr size_t der_bytes = (size_t)NDER * HP * 4;
   // [stage 0][stage 1][derived plane][2 mbarriers][block-sum scratch][flag];
@@ -138,11 +136,11 @@ struct TmaLayout {
 
 // Accessor over a TMA stage (raw fields, populations) plus the derived plane,
 // for the pair of cells (lx, lx + 1) of row ly.
-template <int K, class Store>
+template <int K>
 struct TmaAcc {
-  using LY = TmaLayout<K, Store>;
+  using LY = TmaLayout<K>;
   const float* __restrict__ raw;
-  const Store* __restrict__ pops;
+  const float* __restrict__ pops;
   const float* __restrict__ der;
   int lx, ly;
   __device__ __forceinline__ const float* at(int f, int dx, int dy) const {
@@ -171,18 +169,18 @@ struct TmaAcc {
     return s < 0 ? make_float2(v, own.x) : make_float2(own.y, v);
   }
   __device__ __forceinline__ float2 pop(int i) const {
-    const Store* p = pops + i * LY::PBOX + ly * LY::PW + lx - Lattice<2>::c(i, 0) + LY::XLP;
+    const float* p = pops + i * LY::PBOX + ly * LY::PW + lx - Lattice<2>::c(i, 0) + LY::XL;
     return make_float2(p[0], p[1]);
   }
 };
 
 // Ghost / periodic values for the out-of-domain cells of an edge tile's
 // staged halo (same rules as the staged-plane path).
-template <int K, class Store>
+template <int K>
 __device__ __forceinline__ void fix_halo(const Params<float, K>& P,
-                                         const State<float, Store>& S, float* raw, int x0,
+                                         const State<float, float>& S, float* raw, int x0,
                                          int y0) {
-  using LY = TmaLayout<K, Store>;
+  using LY = TmaLayout<K>;
   constexpr int BX = LY::TX + 2;
   for (int h = threadIdx.x; h < BX * LY::FH; h += LY::NT) {
     const int hx = h % BX, hy = h / BX;
@@ -233,10 +231,10 @@ __device__ __forceinline__ void fix_halo(const Params<float, K>& P,
 // Properties of every staged pair of cells (tile + halo) from the staged raw
 // fields.  (The outer cell of the first and last pair of a row is staged but
 // never read.)
-template <int K, class Store>
+template <int K>
 __device__ __forceinline__ void derive_plane(const Params<float, K>& P, float* raw,
                                              float* der, float P0) {
-  using LY = TmaLayout<K, Store>;
+  using LY = TmaLayout<K>;
   constexpr int PW = LY::HX / 2;
   for (int h = threadIdx.x; h < PW * LY::FH; h += LY::NT) {
     const int hy = h / PW, hx = (h - hy * PW) * 2;
@@ -267,15 +265,15 @@ __device__ __forceinline__ void derive_plane(const Params<float, K>& P, float* r
   }
 }
 
-template <int K, class Store>
+template <int K>
 __device__ __forceinline__ void issue_tile(const TmaMapRefs& M, const Params<float, K>& P,
                                            unsigned char* stage, uint64_t* bar, int x0, int y0) {
-  using LY = TmaLayout<K, Store>;
+  using LY = TmaLayout<K>;
   constexpr unsigned field_bytes = LY::FBOX * 4;
   const unsigned bytes = (unsigned)((P.Ts_field ? 3 : 2) * field_bytes + K * field_bytes +
                                     LY::pop_bytes);
   float* raw = reinterpret_cast<float*>(stage);
-  Store* pops = reinterpret_cast<Store*>(stage + LY::raw_bytes);
+  float* pops = reinterpret_cast<float*>(stage + LY::raw_bytes);
   mbar_expect_tx(bar, bytes);
   tma_load_2d(raw + LY::OFF_T, M.T, x0 - LY::XL, y0 - 1, bar);
   tma_load_2d(raw + LY::OFF_PHI, M.phi, x0 - LY::XL, y0 - 1, bar);
@@ -283,19 +281,19 @@ __device__ __forceinline__ void issue_tile(const TmaMapRefs& M, const Params<flo
   if constexpr (K > 0) tma_load_3d(raw + LY::OFF_Y, M.Y, x0 - LY::XL, y0 - 1, 0, bar);
 #pragma unroll
   for (int i = 0; i < LY::Q; ++i)
-    tma_load_3d(pops + i * LY::PBOX, M.g, x0 - LY::XLP, y0 - Lattice<2>::c(i, 1), i, bar);
+    tma_load_3d(pops + i * LY::PBOX, M.g, x0 - LY::XL, y0 - Lattice<2>::c(i, 1), i, bar);
 }
 
-template <int K, class Store>
-__global__ void __launch_bounds__((TmaLayout<K, Store>::NT), 2)
-step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_closed,
+template <int K>
+__global__ void __launch_bounds__((TmaLayout<K>::NT), 2)
+step_tma_kernel(const Params<float, K> P, const State<float, float> S, int p0_closed,
                 const double* __restrict__ prev_partials, unsigned prev_nb,
                 const __grid_constant__ CUtensorMap mT, const __grid_constant__ CUtensorMap mPhi,
                 const __grid_constant__ CUtensorMap mTs, const __grid_constant__ CUtensorMap mY,
                 const __grid_constant__ CUtensorMap mG, int tiles_x, int n_tiles,
                 long long wait_limit) {
   const TmaMapRefs M{&mT, &mPhi, &mTs, &mY, &mG};
-  using LY = TmaLayout<K, Store>;
+  using LY = TmaLayout<K>;
   // All shared memory of this kernel is the dynamic buffer, its base rounded up
   // to 128 bytes: TMA destinations are 128-byte aligned, mbarriers 8-byte.
   extern __shared__ unsigned char smem_dyn[];
@@ -340,7 +338,7 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
   bool any_flux = false;
   int first = blockIdx.x;
   if (threadIdx.x == 0 && first < n_tiles)
-    issue_tile<K, Store>(M, P, stage[0], &bar[0], (first % tiles_x) * LY::TX,
+    issue_tile<K>(M, P, stage[0], &bar[0], (first % tiles_x) * LY::TX,
                          (first / tiles_x) * LY::TY);
   int it = 0;
   for (int t = first; t < n_tiles; t += gridDim.x, ++it) {
@@ -350,7 +348,7 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
     if (threadIdx.x == 0) {
       if (tn < n_tiles) {
         fence_proxy_async();
-        issue_tile<K, Store>(M, P, stage[s ^ 1], &bar[s ^ 1], (tn % tiles_x) * LY::TX,
+        issue_tile<K>(M, P, stage[s ^ 1], &bar[s ^ 1], (tn % tiles_x) * LY::TX,
                              (tn / tiles_x) * LY::TY);
       }
       s_ok = mbar_wait_bounded(&bar[s], (it >> 1) & 1, wait_limit) ? 1 : 0;
@@ -368,14 +366,14 @@ step_tma_kernel(const Params<float, K> P, const State<float, Store> S, int p0_cl
     float* raw = reinterpret_cast<float*>(stage[s]);
     const bool edge_tile = x0 == 0 || y0 == 0 || x0 + LY::TX >= P.nx || y0 + LY::TY >= P.ny;
     if (edge_tile) {
-      fix_halo<K, Store>(P, S, raw, x0, y0);
+      fix_halo<K>(P, S, raw, x0, y0);
       __syncthreads();
     }
-    derive_plane<K, Store>(P, raw, der, P0);
+    derive_plane<K>(P, raw, der, P0);
     __syncthreads();
     const int x = x0 + lx, y = y0 + ly;
     if (x < P.nx && y < P.ny) {
-      const TmaAcc<K, Store> A{raw, reinterpret_cast<const Store*>(stage[s] + LY::raw_bytes), der,
+      const TmaAcc<K> A{raw, reinterpret_cast<const float*>(stage[s] + LY::raw_bytes), der,
                                lx, ly};
       const CellPos q{x + P.nx * y, x, y, 0, S.even != 0, true};  // nx is even here
       // the stage's population windows are valid off every face

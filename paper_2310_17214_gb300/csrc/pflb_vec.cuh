@@ -108,8 +108,6 @@ __device__ __forceinline__ bool2x vgt(float2 a, float2 b) { return {a.x > b.x, a
 __device__ __forceinline__ bool vge(float a, float b) { return a >= b; }
 __device__ __forceinline__ bool vge(double a, double b) { return a >= b; }
 __device__ __forceinline__ bool2x vge(float2 a, float2 b) { return {a.x >= b.x, a.y >= b.y}; }
-__device__ __forceinline__ bool vand(bool a, bool b) { return a && b; }
-__device__ __forceinline__ bool2x vand(bool2x a, bool2x b) { return {a.x && b.x, a.y && b.y}; }
 __device__ __forceinline__ bool vany(bool a) { return a; }
 __device__ __forceinline__ bool vany(bool2x a) { return a.x || a.y; }
 __device__ __forceinline__ float vsel(bool m, float a, float b) { return m ? a : b; }
