@@ -323,30 +323,35 @@ int pflb_get_state(pflb_domain* d, void* dst, size_t bytes, int where);
  * Asynchronous on the domain's stream. */
 int pflb_set_state(pflb_domain* d, const void* src, size_t bytes, int where);
 
-/* Step kernels.  PFLB_KERNEL_TILED (default): 32 x 8 tiles staged in shared
- * memory with per-cell properties evaluated once (2.5-D z-marching in 3-D).
+/* Step kernels.  PFLB_KERNEL_TILED: a block per tile, staged in shared memory
+ * with per-cell properties evaluated once.  2-D: 32 x 8 cells; in FP64 32 x 8,
+ * 32 x 4 or 32 x 2, whichever spreads best over the SMs.  3-D: a block marches
+ * along z over a run of planes of a 32 x 8 column, long runs first and shorter
+ * ones towards the end of the launch (FP16 storage: equal runs in small domains,
+ * runs of sixteen planes in closed ones).
  * PFLB_KERNEL_TMA: persistent blocks, the next tile's fields and population
  * windows fetched by the tensor memory accelerator into a double-buffered
- * stage (2-D, FP32 compute, nx a multiple of 4 -- 8 with FP16 storage). */
+ * stage (2-D, FP32 storage, nx a multiple of 4). */
 #define PFLB_KERNEL_TILED 0
 #define PFLB_KERNEL_TMA 1
 /* PFLB_KERNEL_PERSISTENT(_32x16): 2-D only; one grid of resident blocks walks
- * the 32 x 8 (or 32 x 16, two rows per thread) tiles, handed out by an
- * atomic counter, so no second wave and no idle SMs at the end. */
+ * the 32 x 8 (or 32 x 16; two rows per thread in FP64 and with FP16 storage)
+ * tiles, handed out by an atomic counter, so no second wave and no idle SMs at
+ * the end. */
 #define PFLB_KERNEL_PERSISTENT 2
 #define PFLB_KERNEL_PERSISTENT_32x16 3
 /* PFLB_KERNEL_MARCH(_PREFETCH): 3-D only; a resident grid in which each block
  * marches a contiguous, equal share of the tile-planes along z (ring of three
- * staged planes holding only what neighbours read); _PREFETCH also issues the
- * next plane's pulls into registers before the current plane is updated,
- * periodic faces wrapped in the addresses. */
+ * staged planes); _PREFETCH issues a plane's populations before the next plane is
+ * staged (FP16 storage: the next plane's before the current one is updated). */
 #define PFLB_KERNEL_MARCH 4
 #define PFLB_KERNEL_MARCH_PREFETCH 5
 #define PFLB_KERNELS 6
 
 /* Select the step kernel of a domain (after pflb_set_fields).  The default is
- * PFLB_KERNEL_MARCH for 3-D domains with FP32 storage, PFLB_KERNEL_TILED
- * otherwise.  Returns PFLB_ERR_UNSUPPORTED if the kernel cannot run this
+ * PFLB_KERNEL_TILED, and PFLB_KERNEL_MARCH for 3-D domains in FP64 or FP32 (not
+ * FP16 storage) with fewer than 16 planes of 32 x 8 columns per resident block
+ * (one block per SM in FP64, three in FP32).  Returns PFLB_ERR_UNSUPPORTED if the kernel cannot run this
  * domain. */
 int pflb_select_kernel(pflb_domain* d, int kernel);
 

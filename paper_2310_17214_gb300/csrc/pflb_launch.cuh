@@ -384,8 +384,9 @@ struct LauncherImpl final : Launcher {
   }
   long long resident3d() { return (sizeof(Real) == 8 ? 1LL : 3LL) * sm_count(); }
   // First run of the shrinking runs: 32 planes, sixteen where that is more than a
-  // resident block's share (FP32, 250 x 100 x 100, 23 planes: 177 us a step, 210
-  // from 32; 256 x 128 x 128, 36 planes: 260, 253 from 32).
+  // resident block's share (FP32 beds, us a step: 250 x 100 x 100, 23 planes, 177
+  // from sixteen, 210 from 32; 256 x 128 x 128, 36 planes, 295 in equal runs, 260
+  // from sixteen, 253 from 32; runs move these by up to 2 %).
   int first_chunk() { return planes() >= 32 * resident3d() ? 32 : 16; }
   // Runs of planes of the FP16-stored 3-D step (256 threads, two blocks per SM),
   // by the planes a resident block has to do.  Below eight, the shortest equal

@@ -7,9 +7,7 @@
 //     boundary cells, which cost more, do not leave SMs idle at the end; a run
 //     stages two halo planes, about the work of two planes.  Short domains
 //     (chunk = 0) take equal runs: block b of a resident grid owns
-//     [b T / G, (b + 1) T / G).  On the 256 x 128 x 128 bed (36 planes a block
-//     in equal runs) FP32 takes 295 us in equal runs, 282 in runs of 8, 256 /
-//     250 with runs that start at 16 / 32;
+//     [b T / G, (b + 1) T / G).  Lengths and times: LauncherImpl::first_chunk;
 //   - a ring of three staged planes in shared memory;
 //   - PRE: the 19 populations of the plane are issued before the next plane is
 //     staged, so the two load phases overlap; otherwise after the staging
@@ -23,8 +21,8 @@ namespace pflb {
 
 // The 3-D tile of the march and the resident blocks per SM it is compiled for:
 // 32 x 8 cells, in FP32 a pair per thread (128 threads, 168 registers: the
-// 256 x 128 x 128 bed takes 295 us in equal runs; 32 x 16 cells in 256 threads
-// at 128 registers spill, 405 us), in FP64 one.
+// 256 x 128 x 128 bed takes 295 us a step in equal runs; 32 x 16 cells in 256
+// threads at 128 registers spill, 405 us), in FP64 one.
 template <class Real> struct MarchTile {
   using T = Tile<typename VecOf<Real>::V, 32, 8>;
   static constexpr int MINB = sizeof(Real) == 8 ? 1 : 3;
